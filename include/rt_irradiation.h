@@ -57,8 +57,9 @@ extern "C" {
                             power series in the column, truncated below 1e-7 of
                             the value, instead of bin by bin. */
 #define RT_FP32_PLAIN 1  /* FP32 bins; plain FP32 running sum (precision study) */
-#define RT_FP64       2  /* FP64 scan and FP64 per-bin arithmetic (libm-grade exp
-                            and expm1); outputs still rounded to float32 */
+#define RT_FP64       2  /* FP64 scan and FP64 arithmetic over the bins, every form to
+                            FP64 rounding (bins thin up to a warp's last cell as one
+                            power series); outputs still rounded to float32 */
 
 #define RT_MAX_NU 128    /* largest number of frequency bins per table */
 

@@ -246,6 +246,7 @@ int finalize(rt_ctx *c)
     cudaError_t e = rt::launch_setup_bins(c->n_nu, c->nu_mid, c->kappa, c->t_star, c->r_star,
                                           c->kappa_bf16, c->f_bin, c->nu_tab, c->kap, c->nu64,
                                           c->sc, c->stream, c->order_d);
+    if (e == cudaSuccess && c->precision == RT_FP64) e = rt::launch_thin_table64(c->nu64, c->sc, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, "setup_bins", e);
     e = rt::launch_setup_geometry(c->nr, c->ntheta, c->nphi, c->r_if, c->theta_if, c->phi_if,
                                   c->t_star, c->rtab, c->rtab64, c->domega, c->domega32, c->sc,
@@ -563,7 +564,7 @@ int rt_create(const rt_grid_desc *g, void *cuda_stream, rt_ctx **out)
     ok = ok && dalloc(&c->f_bin, RT_MAX_NU) == cudaSuccess;
     ok = ok && dalloc(&c->nu_tab, RT_MAX_NU + rt::kNuPad) == cudaSuccess;
     ok = ok && dalloc(&c->kap, rt::kKapBuffer) == cudaSuccess;
-    ok = ok && dalloc(&c->nu64, RT_MAX_NU + rt::kNuPad) == cudaSuccess;
+    ok = ok && dalloc(&c->nu64, rt::kNu64Buffer) == cudaSuccess;
     ok = ok && dalloc(&c->sc, 1) == cudaSuccess;
     ok = ok && dalloc(&c->order_d, RT_MAX_NU) == cudaSuccess;
     ok = ok && dalloc(&c->bad, 1) == cudaSuccess;

@@ -47,6 +47,15 @@ constexpr int kKapBuffer = kKapTable + (RT_MAX_NU + 1) * kThinStride;  // with t
 constexpr float kThinX = 1.0f;
 static_assert(kThinStride >= kThinTerms + 2, "a series row holds s, C_1..C_K and S_0");
 
+// The same series for the FP64 mode, in FP64: rows (s_b, C_1 .. C_kThinTerms64, S_0) after the
+// FP64 bin table. With kappa_i N <= 1 the first omitted term is below 1/19! = 8e-18 of the
+// leading one, under FP64 rounding (18 terms; 16 would leave 2.8e-15).
+constexpr int kThinTerms64 = 18;
+constexpr int kThinStride64 = 20;                                                  // doubles per row
+constexpr int kNu64Table = RT_MAX_NU + kNuPad;                                     // double2 entries of the bin table
+constexpr int kNu64Buffer = kNu64Table + (RT_MAX_NU + 1) * (kThinStride64 / 2);    // double2, with the series rows
+static_assert(kThinStride64 >= kThinTerms64 + 2 && kThinStride64 % 2 == 0, "a series row holds s, C_1..C_K and S_0");
+
 // Scalars of one configured grid, resident in device memory.
 struct DevScalars {
     double f_max;          // largest bin flux F_i (erg s^-1 cm^-2)
@@ -107,7 +116,7 @@ struct TraceArgs {
     float *a;
     const NuEntry *nu;        // [nnu_pad]
     const float *kap;         // [nnu_pad] kappa_i (rho -> 0 force limit)
-    const double2 *nu64;      // [nnu_pad] (kappa_i, F_i/F_max), FP64 mode
+    const double2 *nu64;      // [kNu64Buffer] (kappa_i, F_i/F_max), then the series rows (FP64 mode)
     const float4 *rtab;       // [nr] (dr, Gq, Ga0, 0)
     const RadRow64 *rtab64;    // [nr] same in FP64
     const double *domega;     // [nrays]
@@ -263,6 +272,8 @@ cudaError_t launch_setup_bins(int n_nu, const double *nu_mid_dev, const double *
                               double *f_bin_dev, NuEntry *nu_dev, float *kap_dev,
                               double2 *nu64_dev, DevScalars *sc_dev, cudaStream_t stream,
                               int *order_dev = nullptr);
+// the FP64 mode's series rows, from the bin table launch_setup_bins left in nu64_dev
+cudaError_t launch_thin_table64(double2 *nu64_dev, const DevScalars *sc_dev, cudaStream_t stream);
 cudaError_t launch_setup_geometry(int nr, int ntheta, int nphi, const double *r_if_dev,
                                   const double *theta_if_dev, const double *phi_if_dev,
                                   double t_star, float4 *rtab, RadRow64 *rtab64,

@@ -121,6 +121,48 @@ __global__ void k_thin_table(const NuEntry *nu, const DevScalars *sc, float *thi
     }
 }
 
+// The FP64 mode's rows (kThinTerms64), one warp per row: as k_thin_table, from the FP64
+// bin table.
+__global__ void k_thin_table64(double2 *nu64, const DevScalars *sc)
+{
+    const int b = blockIdx.x, lane = threadIdx.x;
+    const int na = sc->n_active;
+    double *row = reinterpret_cast<double *>(nu64 + kNu64Table) + (size_t)b * kThinStride64;
+    if (b == 0 || b > na) {
+        if (lane < kThinStride64) row[lane] = 0.0;
+        return;
+    }
+    const double s = nu64[b - 1].x;
+    double m[kThinTerms64 + 1];
+#pragma unroll
+    for (int k = 0; k <= kThinTerms64; ++k) m[k] = 0.0;
+    for (int i = lane; i < b; i += 32) {
+        const double2 e = nu64[i];
+        const double r = e.x / s;
+        double p = e.y;
+        m[0] += p;
+#pragma unroll
+        for (int k = 1; k <= kThinTerms64; ++k) {
+            p *= r;
+            m[k] += p;
+        }
+    }
+#pragma unroll
+    for (int k = 0; k <= kThinTerms64; ++k)
+        for (int o = 16; o > 0; o >>= 1) m[k] += __shfl_xor_sync(0xffffffffu, m[k], o);
+    if (lane == 0) {
+        row[0] = s;
+        double fact = 1.0;
+#pragma unroll
+        for (int k = 1; k <= kThinTerms64; ++k) {
+            fact *= k;
+            row[k] = ((k & 1) ? m[k] : -m[k]) / fact;
+        }
+        row[kThinTerms64 + 1] = m[0];
+        for (int k = kThinTerms64 + 2; k < kThinStride64; ++k) row[k] = 0.0;
+    }
+}
+
 // Per-radius and per-ray tables. Gq = 3 R*^2 F_max / (r+^3 - r-^3) turns the
 // per-ray sum of F_i/F_max e^-tau (1-e^-dtau) into power per volume; Ga0 = Gq dr / c
 // is the rho -> 0 force factor.
@@ -217,6 +259,12 @@ cudaError_t launch_setup_bins(int n_nu, const double *nu_mid_dev, const double *
     if (e != cudaSuccess) return e;
     static_assert(kThinStride >= kThinTerms + 2, "a row holds s, C_1..C_K and S_0");
     k_thin_table<<<RT_MAX_NU + 1, 32, 0, stream>>>(nu_dev, sc_dev, kap_dev + kKapTable);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_thin_table64(double2 *nu64_dev, const DevScalars *sc_dev, cudaStream_t stream)
+{
+    k_thin_table64<<<RT_MAX_NU + 1, 32, 0, stream>>>(nu64_dev, sc_dev);
     return cudaGetLastError();
 }
 

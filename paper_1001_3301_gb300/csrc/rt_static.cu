@@ -39,7 +39,7 @@ struct StaticScratch {
     double f_bin[RT_MAX_NU];
     rt::NuEntry nu_tab[RT_MAX_NU + rt::kNuPad];
     float kap[rt::kKapBuffer];  // kappa table, then the thin-ray series rows
-    double2 nu64[RT_MAX_NU + rt::kNuPad];
+    double2 nu64[rt::kNu64Buffer];  // FP64 bin table, then the FP64 mode's series rows
     float4 rtab[kStaticMaxNr];
     rt::RadRow64 rtab64[kStaticMaxNr];
     double domega[kStaticMaxRays];
@@ -181,6 +181,7 @@ extern "C" int rt_irradiate_static(const rt_grid_desc *g, double t_star, double 
     // bin fluxes (Eq. 20) and geometry tables, as rt_set_star / rt_set_opacity_table do
     RT_SCK(rt::launch_setup_bins(n_nu, s->nu_mid, s->kappa, t_star, r_star, kappa_bf16 ? 1 : 0, s->f_bin,
                                  s->nu_tab, s->kap, s->nu64, &s->sc, stream));
+    if (g->precision == RT_FP64) RT_SCK(rt::launch_thin_table64(s->nu64, &s->sc, stream));
     RT_SCK(rt::launch_setup_geometry(g->nr, g->ntheta, g->nphi, s->r_if, s->theta_if, s->phi_if, t_star, s->rtab,
                                      s->rtab64, s->domega, s->domega32, &s->sc, stream));
     rt::DevScalars sc;

@@ -33,6 +33,189 @@ struct TileTypes {
     using ESum = typename std::conditional<MODE == RT_FP64, PlainSum<double>, KahanSum>::type;
 };
 
+// ---- FP64 mode: the bins of a lane's cells -----------------------------------------
+// The FP64 pipe (2 FMA per SM and clock on this part) is what bounds the mode, so the work is
+// counted in FP64 instructions; the shortcuts are the FP32 tracer's, carried to FP64 rounding.
+// Every form yields h = sum_i kappa_i g_i phi(kappa_i dN), phi(x) = (1 - e^{-x}) / x, the power
+// absorbed per unit column: the cell absorbs dN h, the force is Ga0 h, and phi(0) = 1 makes
+// dN = 0 its limit with no separate sum.
+//   - bins thin up to the end of the warp's cells (kappa_i N <= 1 there): one power series in
+//     the column, 2 K + 1 = 37 FMA per cell for all of them (set-up rows, k_thin_table64);
+//   - the others bin by bin, the attenuation carried from cell to cell along the lane
+//     (F_out = F_in (1 - kappa dN phi), Eqs. 31-32), one exp per (lane, bin) at its first
+//     cell; phi by a Taylor polynomial of 5, 8 or 13 terms where the warp's largest kappa dN
+//     keeps the first omitted term below 2^-54, else with Cody and Waite's reduction;
+//   - bins whose attenuation underflows at the warp's smallest column are skipped.
+// exp() and expm1() of every bin of every cell took 46 FP64 instructions per (cell, bin).
+// 128x64x64, 79 bins, tau550 = 1: 3.60 -> 0.55 ms per launch (137 FP64 instructions per cell),
+// 0.26 ms with one CTA per tile (rt_trace.cu).
+constexpr float kX64T5 = 2.09e-3f, kX64T8 = 4.6e-2f, kX64T13 = 0.3465f;  // largest kappa dN of 5, 8, 13 terms
+
+__device__ constexpr double phi_coeff(int k)  // (-1)^k / (k + 1)!
+{
+    double c = 1.0;
+    for (int i = 2; i <= k + 1; ++i) c *= i;
+    return ((k & 1) ? -1.0 : 1.0) / c;
+}
+
+template <int NT>
+__device__ __forceinline__ double phi_taylor(double x)
+{
+    double p = phi_coeff(NT - 1);
+#pragma unroll
+    for (int k = NT - 2; k >= 0; --k) p = fma(p, x, phi_coeff(k));
+    return p;
+}
+
+// e^{-x} and 1 - e^{-x} for x >= 0, each to FP64 rounding: x = n ln 2 + r with |r| <= ln 2 / 2
+// (Cody and Waite 1980; ln 2 split at 41 bits so that n ln2_hi is exact), 1 - e^{-r} = r phi(r).
+// x is cut at 708 (e^{-708} = 3e-308).
+__device__ __forceinline__ void exp_pair(double x, double &e, double &om)
+{
+    constexpr double kMagic = 6755399441055744.0;  // 1.5 2^52: adding it rounds to an integer
+    constexpr double kHi = 0x1.62e42fefa3000p-1, kLo = 0x1.3de6af278ece6p-42;
+    x = x < 708.0 ? x : 708.0;
+    const double t = fma(x, kLog2e, kMagic);
+    const int n = __double2loint(t);
+    const double nd = t - kMagic;
+    double r = fma(-nd, kHi, x);
+    r = fma(-nd, kLo, r);
+    const double u = r * phi_taylor<13>(r);
+    const double er = 1.0 - u;  // in [0.7, 1.42]: the scale by 2^-n stays normal
+    e = __hiloint2double(__double2hiint(er) - (n << 20), __double2loint(er));
+    om = n == 0 ? u : 1.0 - e;
+}
+
+// bins [i0, i1) with an NT-term phi (NT = 0: any kappa dN)
+template <int NT, int C>
+__device__ __forceinline__ void bins64(int i0, int i1, const double2 *s_nu64, unsigned head_m,
+                                       const Cells<double, C> &N, const Cells<double, C> &D, double (&h)[C])
+{
+    if (i0 >= i1) return;  // warp-uniform
+    double rd[NT == 0 ? C : 1];
+    if constexpr (NT == 0) {
+#pragma unroll
+        for (int j = 0; j < C; ++j) rd[j] = D.get(j) > 0.0 ? 1.0 / D.get(j) : 0.0;
+    }
+#pragma unroll 1
+    for (int i = i0; i < i1; ++i) {
+        const double2 e = s_nu64[i];  // (kappa_i, F_i / F_max)
+        double g = e.y * exp(-e.x * N.get(0));
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            if (j > 0 && ((head_m >> j) & 1u)) g = e.y;  // a new ray starts here
+            const double x = e.x * D.get(j);
+            if constexpr (NT > 0) {
+                const double gp = g * phi_taylor<NT>(x);
+                h[j] = fma(e.x, gp, h[j]);
+                g = fma(-x, gp, g);
+            } else {
+                double ex, om;
+                exp_pair(x, ex, om);
+                // dN = 0: phi = 1
+                h[j] = D.get(j) > 0.0 ? fma(g * om, rd[j], h[j]) : fma(e.x, g, h[j]);
+                g *= ex;
+            }
+        }
+    }
+}
+
+// the number of bins (sorted by kappa) with kappa_i n <= bound, a prefix; warp-uniform
+__device__ __forceinline__ int count_below(const float *s_kap, int n_active, int lane, float n, float bound)
+{
+    int b = 0;
+    for (int c0 = 0; c0 < n_active; c0 += 32) {
+        const int i = c0 + lane;
+        b += __popc(__ballot_sync(0xffffffffu, i < n_active && s_kap[i] * n <= bound));
+    }
+    return b;
+}
+
+// h of the lane's cells over all bins
+template <int C>
+__device__ __forceinline__ void absorb64(const TraceArgs &p, const double2 *s_nu64, const float *s_kap, int lane,
+                                         unsigned head_m, const Cells<double, C> &N, const Cells<double, C> &D,
+                                         double (&h)[C])
+{
+    // the warp's largest end column, smallest column and largest dN from the high words of the
+    // FP64 values (non-negative doubles order as their bits; integer, off the FP64 pipe),
+    // rounded outwards. A negative or NaN column (invalid input) only moves class bounds.
+    int nhi = 0, nlo = 0x7fefffff, dhi = 0;
+#pragma unroll
+    for (int j = 0; j < C; ++j) {
+        nhi = max(nhi, __double2hiint(N.get(j) + D.get(j)));
+        nlo = min(nlo, __double2hiint(N.get(j)));
+        dhi = max(dhi, __double2hiint(D.get(j)));
+    }
+    nhi = __reduce_max_sync(0xffffffffu, nhi);
+    nlo = max(__reduce_min_sync(0xffffffffu, nlo), 0);
+    dhi = __reduce_max_sync(0xffffffffu, dhi);
+    const float nmax = (float)__hiloint2double(nhi + 1, 0);
+    const float nmin = (float)__hiloint2double(nlo, 0);
+    const float dmax = (float)__hiloint2double(dhi + 1, 0);
+    const int na = p.n_active;
+    const int bt = count_below(s_kap, na, lane, nmax, 1.0f);
+    // e^{-x} is 0 in FP64 from x = 746 on; a column of 0 (or 0 x Inf) keeps every bin
+    int live = na;
+    if (nmin > 0.0f) live = max(count_below(s_kap, na, lane, nmin, 747.0f), bt);
+#pragma unroll
+    for (int j = 0; j < C; ++j) h[j] = 0.0;
+    if (bt > 0) {
+        const double *row = reinterpret_cast<const double *>(p.nu64 + kNu64Table) + bt * kThinStride64;
+        const double s = __ldg(row);
+        double cc[C], aa[C], dd[C], pc[C];
+        const double c0 = __ldg(row + kThinTerms64), c1 = __ldg(row + kThinTerms64 - 1);
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            cc[j] = s * N.get(j);
+            aa[j] = fma(s, D.get(j), cc[j]);
+            dd[j] = c0;
+            pc[j] = fma(c0, cc[j], c1);
+        }
+#pragma unroll
+        for (int k = kThinTerms64 - 2; k >= 1; --k) {
+            const double ck = __ldg(row + k);
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                dd[j] = fma(dd[j], aa[j], pc[j]);
+                pc[j] = fma(pc[j], cc[j], ck);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < C; ++j) h[j] = s * fma(dd[j], aa[j], pc[j]);
+    }
+    if (bt < live) {
+        const int b5 = min(max(count_below(s_kap, na, lane, dmax, kX64T5), bt), live);
+        const int b8 = min(max(count_below(s_kap, na, lane, dmax, kX64T8), bt), live);
+        const int b13 = min(max(count_below(s_kap, na, lane, dmax, kX64T13), bt), live);
+        bins64<5, C>(bt, b5, s_nu64, head_m, N, D, h);
+        bins64<8, C>(b5, b8, s_nu64, head_m, N, D, h);
+        bins64<13, C>(b8, b13, s_nu64, head_m, N, D, h);
+        bins64<0, C>(b13, live, s_nu64, head_m, N, D, h);
+    }
+}
+
+// sum_i F_i/F_max e^{-kappa_i n} of one ray, the warp's lanes sharing the bins beyond the thin
+// ones (that part from the series row); the result in every lane
+__device__ __forceinline__ double escape64(const TraceArgs &p, const double2 *s_nu64, const float *s_kap, int lane,
+                                           double n)
+{
+    const float nf = (float)__hiloint2double(max(__double2hiint(n), 0) + 1, 0);
+    const int bt = count_below(s_kap, p.n_active, lane, nf, 1.0f);
+    double s = 0.0;
+    for (int i = bt + lane; i < p.n_active; i += 32) s += s_nu64[i].y * exp(-s_nu64[i].x * n);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (bt > 0) {
+        const double *row = reinterpret_cast<const double *>(p.nu64 + kNu64Table) + bt * kThinStride64;
+        const double u = __ldg(row) * n;
+        double q = __ldg(row + kThinTerms64);
+#pragma unroll
+        for (int k = kThinTerms64 - 1; k >= 1; --k) q = fma(q, u, __ldg(row + k));
+        s += fma(-q, u, __ldg(row + kThinTerms64 + 1));
+    }
+    return s;
+}
+
 // One CTA traces the tiles [t_begin, t_end) of the grid described by p,
 // prefetching tile t+1 (cp.async, double buffer) while it computes tile t and
 // handing the column of the ray that runs into the next tile over in shared
@@ -169,7 +352,7 @@ __device__ __forceinline__ void trace_tile_range(const TraceArgs &p, unsigned t_
         const int kl = (int)(fl - rayl * R1);
         const int idx0 = (int)(rayl * (unsigned)nr + (unsigned)(kl < nr ? kl : nr) - m0);
         Cells<Real, C> D, N;
-        unsigned real_m = 0, virt_m = 0, head_m = 0, zero_m = 0;
+        unsigned real_m = 0, virt_m = 0, head_m = 0, zero_m = 0;  // FP64 mode: zero_m = cells with dust
         bool bad = false;
         {
             int k = kl, idx = idx0;
@@ -183,7 +366,7 @@ __device__ __forceinline__ void trace_tile_range(const TraceArgs &p, unsigned t_
                         const float rho = s_rho[skew(idx)], td = s_t[skew(idx)];
                         bad |= !(rho >= 0.0f && rho <= FLT_MAX) || (td != td);
                         D.set(j, column(rho, td, k));
-                        if (td <= p.t_sub && D.get(j) == Real(0)) zero_m |= 1u << j;
+                        if (td <= p.t_sub && (MODE == RT_FP64 || D.get(j) == Real(0))) zero_m |= 1u << j;
                         ++idx;
                     } else {
                         virt_m |= 1u << j;
@@ -244,16 +427,11 @@ __device__ __forceinline__ void trace_tile_range(const TraceArgs &p, unsigned t_
         Cells<Real, C> acc;
 #pragma unroll
         for (int j = 0; j < C; ++j) acc.set(j, Real(0));
+        double h64[MODE == RT_FP64 ? C : 1];
         if constexpr (MODE == RT_FP64) {
-#pragma unroll 1
-            for (int i = 0; i < p.nnu_pad; ++i) {
-                const double2 e = s_nu64[i];  // (kappa_i, F_i / F_max)
+            absorb64<C>(p, s_nu64, s_kap, lane, head_m, N, D, h64);
 #pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    const double g = e.y * exp(-e.x * N.get(j));
-                    acc.set(j, fma(g, -expm1(-e.x * D.get(j)), acc.get(j)));
-                }
-            }
+            for (int j = 0; j < C; ++j) acc.set(j, D.get(j) * h64[j]);
         } else {
             // the warp's largest and smallest non-zero column decide each bin's class
             float dmax = 0.0f, dmin = INFINITY;
@@ -278,17 +456,17 @@ __device__ __forceinline__ void trace_tile_range(const TraceArgs &p, unsigned t_
 
         // rho == 0 cells with dust: the force limit sum_i kappa_i g_i (rare; per
         // slot, only in warps that hold such a cell). Reuses D (0 there).
+        if constexpr (MODE != RT_FP64) {
         if (__any_sync(0xffffffffu, zero_m != 0u)) {
 #pragma unroll
         for (int j = 0; j < C; ++j) {
             if (__any_sync(0xffffffffu, (zero_m >> j) & 1u)) {
                 Real s = Real(0);
-                for (int i = 0; i < p.nnu_pad; ++i) {
-                    if constexpr (MODE == RT_FP64) s = fma((double)s_kap[i] * s_nu64[i].y, exp(-s_nu64[i].x * N.get(j)), s);
-                    else s = fmaf(s_kap[i], ex2_approx(fmaf(s_nu[i].x, N.get(j), s_nu[i].z)), s);
-                }
+                for (int i = 0; i < p.nnu_pad; ++i)
+                    s = fmaf(s_kap[i], ex2_approx(fmaf(s_nu[i].x, N.get(j), s_nu[i].z)), s);
                 if ((zero_m >> j) & 1u) D.set(j, s);
             }
+        }
         }
         }
 
@@ -303,11 +481,12 @@ __device__ __forceinline__ void trace_tile_range(const TraceArgs &p, unsigned t_
                 const Real ntot = __shfl_sync(0xffffffffu, N.get(j), src);
                 const unsigned fsrc = __shfl_sync(0xffffffffu, fl, src) + (unsigned)j;
                 Real s = Real(0);
-                for (int i = lane; i < p.nnu_pad; i += 32) {
-                    if constexpr (MODE == RT_FP64) s += s_nu64[i].y * exp(-s_nu64[i].x * ntot);
-                    else s += ex2_approx(fmaf(s_nu[i].x, ntot, s_nu[i].z));
+                if constexpr (MODE == RT_FP64) {
+                    s = escape64(p, s_nu64, s_kap, lane, ntot);
+                } else {
+                    for (int i = lane; i < p.nnu_pad; i += 32) s += ex2_approx(fmaf(s_nu[i].x, ntot, s_nu[i].z));
+                    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                 }
-                for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                 if (lane == 0) eesc.add(s * solid_angle<MODE>(p, p.r1div.div(fsrc)));
             }
         }
@@ -338,8 +517,8 @@ __device__ __forceinline__ void trace_tile_range(const TraceArgs &p, unsigned t_
                     Real q, a;
                     if constexpr (MODE == RT_FP64) {
                         const RadRow64 g = p.rtab64[k];
-                        q = zc ? 0.0 : g.y * acc.get(j);
-                        a = g.z * (zc ? dj : (dj > 0.0 ? acc.get(j) / dj : 0.0));
+                        q = g.y * acc.get(j);
+                        a = zc ? g.z * h64[j] : 0.0;  // zc: a cell with dust
                     } else {
                         q = (dj > 0.0f && !zc) ? rad_gq(k) * acc.get(j) : 0.0f;
                         a = rad_ga(k) * (zc ? dj : (dj > 0.0f ? __fdividef(acc.get(j), dj) : 0.0f));
