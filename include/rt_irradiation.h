@@ -444,18 +444,18 @@ typedef struct rt_fld_stats {
  *   e_new       device, same layout, caller-allocated, not aliasing e_old: E_R after it;
  *   dt (s) > 0 (1e300 gives the steady state), c_v (erg g^-1 K^-1) >= 0,
  *   t_bg (K) >= 0: E = a t_bg^4 half a cell beyond the outer radius;
- *   tol > 0, max_iter >= 1: mixed-precision iterative refinement (true residual in
- *   FP32, conjugate gradients for each correction, FP64 reductions) from
- *   E' = E_old until a pass changes no cell by more than tol relative, or max_iter
- *   conjugate-gradient iterations in total. Grids of more than 512 cells are
- *   preconditioned by an aggregation-multigrid V-cycle (Galerkin coarse levels
- *   halving every direction), smaller ones by Jacobi.
- *   stats       NULL or a host struct: iterations, refinement passes, the last
- *               pass's relative change and the number of multigrid levels.
+ *   tol > 0, max_iter >= 1: conjugate gradients (FP32 vectors, FP64 reductions) from
+ *   E' = E_old in groups of steps; after each group the residual is taken afresh, and
+ *   the solve ends when a group changed no cell by more than tol relative, or after
+ *   max_iter iterations in total. Grids of more than 512 cells are preconditioned by an
+ *   aggregation-multigrid V-cycle (Galerkin coarse levels halving every direction; next
+ *   to the poles whole phi rings are smoothed at once), smaller ones by Jacobi.
+ *   stats       NULL or a host struct: iterations, passes (groups), the last
+ *               group's relative change and the number of multigrid levels.
  * Finite volumes: harmonic-mean face coefficients, no flux through the inner radius
  * or the theta ends, periodic in phi when nphi > 1 (the wrap distance measured
  * around the full circle). Runs on a private stream ordered after the context's
- * stream and synchronises it every 8 iterations; returns with e_new complete. Errors:
+ * stream and synchronises it at the end; returns with e_new complete. Errors:
  * RT_ERR_NOT_CONFIGURED, RT_ERR_INVALID_ARG, RT_ERR_NONFINITE_INPUT (rho < 0,
  * T <= 0, E_old < 0, q_abs < 0 or NaN/Inf; e_new is then unchanged),
  * RT_ERR_TIMEOUT (tol not reached in max_iter; e_new holds the last iterate),

@@ -14,15 +14,16 @@
 // F = (2 s' + g') / (6 s'^2 + 3 s' g' + g'^2), s' = kappa_R rho L, g' = L |grad E| / E.
 //
 // The matrix is symmetric positive definite. It is applied matrix-free and solved
-// by Jacobi-preconditioned conjugate gradients inside mixed-precision iterative
-// refinement (FP32 vectors, FP64 reductions, every scalar of the iteration kept on
-// the device), from E_old, until the last refinement changed no cell by more than
-// tol relative.
+// by multigrid-preconditioned conjugate gradients with residual replacement (FP32
+// vectors, FP64 reductions, every scalar and the loop itself on the device), from
+// E_old, until a group of steps changed no cell by more than tol relative.
 #include <cuda_bf16.h>
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "rt_internal.cuh"
@@ -35,9 +36,13 @@ constexpr double kRossLnLo = 0.0, kRossLnHi = 11.512925464970229;  // ln 1 K .. 
 
 struct FldState {
     long long cap = 0;
-    float *buf = nullptr;  // F, tc, b0, w[3], s, 1/dg, b, d, r, p, q, z: 15 n floats, then BF16
-                           // copies of s, w[3], 1/dg (5 n halves) for the finest V-cycle
+    float *buf = nullptr;  // F (then the second p), tc (then x), b0, w[3], s, 1/dg, b, d, r, p, q, z:
+                           // 14 n floats, then BF16 copies of s, w[3], 1/dg (5 n halves) for the
+                           // finest V-cycle
     float *mg_buf = nullptr;              // coarse levels: s, w[3], 1/dg, b, x each
+    float *line_buf = nullptr;            // phi-line smoother: factors, separator inverses, x
+    int line_j0 = 0, line_j1 = 0;         // rows j < line_j0 and j >= line_j1 are smoothed by phi lines
+    bool lines_set = false;
     std::vector<int> mg_dims;             // (nr, ntheta, nphi) of every level, finest first
     double *part = nullptr, *scal = nullptr;
     unsigned *bad = nullptr, *count = nullptr;
@@ -46,13 +51,13 @@ struct FldState {
     float *lkr = nullptr;  // ln kappa_R on the ln T nodes
     unsigned long long lkr_fp = 0;
     bool lkr_valid = false;
-    // the solve runs on a private stream (after the context's stream), so that its
-    // inner-iteration bursts can be captured and replayed as a CUDA graph
+    // the solve runs on a private stream, after the context's stream; its loop is a graph with
+    // a conditional node that points at this workspace only (built once per context)
     cudaStream_t gs = nullptr;
     cudaEvent_t ev_in = nullptr;
-    cudaGraphExec_t burst = nullptr;
-    const void *burst_x = nullptr, *burst_buf = nullptr;  // what the captured launches point at
-    bool no_graph = false;
+    cudaGraphExec_t loop = nullptr;
+    bool no_graph = false;  // the graph could not be built: the host drives the loop
+    double *scal_h = nullptr;  // pinned: the scalars and the validity word of the last solve
 };
 
 namespace {
@@ -207,7 +212,8 @@ struct FldFaceArgs {
     FldGeo g;
     const float *F, *tc, *b0;
     float e_bg;               // a T_bg^4
-    float *w, *s, *idg, *b;   // w [3][n]: to the k+1, j+1 and l+1 neighbours
+    const float *e;           // E_old, the solve's start value x
+    float *w, *s, *idg, *b, *x;  // w [3][n]: to the k+1, j+1 and l+1 neighbours
     unsigned short *hs, *hw, *hidg;  // BF16 copies of s, w, 1/dg (the finest V-cycle's operator)
     long long n;
 };
@@ -260,6 +266,7 @@ __global__ void __launch_bounds__(256) k_fld_faces(const FldFaceArgs p)
         p.s[c] = sc;
         p.idg[c] = idg;
         p.b[c] = rhs;
+        p.x[c] = p.e[c];  // x may be tc's buffer: this cell's tc is read above, no other's
         p.hw[c] = __bfloat16_as_ushort(__float2bfloat16_rn(wr));
         p.hw[n + c] = __bfloat16_as_ushort(__float2bfloat16_rn(wt));
         p.hw[2 * n + c] = __bfloat16_as_ushort(__float2bfloat16_rn(wp));
@@ -273,26 +280,43 @@ __global__ void __launch_bounds__(256) k_fld_faces(const FldFaceArgs p)
 // and boundary term s is stored apart from the face weights, so nothing small is
 // left as the difference of large rounded numbers (a diagonal holding s + sum w
 // would bury s under the rounding of the face weights wherever diffusion dominates).
-// Mixed-precision iterative refinement: each pass computes the true residual
-// r = b - A x, solves A d = r by preconditioned CG from d = 0 until the
-// preconditioned residual norm fell by the inner drop, and adds d to x. FP32
-// recurrences lose the true residual after a few hundred iterations; the restart
-// from the true residual recovers it, and the passes end when max |d| / |x| < tol.
-// The drops were measured per step on the 256x128x256 disk: with multigrid, loose
-// inner solves and more passes are cheapest (0.2: 65.8 ms, 12 passes; 1e-2: 77.9
-// ms, 6 passes); for Jacobi, 1e-2 took the fewest iterations in an FP32 emulation.
-constexpr double kInnerDrop = 1e-2;    // Jacobi-preconditioned inner solves
-constexpr double kInnerDropMg = 2e-1;  // multigrid-preconditioned inner solves
+//
+// Preconditioned conjugate gradients with group-wise residual replacement (Sleijpen and
+// van der Vorst 1996): the steps of a group add up in d; once r.z fell by kGroupDrop^2, d
+// goes into x, r is taken afresh as b - A x (FP32 recurrences lose the true residual after a
+// few hundred steps) and the directions carry on. The groups end when max |d| / |x| < tol.
+// Keeping the directions over a replacement took 37 steps against 41 with restarts (FP64
+// emulation, 128x64x64), and a group costs one stencil pass in place of an update.
+//
+// One iteration is a fixed list of kernels whose scalars live on the device:
+//   k_it_flush     (at a group's end only) x += d; max |d| / |x|; done?
+//   k_it_residual  r -= alpha q, or r = b - A x after a flush; the phi lines' first solve
+//   k_mg_down ... k_mg_tail ... k_mg_up: z = M^-1 r, r.z, beta (k_it_jacobi on small grids)
+//   k_it_apply     d += alpha p; p = z + beta p; q = A p; alpha = r.z / p.q
+// so p, q, d move once per iteration (the direction update and the step are folded into
+// passes that read their arrays anyway). The loop is a graph with a conditional node, kUnroll
+// iterations per body: no host round trip until the solve is done, no idle launches but the
+// last body's.
+constexpr double kGroupDrop = 0.1;
+constexpr int kUnroll = 4;  // even: p alternates between two buffers
 
 // device scalars of the solve
 enum : int {
-    kRz = 0,     // r.z of the current inner iterate
-    kRz0,        // r.z at the start of the inner solve
+    kRz = 0,   // r.z
+    kRz0,      // r.z at the start of the group
     kAlpha,
     kBeta,
-    kDone,       // 1 once the inner solve converged (the remaining launches return at once)
-    kIters,      // inner iterations taken in total
-    kCorr,       // max |d| / |x| of the last pass (infinite: x not finite)
+    kPend,     // 1: the step alpha p is not yet in d
+    kDLive,    // 1: d holds steps of this group (else it counts as 0)
+    kFlush,    // 1: the group ends before the next residual; 2: first residual of the solve
+    kLast,     // 1: max_iter reached, the next flush ends the solve
+    kDone,     // 1: x is final (or the input was invalid); every later launch returns at once
+    kIters,
+    kPasses,   // groups
+    kCorr,     // max |d| / |x| of the last group (infinite: x not finite)
+    kTol,
+    kMaxIter,
+    kLoops,    // bodies of the loop run so far
     kNScal
 };
 
@@ -301,80 +325,81 @@ struct CgArgs {
     FastDiv div_nr, div_nth;
     long long n;
     const float *w, *s, *idg, *b;
-    float *x, *d, *r, *p, *q;
+    float *x, *d, *r, *q, *z;
     double *part;     // [grid]
     double *scal;     // kNScal
     unsigned *count;  // blocks finished (last-block reductions)
 };
 
-__device__ __forceinline__ float apply_flux(const CgArgs &a, const float *v, unsigned c)
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
+// operator entries in FP32, or the finest V-cycle's BF16 copies
+__device__ __forceinline__ float4 ldo4(const float *p) { return ld4(p); }
+__device__ __forceinline__ float ldo1(const float *p) { return *p; }
+__device__ __forceinline__ float4 ldo4(const unsigned short *p)
 {
-    int k, j, l;
-    cell_ijk(c, a.nr, a.nth, a.div_nr, a.div_nth, k, j, l);
-    const unsigned n = (unsigned)a.n, plane = (unsigned)a.nr * (unsigned)a.nth;
-    const float vc = v[c];
-    float acc = a.s[c] * vc;
-    if (k + 1 < a.nr) acc = fmaf(a.w[c], vc - v[c + 1], acc);
-    if (k > 0) acc = fmaf(a.w[c - 1], vc - v[c - 1], acc);
-    if (j + 1 < a.nth) acc = fmaf(a.w[n + c], vc - v[c + a.nr], acc);
-    if (j > 0) acc = fmaf(a.w[n + c - a.nr], vc - v[c - a.nr], acc);
-    if (a.nph > 1) {
-        const unsigned cb = l + 1 < a.nph ? c + plane : c - (unsigned)l * plane;
-        const unsigned ca = l > 0 ? c - plane : c + (unsigned)(a.nph - 1) * plane;
-        acc = fmaf(a.w[2 * n + c], vc - v[cb], acc);
-        acc = fmaf(a.w[2 * n + ca], vc - v[ca], acc);
+    const uint2 u = *reinterpret_cast<const uint2 *>(p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xffff0000u));
+}
+__device__ __forceinline__ float ldo1(const unsigned short *p) { return __uint_as_float((unsigned)*p << 16); }
+
+// A v at cell c = (k, j, l); v(i, k', j', l') gives the neighbours' values
+template <class T, class V>
+__device__ __forceinline__ float flux_one(int nr, int nth, int nph, unsigned n, const T *s, const T *w, const V &v,
+                                          unsigned c, int k, int j, int l, float vc)
+{
+    const unsigned plane = (unsigned)nr * (unsigned)nth;
+    float acc = ldo1(s + c) * vc;
+    if (k + 1 < nr) acc = fmaf(ldo1(w + c), vc - v(c + 1, k + 1, j, l), acc);
+    if (k > 0) acc = fmaf(ldo1(w + c - 1), vc - v(c - 1, k - 1, j, l), acc);
+    if (j + 1 < nth) acc = fmaf(ldo1(w + n + c), vc - v(c + nr, k, j + 1, l), acc);
+    if (j > 0) acc = fmaf(ldo1(w + n + c - nr), vc - v(c - nr, k, j - 1, l), acc);
+    if (nph > 1) {
+        const int lb = l + 1 < nph ? l + 1 : 0, la = l > 0 ? l - 1 : nph - 1;
+        const unsigned cb = c + (unsigned)(lb - l) * plane, ca = c + (unsigned)(la - l) * plane;
+        acc = fmaf(ldo1(w + 2 * n + c), vc - v(cb, k, j, lb), acc);
+        acc = fmaf(ldo1(w + 2 * n + ca), vc - v(ca, k, j, la), acc);
     }
     return acc;
 }
 
-// block reduction (sum, or max for MAX) into thread 0
-template <bool MAX>
-__device__ double block_reduce(double v)
+// A v on the quad c .. c+3 of one ray (nr % 4 == 0: the four cells share (j, l) and every
+// offset is a multiple of 16 bytes); vrow gives the quad at the same k of another row, v one cell
+template <class T, class VR, class V>
+__device__ __forceinline__ float4 flux_quad(int nr, int nth, int nph, unsigned n, const T *s_, const T *w_,
+                                            const VR &vrow, const V &v, unsigned c, int k, int j, int l, float4 vc)
 {
-    __shared__ double s_w[32];
-    for (int o = 16; o > 0; o >>= 1) {
-        const double u = __shfl_xor_sync(0xffffffffu, v, o);
-        v = MAX ? fmax(v, u) : v + u;
+    const unsigned plane = (unsigned)nr * (unsigned)nth;
+    const float4 s = ldo4(s_ + c), wr = ldo4(w_ + c);
+    float4 acc = make_float4(s.x * vc.x, s.y * vc.y, s.z * vc.z, s.w * vc.w);
+    acc.x = fmaf(wr.x, vc.x - vc.y, acc.x);
+    acc.y = fmaf(wr.y, vc.y - vc.z, acc.y);
+    acc.z = fmaf(wr.z, vc.z - vc.w, acc.z);
+    acc.y = fmaf(wr.x, vc.y - vc.x, acc.y);
+    acc.z = fmaf(wr.y, vc.z - vc.y, acc.z);
+    acc.w = fmaf(wr.z, vc.w - vc.z, acc.w);
+    if (k + 4 < nr) acc.w = fmaf(wr.w, vc.w - v(c + 4, k + 4, j, l), acc.w);
+    if (k > 0) acc.x = fmaf(ldo1(w_ + c - 1), vc.x - v(c - 1, k - 1, j, l), acc.x);
+    auto face4 = [&](float4 w, float4 u) {
+        acc.x = fmaf(w.x, vc.x - u.x, acc.x);
+        acc.y = fmaf(w.y, vc.y - u.y, acc.y);
+        acc.z = fmaf(w.z, vc.z - u.z, acc.z);
+        acc.w = fmaf(w.w, vc.w - u.w, acc.w);
+    };
+    if (j + 1 < nth) face4(ldo4(w_ + n + c), vrow(c + nr, k, j + 1, l));
+    if (j > 0) face4(ldo4(w_ + n + c - nr), vrow(c - nr, k, j - 1, l));
+    if (nph > 1) {
+        const int lb = l + 1 < nph ? l + 1 : 0, la = l > 0 ? l - 1 : nph - 1;
+        const unsigned cb = c + (unsigned)(lb - l) * plane, ca = c + (unsigned)(la - l) * plane;
+        face4(ldo4(w_ + 2 * n + c), vrow(cb, k, j, lb));
+        face4(ldo4(w_ + 2 * n + ca), vrow(ca, k, j, la));
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) s_w[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t = MAX ? fmax(t, s_w[i]) : t + s_w[i];
-    return t;
-}
-
-// Writes this block's partial; the block that finishes last reduces all partials in
-// a fixed order (deterministic) and returns true in its thread 0 with the total.
-template <bool MAX>
-__device__ bool grid_reduce(const CgArgs &a, double v, double *out)
-{
-    __shared__ bool s_last;
-    const double t = block_reduce<MAX>(v);
-    if (threadIdx.x == 0) {
-        a.part[blockIdx.x] = t;
-        __threadfence();
-        s_last = atomicAdd(a.count, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return false;
-    double u = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) {
-        const double pi = __ldcg(a.part + i);
-        u = MAX ? fmax(u, pi) : u + pi;
-    }
-    const double tot = block_reduce<MAX>(u);
-    if (threadIdx.x == 0) {
-        *out = tot;
-        *a.count = 0u;
-    }
-    return threadIdx.x == 0;
+    return acc;
 }
 
 // Per-thread sums in compensated FP32 (TwoSum; GB300's FP64 rate is a small
-// fraction of its FP32 rate), handed to the FP64 block and grid reductions once.
+// fraction of its FP32 rate). A block's sum stays a pair of floats (48 bits), its partial is FP64.
 struct KSum {
     float s = 0.0f, c = 0.0f;
     __device__ __forceinline__ void add(float v)
@@ -384,225 +409,572 @@ struct KSum {
         c += (s - (t - bp)) + (v - bp);
         s = t;
     }
+    __device__ __forceinline__ void add(const KSum &o)
+    {
+        add(o.s);
+        c += o.c;
+    }
+    __device__ __forceinline__ KSum shfl(int m) const
+    {
+        KSum r;
+        r.s = __shfl_xor_sync(0xffffffffu, s, m);
+        r.c = __shfl_xor_sync(0xffffffffu, c, m);
+        return r;
+    }
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
-
-#define FLD_CELLS(c)                                                                          \
-    for (unsigned c = blockIdx.x * blockDim.x + threadIdx.x; c < (unsigned)a.n; c += gridDim.x * blockDim.x)
-
-// r = b - A x, d = 0, p = z = r / dg; rz0 = r.z; restarts the inner solve
-__global__ void __launch_bounds__(256) k_cg_residual(const CgArgs a)
-{
-    KSum rz;
-    FLD_CELLS(c)
+struct KMax {
+    float s = 0.0f;
+    __device__ __forceinline__ void add(const KMax &o) { s = fmaxf(s, o.s); }
+    __device__ __forceinline__ KMax shfl(int m) const
     {
-        const float rc = a.b[c] - apply_flux(a, a.x, c);
-        const float zc = rc * a.idg[c];
-        a.r[c] = rc;
-        a.d[c] = 0.0f;
-        a.p[c] = zc;
-        rz.add(rc * zc);
+        KMax r;
+        r.s = __shfl_xor_sync(0xffffffffu, s, m);
+        return r;
+    }
+    __device__ __forceinline__ double value() const { return (double)s; }
+};
+struct DSum {  // the last block's sum of the FP64 partials
+    double s = 0.0;
+    __device__ __forceinline__ void add(const DSum &o) { s += o.s; }
+    __device__ __forceinline__ DSum shfl(int m) const
+    {
+        DSum r;
+        r.s = __shfl_xor_sync(0xffffffffu, s, m);
+        return r;
+    }
+};
+
+// block reduction into thread 0: two levels of shuffles
+template <class S>
+__device__ __forceinline__ S block_reduce(S v)
+{
+    __shared__ S s_w[32];
+    for (int o = 16; o > 0; o >>= 1) v.add(v.shfl(o));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __syncthreads();
+    if (lane == 0) s_w[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        v = lane < nw ? s_w[lane] : S();
+        for (int o = 16; o > 0; o >>= 1) v.add(v.shfl(o));
+    }
+    return v;
+}
+
+// Writes this block's partial at part[at + blockIdx.x]; the block that finishes last reduces the
+// first at + gridDim.x partials in a fixed order (deterministic) and returns true in its thread 0
+// with the total. (at: the partials an earlier kernel left for this one.)
+template <class S>
+__device__ bool grid_reduce(const CgArgs &a, const S &v, double *out, int at = 0)
+{
+    __shared__ bool s_last;
+    const S t = block_reduce(v);
+    if (threadIdx.x == 0) {
+        a.part[at + blockIdx.x] = t.value();
+        __threadfence();
+        s_last = atomicAdd(a.count, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last) return false;
+    constexpr bool kMax = std::is_same<S, KMax>::value;
+    DSum u;
+    KMax m;
+    for (int i = threadIdx.x; i < at + (int)gridDim.x; i += blockDim.x) {
+        const double pi = __ldcg(a.part + i);
+        if (kMax) m.s = fmaxf(m.s, (float)pi);
+        else u.s += pi;
     }
     double tot;
-    if (grid_reduce<false>(a, rz.value(), &tot)) {
-        a.scal[kRz] = tot;
-        a.scal[kRz0] = tot;
-        a.scal[kDone] = tot > 0.0 ? 0.0 : 1.0;
+    if constexpr (kMax) tot = block_reduce(m).value();
+    else tot = block_reduce(u).s;
+    if (threadIdx.x == 0) {
+        *out = tot;
+        *a.count = 0u;
+    }
+    return threadIdx.x == 0;
+}
+
+// the level-0 kernels' cells: quads of one ray (Q) or single cells, the blocks from b0 on
+template <bool Q, class F>
+__device__ __forceinline__ void for_cells(const CgArgs &a, unsigned b0, const F &f)
+{
+    constexpr unsigned W = Q ? 4u : 1u;
+    for (unsigned c = W * ((blockIdx.x - b0) * blockDim.x + threadIdx.x); c < (unsigned)a.n;
+         c += W * (gridDim.x - b0) * blockDim.x) {
+        int k, j, l;
+        cell_ijk(c, a.nr, a.nth, a.div_nr, a.div_nth, k, j, l);
+        f(c, k, j, l);
     }
 }
 
-// q = A p; alpha = rz / p.q
-__global__ void __launch_bounds__(256) k_cg_apply(const CgArgs a)
-{
-    if (a.scal[kDone] != 0.0) return;
-    KSum pq;
-    FLD_CELLS(c)
+// Rows smoothed by whole phi lines on the finest level. Next to the poles the phi faces are
+// close together and a row couples to itself in phi far more strongly (as 1 / sin^2 theta) than
+// to its neighbours, which a point smoother and 2 x 2 x 2 aggregates cannot follow: the slowest
+// modes of the point-smoothed V-cycle all sat there. So in the rows where the phi faces hold
+// more than kLineShare of the diagonal (geometry only; a run of rows at each theta end) the
+// Jacobi diagonal of the smoother is replaced by the row's periodic tridiagonal blocks T (one
+// phi ring per (j, k)): x0 = omega T^-1 b before the restriction and x1 + omega T^-1 (b - A x1)
+// after the prolongation, symmetric as before and omega lambda(T^-1 A) < 2 as for the points.
+// FP64 PCG on the CPU to a 1e-8 residual: 79 -> 31 iterations on 128x64x64 with 12 % of the
+// rows; lines in every row 29, radial lines 79. On the GPU 253 -> 60 iterations per step on
+// 256x128x256 (dt = 1e4 s), and the largest error of a cell 1.7e-4 -> 5e-6.
+struct LineOp {
+    int j0, j1, nl;             // rows j < j0 and j >= j1: nl of them (j0 = 0, j1 = nth: none)
+    int seg;                    // segments a ring is cut into (its last cells are the separators)
+    int blocks;                 // CTAs of the line role: one per row and 32 k
+    float *m, *vl, *vr, *inv;   // [nph][nl][nr]: pivots, responses to the left and right separator;
+                                // [nl][seg][seg][nr]: inverse of the separators' Schur complement
+    float *x, *res;             // [nph][nl][nr]: omega T^-1 b, and the residual of the second solve
+    __device__ __forceinline__ bool has(int j) const { return j < j0 || j >= j1; }
+    __device__ __forceinline__ unsigned at(int nr, int k, int j, int l) const
     {
-        const float qc = apply_flux(a, a.p, c);
-        a.q[c] = qc;
-        pq.add(a.p[c] * qc);
+        return ((unsigned)l * (unsigned)nl + (unsigned)(j < j0 ? j : j - j1 + j0)) * (unsigned)nr + (unsigned)k;
     }
-    double tot;
-    if (grid_reduce<false>(a, pq.value(), &tot)) {
-        a.scal[kAlpha] = tot > 0.0 ? a.scal[kRz] / tot : 0.0;
-        if (!(tot > 0.0)) a.scal[kDone] = 1.0;
-    }
-}
+};
+constexpr int kLineMaxSeg = 16;
+constexpr int kLineChunk = 8;        // cells whose loads a thread has in flight together
+constexpr double kLineShare = 0.85;  // of the diagonal held by the phi faces
+constexpr int kLineMinPhi = 16;
+constexpr int kLineSmemPhi = 1024;   // rings up to this keep the sweep's values in shared memory
 
-// d += alpha p, r -= alpha q; beta = rz_new / rz; done once rz_new <= drop^2 rz0
-__global__ void __launch_bounds__(256) k_cg_update(const CgArgs a)
+// The ring of one row j and 32 consecutive k per block: lane = k, warp = ring segment
+// (coalesced along k; a ring's cells lie a plane apart). Each segment eliminates its interior
+// with zero separators, the separators (its last cell) follow from the precomputed inverse of
+// their cyclic Schur complement, and the interior takes the two separators' responses: the
+// dependent chain is nph / seg cells instead of nph. The few rings are latency-bound, so the
+// loads of a chunk of cells are issued before its arithmetic and its stores (256x128x256: 26 and
+// 39 us per solve with loads and stores interleaved, 22 us, 512 threads at 64 registers).
+// lb(c, i) and sb(c, b): load and keep the right-hand side of cell c; ld(c, i, e) loads what out
+// needs; out(c, i, x, e) takes the solution (i: the cell's index in the line arrays).
+// SM: the sweep's values in shared memory, else in gy (a line array that lb has read).
+template <bool SM, class LB, class SB, class LD, class OUT>
+__device__ __forceinline__ void line_solve(const LineOp &L, const CgArgs &a, float *gy, const LB &lb, const SB &sb,
+                                           const LD &ld, const OUT &out)
 {
-    if (a.scal[kDone] != 0.0) return;
-    const float alpha = (float)a.scal[kAlpha];
-    KSum rz;
-    FLD_CELLS(c)
-    {
-        a.d[c] = fmaf(alpha, a.p[c], a.d[c]);
-        const float rc = fmaf(-alpha, a.q[c], a.r[c]);
-        a.r[c] = rc;
-        rz.add(rc * (rc * a.idg[c]));
-    }
-    double tot;
-    if (grid_reduce<false>(a, rz.value(), &tot)) {
-        a.scal[kBeta] = a.scal[kRz] > 0.0 ? tot / a.scal[kRz] : 0.0;
-        a.scal[kRz] = tot;
-        a.scal[kIters] += 1.0;
-        if (!(tot > kInnerDrop * kInnerDrop * a.scal[kRz0])) a.scal[kDone] = 1.0;
-    }
-}
-
-// p = r / dg + beta p
-__global__ void __launch_bounds__(256) k_cg_direction(const CgArgs a)
-{
-    if (a.scal[kDone] != 0.0) return;
-    const float beta = (float)a.scal[kBeta];
-    FLD_CELLS(c) a.p[c] = fmaf(beta, a.p[c], a.r[c] * a.idg[c]);
-}
-
-// x += d; kCorr = max |d| / |x|, capped at 1e30 (infinite if an x is not finite)
-__global__ void __launch_bounds__(256) k_cg_accumulate(const CgArgs a)
-{
-    float m = 0.0f;
-    FLD_CELLS(c)
-    {
-        const float dc = a.d[c];
-        const float xc = a.x[c] + dc;
-        a.x[c] = xc;
-        if (!isfinite(xc)) m = INFINITY;
-        else if (dc != 0.0f) m = fmaxf(m, fminf(fabsf(dc) / fmaxf(fabsf(xc), 1e-37f), 1e30f));
-    }
-    double tot;
-    if (grid_reduce<true>(a, (double)m, &tot)) a.scal[kCorr] = tot;
-}
-
-// --- the same kernels on four consecutive cells per thread (nr % 4 == 0: the four
-// cells share (j, l), every array offset is a multiple of 16 bytes) -----------------
-#define FLD_QUADS(c)                                                                          \
-    for (unsigned c = 4u * (blockIdx.x * blockDim.x + threadIdx.x); c < (unsigned)a.n;         \
-         c += 4u * gridDim.x * blockDim.x)
-
-__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
-
-// A v on cells c .. c+3 of one ray
-__device__ __forceinline__ float4 apply_flux4(const CgArgs &a, const float *v, unsigned c)
-{
-    int k, j, l;
-    cell_ijk(c, a.nr, a.nth, a.div_nr, a.div_nth, k, j, l);
-    const unsigned n = (unsigned)a.n, plane = (unsigned)a.nr * (unsigned)a.nth;
-    const float4 vc = ld4(v + c), s = ld4(a.s + c), wr = ld4(a.w + c);
-    float4 acc = make_float4(s.x * vc.x, s.y * vc.y, s.z * vc.z, s.w * vc.w);
-    // radial faces: inside the quad, and to c-1 / c+4
-    acc.x = fmaf(wr.x, vc.x - vc.y, acc.x);
-    acc.y = fmaf(wr.y, vc.y - vc.z, acc.y);
-    acc.z = fmaf(wr.z, vc.z - vc.w, acc.z);
-    acc.y = fmaf(wr.x, vc.y - vc.x, acc.y);
-    acc.z = fmaf(wr.y, vc.z - vc.y, acc.z);
-    acc.w = fmaf(wr.z, vc.w - vc.z, acc.w);
-    if (k + 4 < a.nr) acc.w = fmaf(wr.w, vc.w - v[c + 4], acc.w);
-    if (k > 0) acc.x = fmaf(a.w[c - 1], vc.x - v[c - 1], acc.x);
-    auto face4 = [&](float4 w, float4 u) {
-        acc.x = fmaf(w.x, vc.x - u.x, acc.x);
-        acc.y = fmaf(w.y, vc.y - u.y, acc.y);
-        acc.z = fmaf(w.z, vc.z - u.z, acc.z);
-        acc.w = fmaf(w.w, vc.w - u.w, acc.w);
+    extern __shared__ float s_y[];  // [longest interior][threads]
+    __shared__ float s_f[kLineMaxSeg][32], s_r[kLineMaxSeg][32], s_s[kLineMaxSeg][32];
+    constexpr int U = kLineChunk;
+    const int lane = threadIdx.x & 31, sg = threadIdx.x >> 5, S = L.seg, T = blockDim.x;
+    const int kt = (a.nr + 31) / 32;
+    const int jl = blockIdx.x / kt, k = (blockIdx.x - jl * kt) * 32 + lane;
+    const int j = jl < L.j0 ? jl : jl - L.j0 + L.j1;
+    const bool act = k < a.nr;
+    const int l0 = sg * a.nph / S, le = (sg + 1) * a.nph / S - 1;  // interior [l0, le), separator le
+    const unsigned plane = (unsigned)a.nr * (unsigned)a.nth, lp = (unsigned)L.nl * (unsigned)a.nr;
+    const unsigned c0 = (unsigned)j * a.nr + k, i0 = (unsigned)jl * a.nr + k;
+    const float *wp = a.w + 2 * a.n + c0;
+    auto yv = [&](int l) -> float & {
+        if constexpr (SM) return s_y[(l - l0) * T + threadIdx.x];
+        else return gy[i0 + l * lp];
     };
-    if (j + 1 < a.nth) face4(ld4(a.w + n + c), ld4(v + c + a.nr));
-    if (j > 0) face4(ld4(a.w + n + c - a.nr), ld4(v + c - a.nr));
-    if (a.nph > 1) {
-        const unsigned cb = l + 1 < a.nph ? c + plane : c - (unsigned)l * plane;
-        const unsigned ca = l > 0 ? c - plane : c + (unsigned)(a.nph - 1) * plane;
-        face4(ld4(a.w + 2 * n + c), ld4(v + cb));
-        face4(ld4(a.w + 2 * n + ca), ld4(v + ca));
+    float y = 0.0f, w0 = 0.0f, bs = 0.0f, wsep = 0.0f;
+    float mm[U], ww[U];
+    if (act) {
+        bs = lb(c0 + le * plane, i0 + le * lp);
+        wsep = __ldg(wp + le * plane);
+        for (int lc = l0; lc < le; lc += U) {
+            float bb[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (lc + u < le) {
+                    bb[u] = lb(c0 + (lc + u) * plane, i0 + (lc + u) * lp);
+                    mm[u] = __ldg(L.m + i0 + (lc + u) * lp);
+                    ww[u] = __ldg(wp + (lc + u) * plane);
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (lc + u < le) {
+                    y = fmaf(w0, y, bb[u]) * mm[u];
+                    w0 = ww[u];
+                    yv(lc + u) = y;
+                    sb(c0 + (lc + u) * plane, bb[u]);
+                }
+        }
+        sb(c0 + le * plane, bs);
+        // backward: from the last chunk (its factors are in registers) to the first
+        float x = 0.0f;
+        for (int lc = l0 + (le - 1 - l0) / U * U; lc >= l0; lc -= U) {
+            if (lc + U < le) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    mm[u] = __ldg(L.m + i0 + (lc + u) * lp);
+                    ww[u] = __ldg(wp + (lc + u) * plane);
+                }
+            }
+#pragma unroll
+            for (int u = U - 1; u >= 0; --u)
+                if (lc + u < le) {  // (x starts at 0: the last interior cell keeps its y)
+                    x = fmaf(ww[u] * mm[u], x, yv(lc + u));
+                    yv(lc + u) = x;
+                }
+        }
+        s_f[sg][lane] = x;
     }
-    return acc;
+    __syncthreads();
+    if (act) s_r[sg][lane] = bs + w0 * y + wsep * s_f[sg + 1 < S ? sg + 1 : 0][lane];
+    float iv[kLineMaxSeg];
+    if (act) {
+        const float *inv = L.inv + ((size_t)jl * S + sg) * S * a.nr + k;
+#pragma unroll
+        for (int t = 0; t < kLineMaxSeg; ++t) iv[t] = t < S ? __ldg(inv + (size_t)t * a.nr) : 0.0f;
+    }
+    __syncthreads();
+    float sr = 0.0f;
+    if (act) {
+#pragma unroll
+        for (int t = 0; t < kLineMaxSeg; ++t)
+            if (t < S) sr = fmaf(iv[t], s_r[t][lane], sr);
+        s_s[sg][lane] = sr;
+    }
+    __syncthreads();
+    if (!act) return;
+    const float sl = s_s[sg > 0 ? sg - 1 : S - 1][lane];
+    float2 es;
+    ld(c0 + le * plane, i0 + le * lp, es);
+    for (int lc = l0; lc < le; lc += U) {
+        float2 e[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (lc + u < le) {
+                ld(c0 + (lc + u) * plane, i0 + (lc + u) * lp, e[u]);
+                mm[u] = __ldg(L.vl + i0 + (lc + u) * lp);
+                ww[u] = __ldg(L.vr + i0 + (lc + u) * lp);
+            }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (lc + u < le)
+                out(c0 + (lc + u) * plane, i0 + (lc + u) * lp,
+                    fmaf(ww[u], sr, fmaf(mm[u], sl, yv(lc + u))), e[u]);
+    }
+    out(c0 + le * plane, i0 + le * lp, sr, es);
 }
 
-__global__ void __launch_bounds__(256) k_cg_residual4(const CgArgs a)
+// the factors of every ring: pivots, separator responses and the inverse of the separators'
+// cyclic tridiagonal Schur complement (FP64 recurrences; once per step)
+__global__ void __launch_bounds__(512) k_line_setup(const LineOp L, const CgArgs a)
 {
-    KSum rz;
-    FLD_QUADS(c)
-    {
-        const float4 ax = apply_flux4(a, a.x, c), b = ld4(a.b + c), idg = ld4(a.idg + c);
-        const float4 r = make_float4(b.x - ax.x, b.y - ax.y, b.z - ax.z, b.w - ax.w);
-        const float4 z = make_float4(r.x * idg.x, r.y * idg.y, r.z * idg.z, r.w * idg.w);
-        st4(a.r + c, r);
-        st4(a.d + c, make_float4(0.0f, 0.0f, 0.0f, 0.0f));
-        st4(a.p + c, z);
-        rz.add(r.x * z.x);
-        rz.add(r.y * z.y);
-        rz.add(r.z * z.z);
-        rz.add(r.w * z.w);
+    __shared__ double s_d[kLineMaxSeg][32], s_e[kLineMaxSeg][32], s_v[kLineMaxSeg][32];
+    const int lane = threadIdx.x & 31, sg = threadIdx.x >> 5, S = L.seg;
+    const int kt = (a.nr + 31) / 32;
+    const int jl = blockIdx.x / kt, k = (blockIdx.x - jl * kt) * 32 + lane;
+    const int j = jl < L.j0 ? jl : jl - L.j0 + L.j1;
+    const bool act = k < a.nr;
+    const int l0 = sg * a.nph / S, l1 = (sg + 1) * a.nph / S;
+    const unsigned n = (unsigned)a.n, plane = (unsigned)a.nr * (unsigned)a.nth;
+    const unsigned lp = (unsigned)L.nl * (unsigned)a.nr, i0 = (unsigned)jl * a.nr + k;
+    auto cell = [&](int l) { return (unsigned)l * plane + (unsigned)j * a.nr + k; };
+    auto wph = [&](int l) { return (double)__ldg(a.w + 2 * n + cell(l)); };
+    auto diag = [&](int l) {
+        const unsigned c = cell(l);
+        double d = (double)__ldg(a.s + c) + wph(l) + wph(l > 0 ? l - 1 : a.nph - 1);
+        if (k + 1 < a.nr) d += (double)__ldg(a.w + c);
+        if (k > 0) d += (double)__ldg(a.w + c - 1);
+        if (j + 1 < a.nth) d += (double)__ldg(a.w + n + c);
+        if (j > 0) d += (double)__ldg(a.w + n + c - a.nr);
+        return d;
+    };
+    double m = 0.0, v = 0.0, w0 = 0.0, dsep = 0.0;
+    if (act) {
+        // interior pivots, and the forward part of the left separator's response
+        const double wl = wph(l0 > 0 ? l0 - 1 : a.nph - 1);  // left separator to the first interior cell
+#pragma unroll 4
+        for (int l = l0; l < l1 - 1; ++l) {
+            const double piv = diag(l) - w0 * w0 * m;
+            m = piv > 0.0 ? 1.0 / piv : 0.0;
+            v = (l == l0 ? wl : w0 * v) * m;
+            w0 = wph(l);
+            L.m[i0 + l * lp] = (float)m;
+            L.vl[i0 + l * lp] = (float)v;
+        }
+        // backward; w0 couples the last interior cell and the separator
+        double u = w0 * m;  // the right separator's response
+        const double vlast = v, ulast = u;
+        L.vr[i0 + (l1 - 2) * lp] = (float)u;
+#pragma unroll 4
+        for (int l = l1 - 3; l >= l0; --l) {
+            const double g = wph(l) * (double)L.m[i0 + l * lp];
+            u *= g;
+            v = fma(g, v, (double)L.vl[i0 + l * lp]);
+            L.vl[i0 + l * lp] = (float)v;
+            L.vr[i0 + l * lp] = (float)u;
+        }
+        // Schur complement: own diagonal here, the left neighbour's share through s_v
+        dsep = diag(l1 - 1) - w0 * ulast;
+        s_v[sg][lane] = wl * v;      // first cell's response to the left separator, times its coupling
+        s_e[sg][lane] = w0 * vlast;  // coupling of separators sg - 1 and sg
+    }
+    __syncthreads();
+    if (act) s_d[sg][lane] = dsep - s_v[sg + 1 < S ? sg + 1 : 0][lane];
+    __syncthreads();
+    if (!act) return;
+    // column sg of the inverse: cyclic tridiagonal solve (Thomas, with Sherman and Morrison's
+    // rank-one correction for the wrap), couplings e[t] between separators t - 1 and t
+    double cp[kLineMaxSeg], y[kLineMaxSeg], q[kLineMaxSeg];
+    const double wrap = s_e[0][lane], gam = -s_d[0][lane];
+    double den = 0.0;
+    for (int t = 0; t < S; ++t) {
+        double d = s_d[t][lane];
+        if (t == 0) d -= gam;
+        if (t == S - 1) d -= wrap * wrap / gam;
+        const double e = t > 0 ? s_e[t][lane] : 0.0;
+        den = 1.0 / (t > 0 ? d - e * cp[t - 1] : d);
+        cp[t] = t + 1 < S ? s_e[t + 1][lane] * den : 0.0;
+        y[t] = ((t == sg ? 1.0 : 0.0) + (t > 0 ? e * y[t - 1] : 0.0)) * den;
+        q[t] = ((t == 0 ? gam : t == S - 1 ? -wrap : 0.0) + (t > 0 ? e * q[t - 1] : 0.0)) * den;
+    }
+    for (int t = S - 2; t >= 0; --t) {
+        y[t] += cp[t] * y[t + 1];
+        q[t] += cp[t] * q[t + 1];
+    }
+    const double f = (y[0] - wrap * y[S - 1] / gam) / (1.0 + q[0] - wrap * q[S - 1] / gam);
+    for (int t = 0; t < S; ++t) L.inv[(((size_t)jl * S + t) * S + sg) * a.nr + k] = (float)(y[t] - f * q[t]);
+}
+
+// --- the iteration ----------------------------------------------------------------
+// the scalars of a new solve (bad: the input was invalid, nothing runs)
+__global__ void k_it_start(double *sc, const unsigned *bad, unsigned *count, double tol, double max_iter)
+{
+    *count = 0u;
+    for (int i = 0; i < kNScal; ++i) sc[i] = 0.0;
+    sc[kFlush] = 2.0;
+    sc[kCorr] = INFINITY;
+    sc[kTol] = tol;
+    sc[kMaxIter] = max_iter;
+    sc[kDone] = *bad ? 1.0 : 0.0;
+}
+
+// a group's end: x += d (and the step still to go into d); kCorr = max |d| / |x|, capped at
+// 1e30 (infinite if an x is not finite). pc: the current direction
+template <bool Q>
+__global__ void __launch_bounds__(256) k_it_flush(const CgArgs a, const float *pc)
+{
+    double *sc = a.scal;
+    if (sc[kDone] != 0.0 || sc[kFlush] != 1.0) return;
+    const bool pend = sc[kPend] != 0.0, live = sc[kDLive] != 0.0;
+    const float alpha = (float)sc[kAlpha];
+    KMax m;
+    auto one = [&](float x, float d) {
+        if (!isfinite(x)) m.s = INFINITY;
+        else if (d != 0.0f) m.s = fmaxf(m.s, fminf(fabsf(d) / fmaxf(fabsf(x), 1e-37f), 1e30f));
+    };
+    constexpr unsigned W = Q ? 4u : 1u;
+    for (unsigned c = W * (blockIdx.x * blockDim.x + threadIdx.x); c < (unsigned)a.n; c += W * gridDim.x * blockDim.x) {
+        if constexpr (Q) {
+            float4 d = make_float4(0.0f, 0.0f, 0.0f, 0.0f), x = ld4(a.x + c);
+            if (live) d = ld4(a.d + c);
+            if (pend) {
+                const float4 p = ld4(pc + c);
+                d = make_float4(fmaf(alpha, p.x, d.x), fmaf(alpha, p.y, d.y), fmaf(alpha, p.z, d.z), fmaf(alpha, p.w, d.w));
+            }
+            x = make_float4(x.x + d.x, x.y + d.y, x.z + d.z, x.w + d.w);
+            st4(a.x + c, x);
+            one(x.x, d.x);
+            one(x.y, d.y);
+            one(x.z, d.z);
+            one(x.w, d.w);
+        } else {
+            float d = live ? a.d[c] : 0.0f;
+            if (pend) d = fmaf(alpha, pc[c], d);
+            const float x = a.x[c] + d;
+            a.x[c] = x;
+            one(x, d);
+        }
     }
     double tot;
-    if (grid_reduce<false>(a, rz.value(), &tot)) {
-        a.scal[kRz] = tot;
-        a.scal[kRz0] = tot;
-        a.scal[kDone] = tot > 0.0 ? 0.0 : 1.0;
+    if (grid_reduce(a, m, &tot)) {
+        sc[kCorr] = tot;
+        sc[kPasses] += 1.0;
+        sc[kPend] = 0.0;
+        sc[kDLive] = 0.0;
+        if (tot < sc[kTol] || isinf(tot) || sc[kLast] != 0.0) sc[kDone] = 1.0;
     }
 }
 
-__global__ void __launch_bounds__(256) k_cg_apply4(const CgArgs a)
+constexpr float kMgOmega = 0.8f;
+
+// r -= alpha q, or r = b - A x after a flush; in the line rows (the first blocks) also
+// x0 = omega T^-1 r, the V-cycle's first smoothing step there
+template <bool Q, bool SM>
+__global__ void __launch_bounds__(512, 2) k_it_residual(const CgArgs a, const LineOp L)
 {
-    if (a.scal[kDone] != 0.0) return;
+    const double *sc = a.scal;
+    if (sc[kDone] != 0.0) return;
+    const bool fresh = sc[kFlush] != 0.0;
+    const float alpha = (float)sc[kAlpha];
+    const unsigned n = (unsigned)a.n;
+    auto xv = [&](unsigned i, int, int, int) { return a.x[i]; };
+    if ((int)blockIdx.x < L.blocks) {
+        if (fresh) {  // the block's rings first, then solved from r
+            const int kt = (a.nr + 31) / 32, jl = blockIdx.x / kt, k = (blockIdx.x - jl * kt) * 32 + (threadIdx.x & 31);
+            const int j = jl < L.j0 ? jl : jl - L.j0 + L.j1;
+            if (k < a.nr) {
+#pragma unroll 1
+                for (int l = threadIdx.x >> 5; l < a.nph; l += blockDim.x >> 5) {
+                    const unsigned c = ((unsigned)l * a.nth + j) * a.nr + k;
+                    a.r[c] = a.b[c] - flux_one(a.nr, a.nth, a.nph, n, a.s, a.w, xv, c, k, j, l, a.x[c]);
+                }
+            }
+            __syncthreads();
+        }
+        line_solve<SM>(L, a, L.x, [&](unsigned c, unsigned) { return fresh ? a.r[c] : fmaf(-alpha, a.q[c], a.r[c]); },
+                       [&](unsigned c, float r) { if (!fresh) a.r[c] = r; }, [](unsigned, unsigned, float2 &) {},
+                       [&](unsigned, unsigned i, float x, float2) { L.x[i] = kMgOmega * x; });
+        return;
+    }
+    if (Q && !fresh) {  // four quads in flight per thread: the line role's registers leave few warps
+        const unsigned step = 4u * (gridDim.x - L.blocks) * blockDim.x;
+        for (unsigned c0 = 4u * ((blockIdx.x - L.blocks) * blockDim.x + threadIdx.x); c0 < n; c0 += 4u * step) {
+            float4 q[4], r[4];
+            bool on[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned c = c0 + u * step;
+                int k, j, l;
+                cell_ijk(c, a.nr, a.nth, a.div_nr, a.div_nth, k, j, l);
+                on[u] = c < n && !L.has(j);
+                if (on[u]) {
+                    q[u] = ld4(a.q + c);
+                    r[u] = ld4(a.r + c);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (on[u])
+                    st4(a.r + c0 + u * step, make_float4(fmaf(-alpha, q[u].x, r[u].x), fmaf(-alpha, q[u].y, r[u].y),
+                                                         fmaf(-alpha, q[u].z, r[u].z), fmaf(-alpha, q[u].w, r[u].w)));
+        }
+        return;
+    }
+    for_cells<Q>(a, L.blocks, [&](unsigned c, int k, int j, int l) {
+        if (L.has(j)) return;
+        if constexpr (Q) {
+            auto xr = [&](unsigned i, int, int, int) { return ld4(a.x + i); };
+            const float4 ax = flux_quad(a.nr, a.nth, a.nph, n, a.s, a.w, xr, xv, c, k, j, l, ld4(a.x + c));
+            const float4 b = ld4(a.b + c);
+            st4(a.r + c, make_float4(b.x - ax.x, b.y - ax.y, b.z - ax.z, b.w - ax.w));
+        } else {
+            a.r[c] = fresh ? a.b[c] - flux_one(a.nr, a.nth, a.nph, n, a.s, a.w, xv, c, k, j, l, a.x[c])
+                           : fmaf(-alpha, a.q[c], a.r[c]);
+        }
+    });
+}
+
+// d += alpha p, p = z + beta p (pc -> pn), q = A p and alpha = r.z / p.q, the new p formed at the
+// stencil's points from z and the old one
+template <bool Q>
+__global__ void __launch_bounds__(256, Q ? 4 : 6) k_it_apply(const CgArgs a, const float *pc, float *pn)
+{
+    double *sc = a.scal;
+    if (sc[kDone] != 0.0) return;
+    const float alpha = (float)sc[kAlpha], beta = (float)sc[kBeta];
+    const bool pend = sc[kPend] != 0.0, live = sc[kDLive] != 0.0, carry = beta != 0.0f;
+    const float *z = a.z;
+    const unsigned n = (unsigned)a.n;
     KSum pq;
-    FLD_QUADS(c)
-    {
-        const float4 q = apply_flux4(a, a.p, c), p = ld4(a.p + c);
-        st4(a.q + c, q);
-        pq.add(p.x * q.x);
-        pq.add(p.y * q.y);
-        pq.add(p.z * q.z);
-        pq.add(p.w * q.w);
-    }
+    auto p1 = [&](unsigned i, int, int, int) { return carry ? fmaf(beta, pc[i], z[i]) : z[i]; };
+    for_cells<Q>(a, 0u, [&](unsigned c, int k, int j, int l) {
+        if constexpr (Q) {
+            auto pr = [&](unsigned i, int, int, int) {
+                const float4 zz = ld4(z + i);
+                if (!carry) return zz;
+                const float4 p = ld4(pc + i);
+                return make_float4(fmaf(beta, p.x, zz.x), fmaf(beta, p.y, zz.y), fmaf(beta, p.z, zz.z),
+                                   fmaf(beta, p.w, zz.w));
+            };
+            const float4 p = pr(c, k, j, l);
+            const float4 q = flux_quad(a.nr, a.nth, a.nph, n, a.s, a.w, pr, p1, c, k, j, l, p);
+            if (pend) {
+                const float4 o = ld4(pc + c);
+                float4 d = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (live) d = ld4(a.d + c);
+                st4(a.d + c, make_float4(fmaf(alpha, o.x, d.x), fmaf(alpha, o.y, d.y), fmaf(alpha, o.z, d.z),
+                                         fmaf(alpha, o.w, d.w)));
+            }
+            st4(pn + c, p);
+            st4(a.q + c, q);
+            pq.add(p.x * q.x);
+            pq.add(p.y * q.y);
+            pq.add(p.z * q.z);
+            pq.add(p.w * q.w);
+        } else {
+            const float p = p1(c, k, j, l);
+            const float q = flux_one(a.nr, a.nth, a.nph, n, a.s, a.w, p1, c, k, j, l, p);
+            if (pend) a.d[c] = fmaf(alpha, pc[c], live ? a.d[c] : 0.0f);
+            pn[c] = p;
+            a.q[c] = q;
+            pq.add(p * q);
+        }
+    });
     double tot;
-    if (grid_reduce<false>(a, pq.value(), &tot)) {
-        a.scal[kAlpha] = tot > 0.0 ? a.scal[kRz] / tot : 0.0;
-        if (!(tot > 0.0)) a.scal[kDone] = 1.0;
+    if (grid_reduce(a, pq, &tot)) {
+        if (pend) sc[kDLive] = 1.0;
+        sc[kAlpha] = tot > 0.0 ? sc[kRz] / tot : 0.0;
+        sc[kPend] = sc[kLast] != 0.0 ? 0.0 : 1.0;  // past max_iter the new step is not taken
+        if (!(tot > 0.0)) sc[kFlush] = 1.0;
     }
 }
 
-__global__ void __launch_bounds__(256) k_cg_update4(const CgArgs a)
+// r.z closes a step: beta, the iteration count, and whether the group ends. A group's first
+// r.z is of the true residual: where that exceeds the recurrence's the directions restart.
+__device__ __forceinline__ void close_step(const CgArgs &a, double tot)
+{
+    double *sc = a.scal;
+    const double flush = sc[kFlush], old = sc[kRz];
+    if (flush == 2.0) {  // the first residual
+        sc[kBeta] = 0.0;
+        sc[kRz0] = tot;
+        if (!(tot > 0.0)) {  // x solves the system as it is (or it is not finite)
+            sc[kCorr] = tot == 0.0 ? 0.0 : INFINITY;
+            sc[kPasses] = 1.0;
+            sc[kDone] = 1.0;
+        }
+        sc[kFlush] = 0.0;
+    } else {
+        double beta = old > 0.0 ? tot / old : 0.0;
+        if (flush == 1.0) {
+            sc[kRz0] = tot;
+            if (tot > old) beta = 0.0;
+        }
+        sc[kBeta] = beta;
+        sc[kIters] += 1.0;
+        const bool last = sc[kIters] >= sc[kMaxIter];
+        sc[kLast] = last ? 1.0 : 0.0;
+        sc[kFlush] = last || !(tot > kGroupDrop * kGroupDrop * sc[kRz0]) ? 1.0 : 0.0;
+    }
+    sc[kRz] = tot;
+}
+
+// z = r / dg: the preconditioner of grids too small for levels
+__global__ void __launch_bounds__(256) k_it_jacobi(const CgArgs a)
 {
     if (a.scal[kDone] != 0.0) return;
-    const float alpha = (float)a.scal[kAlpha];
     KSum rz;
-    FLD_QUADS(c)
-    {
-        const float4 p = ld4(a.p + c), q = ld4(a.q + c), idg = ld4(a.idg + c);
-        float4 d = ld4(a.d + c), r = ld4(a.r + c);
-        d = make_float4(fmaf(alpha, p.x, d.x), fmaf(alpha, p.y, d.y), fmaf(alpha, p.z, d.z), fmaf(alpha, p.w, d.w));
-        r = make_float4(fmaf(-alpha, q.x, r.x), fmaf(-alpha, q.y, r.y), fmaf(-alpha, q.z, r.z),
-                        fmaf(-alpha, q.w, r.w));
-        st4(a.d + c, d);
-        st4(a.r + c, r);
-        rz.add(r.x * (r.x * idg.x));
-        rz.add(r.y * (r.y * idg.y));
-        rz.add(r.z * (r.z * idg.z));
-        rz.add(r.w * (r.w * idg.w));
-    }
+    for_cells<false>(a, 0u, [&](unsigned c, int, int, int) {
+        const float r = a.r[c], z = r * a.idg[c];
+        a.z[c] = z;
+        rz.add(r * z);
+    });
     double tot;
-    if (grid_reduce<false>(a, rz.value(), &tot)) {
-        a.scal[kBeta] = a.scal[kRz] > 0.0 ? tot / a.scal[kRz] : 0.0;
-        a.scal[kRz] = tot;
-        a.scal[kIters] += 1.0;
-        if (!(tot > kInnerDrop * kInnerDrop * a.scal[kRz0])) a.scal[kDone] = 1.0;
-    }
+    if (grid_reduce(a, rz, &tot)) close_step(a, tot);
 }
 
-__global__ void __launch_bounds__(256) k_cg_direction4(const CgArgs a)
+// the loop's condition, at the end of its body (with a limit of its own: whatever the scalars
+// say, the loop ends)
+__global__ void k_it_loop(double *sc, cudaGraphConditionalHandle h)
 {
-    if (a.scal[kDone] != 0.0) return;
-    const float beta = (float)a.scal[kBeta];
-    FLD_QUADS(c)
-    {
-        const float4 r = ld4(a.r + c), idg = ld4(a.idg + c), p = ld4(a.p + c);
-        st4(a.p + c, make_float4(fmaf(beta, p.x, r.x * idg.x), fmaf(beta, p.y, r.y * idg.y),
-                                 fmaf(beta, p.z, r.z * idg.z), fmaf(beta, p.w, r.w * idg.w)));
-    }
+    sc[kLoops] += 1.0;
+    cudaGraphSetConditional(h, sc[kDone] == 0.0 && sc[kLoops] * kUnroll < sc[kMaxIter] + 4.0 * kUnroll ? 1u : 0u);
 }
 
-#undef FLD_QUADS
+// the step's result, unless the input was invalid
+__global__ void __launch_bounds__(256) k_it_store(const float *x, float *out, long long n, const unsigned *bad)
+{
+    if (*bad) return;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x)
+        out[c] = x[c];
+}
+
 // --- aggregation multigrid preconditioner ---------------------------------------
 // Levels coarsen by 2 in every direction longer than one cell. The coarse operator
 // is the Galerkin product with piecewise-constant prolongation: the storage terms
@@ -611,11 +983,13 @@ __global__ void __launch_bounds__(256) k_cg_direction4(const CgArgs a)
 // every level keeps the flux form. One V-cycle per CG iteration: a damped Jacobi
 // step from zero, the restricted residual, the coarser levels, the prolonged
 // correction and one more Jacobi step (symmetric, so CG keeps its guarantees);
-// 16 Jacobi sweeps on the coarsest level (<= 1024 cells, one CTA). The fine-level
-// intermediates are formed on the fly at the stencil's points, never stored.
-constexpr float kMgOmega = 0.8f;
-constexpr int kMgCoarseSweeps = 16;
+// kMgCoarseSweeps Jacobi sweeps on the coarsest level (8 against 16: 25 / 33 iterations against
+// 24 / 33 in the CPU emulation). The intermediates are formed on the fly at the stencil's
+// points, never stored. The levels of at most kTailCells cells run in one CTA (k_mg_tail).
+constexpr int kMgCoarseSweeps = 8;
 constexpr unsigned kMgCoarsest = 512;  // coarsen while a level has more cells
+constexpr unsigned kTailCells = 2048;
+constexpr int kTailLevels = 8;
 
 struct MgLevel {
     int nr, nth, nph;
@@ -636,27 +1010,10 @@ struct HalfOp {
 struct MgPair {
     MgLevel f, c;    // fine and coarse level
     int sr, st, sp;  // log2 of the aggregation factors (0 or 1)
-    CgArgs cg;       // scalars and reduction scratch (the finest pair's up kernel)
+    CgArgs cg;       // scalars and reduction scratch
     HalfOp h;        // the finest level's BF16 operator (finest pair, four-cell kernels)
+    LineOp ln;       // the finest level's phi lines (finest pair)
 };
-
-template <class V>
-__device__ __forceinline__ float apply_lv(const MgLevel &L, const V &v, unsigned c, int k, int j, int l, float vc)
-{
-    const unsigned n = L.n, plane = (unsigned)L.nr * (unsigned)L.nth;
-    float acc = L.s[c] * vc;
-    if (k + 1 < L.nr) acc = fmaf(L.w[c], vc - v(c + 1), acc);
-    if (k > 0) acc = fmaf(L.w[c - 1], vc - v(c - 1), acc);
-    if (j + 1 < L.nth) acc = fmaf(L.w[n + c], vc - v(c + L.nr), acc);
-    if (j > 0) acc = fmaf(L.w[n + c - L.nr], vc - v(c - L.nr), acc);
-    if (L.nph > 1) {
-        const unsigned cb = l + 1 < L.nph ? c + plane : c - (unsigned)l * plane;
-        const unsigned ca = l > 0 ? c - plane : c + (unsigned)(L.nph - 1) * plane;
-        acc = fmaf(L.w[2 * n + c], vc - v(cb), acc);
-        acc = fmaf(L.w[2 * n + ca], vc - v(ca), acc);
-    }
-    return acc;
-}
 
 #define MG_LOOP(i, N) for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < (N); i += gridDim.x * blockDim.x)
 
@@ -713,327 +1070,344 @@ __global__ void __launch_bounds__(256) k_mg_diag(const MgLevel L)
 }
 
 // coarse right-hand side: the aggregate's sum of the fine residuals after the
-// first Jacobi step x0 = omega b / dg (the 2 x 2 x 2 loop unrolled, so that the
-// loads of all eight fine cells are in flight together)
+// first smoothing step x0 (omega b / dg; the stored line solution in line rows, LINES). Eight
+// threads per coarse cell, one fine cell each, summed by shuffles: the coarse levels have few
+// cells and a thread that walked all eight was a chain of loads (6.5 us on 2048 coarse cells and
+// 12.6 us on 131072; 3.1 and 4.5 us now).
+template <bool LINES>
 __global__ void __launch_bounds__(256) k_mg_down(const MgPair P)
 {
     if (P.cg.scal[kDone] != 0.0) return;
     const MgLevel &F = P.f, &C = P.c;
     const float *idg = F.idg, *b = F.b;
-    auto x0 = [=](unsigned i) { return kMgOmega * idg[i] * b[i]; };
-    MG_LOOP(cc, C.n)
-    {
-        int K, J, L;
-        cell_ijk(cc, C.nr, C.nth, C.dnr, C.dnth, K, J, L);
-        float sum = 0.0f;
-#pragma unroll
-        for (int dl = 0; dl < 2; ++dl)
-#pragma unroll
-            for (int dj = 0; dj < 2; ++dj)
-#pragma unroll
-                for (int dk = 0; dk < 2; ++dk) {
-                    const int l = (L << P.sp) + dl, j = (J << P.st) + dj, k = (K << P.sr) + dk;
-                    const bool in = (dl <= P.sp && l < F.nph) && (dj <= P.st && j < F.nth) && (dk <= P.sr && k < F.nr);
-                    if (in) {
-                        const unsigned c = ((unsigned)l * F.nth + j) * F.nr + k;
-                        sum += b[c] - apply_lv(F, x0, c, k, j, l, x0(c));
-                    }
-                }
-        C.b[cc] = sum;
-    }
-}
-
-// the coarsest level (n <= 1024): kMgCoarseSweeps damped Jacobi sweeps from zero,
-// the level's operator staged in shared memory once
-__global__ void __launch_bounds__(256) k_mg_coarsest(const MgLevel L, const double *scal)
-{
-    if (scal[kDone] != 0.0) return;
-    __shared__ float xs[1024], ss[1024], wr[1024], wt[1024], wp[1024], id[1024], bs[1024];
-    const unsigned n = L.n;
-    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
-        ss[i] = L.s[i];
-        wr[i] = L.w[i];
-        wt[i] = L.w[n + i];
-        wp[i] = L.w[2 * n + i];
-        id[i] = L.idg[i];
-        bs[i] = L.b[i];
-        xs[i] = kMgOmega * L.idg[i] * L.b[i];
-    }
-    __syncthreads();
-    const unsigned plane = (unsigned)L.nr * (unsigned)L.nth;
-    for (int sweep = 1; sweep < kMgCoarseSweeps; ++sweep) {
-        float nv[4];
-        int m = 0;
-        for (unsigned i = threadIdx.x; i < n; i += blockDim.x, ++m) {
-            int k, j, l;
-            cell_ijk(i, L.nr, L.nth, L.dnr, L.dnth, k, j, l);
-            const float xi = xs[i];
-            float acc = ss[i] * xi;
-            if (k + 1 < L.nr) acc = fmaf(wr[i], xi - xs[i + 1], acc);
-            if (k > 0) acc = fmaf(wr[i - 1], xi - xs[i - 1], acc);
-            if (j + 1 < L.nth) acc = fmaf(wt[i], xi - xs[i + L.nr], acc);
-            if (j > 0) acc = fmaf(wt[i - L.nr], xi - xs[i - L.nr], acc);
-            if (L.nph > 1) {
-                const unsigned cb = l + 1 < L.nph ? i + plane : i - (unsigned)l * plane;
-                const unsigned ca = l > 0 ? i - plane : i + (unsigned)(L.nph - 1) * plane;
-                acc = fmaf(wp[i], xi - xs[cb], acc);
-                acc = fmaf(wp[ca], xi - xs[ca], acc);
-            }
-            nv[m] = fmaf(kMgOmega * id[i], bs[i] - acc, xi);
+    auto x0 = [&](unsigned i, int k, int j, int l) {
+        if constexpr (LINES) {
+            if (P.ln.has(j)) return P.ln.x[P.ln.at(F.nr, k, j, l)];
         }
-        __syncthreads();
-        m = 0;
-        for (unsigned i = threadIdx.x; i < n; i += blockDim.x, ++m) xs[i] = nv[m];
-        __syncthreads();
+        return kMgOmega * idg[i] * b[i];
+    };
+    const int sub = threadIdx.x & 7, dk = sub & 1, dj = (sub >> 1) & 1, dl = sub >> 2;
+    const unsigned step = (gridDim.x * blockDim.x) >> 3;
+    // (every thread of a warp walks the same number of rounds: the shuffles need them all)
+    for (unsigned c0 = (blockIdx.x * blockDim.x) >> 3; c0 < C.n; c0 += step) {
+        const unsigned cc = c0 + (threadIdx.x >> 3);
+        float res = 0.0f;
+        if (cc < C.n) {
+            int K, J, L;
+            cell_ijk(cc, C.nr, C.nth, C.dnr, C.dnth, K, J, L);
+            const int l = (L << P.sp) + dl, j = (J << P.st) + dj, k = (K << P.sr) + dk;
+            if ((dl <= P.sp && l < F.nph) && (dj <= P.st && j < F.nth) && (dk <= P.sr && k < F.nr)) {
+                const unsigned c = ((unsigned)l * F.nth + j) * F.nr + k;
+                res = b[c] - flux_one(F.nr, F.nth, F.nph, F.n, F.s, F.w, x0, c, k, j, l, x0(c, k, j, l));
+            }
+        }
+        for (int o = 1; o < 8; o <<= 1) res += __shfl_xor_sync(0xffffffffu, res, o);
+        if (sub == 0 && cc < C.n) C.b[cc] = res;
     }
-    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) L.x[i] = xs[i];
 }
 
-// prolonged correction and the second Jacobi step: x = x1 + omega (b - A x1) / dg,
-// x1 = omega b / dg + x_coarse[aggregate]. On the finest pair (top) x is z = M^-1 r
-// and its r.z closes the CG step: init sets rz0 and beta = 0, otherwise beta, rz,
-// the iteration count and the convergence flag.
-__global__ void __launch_bounds__(256) k_mg_up(const MgPair P, int top, int init)
+// prolonged correction and the second Jacobi step of a coarse level: x = x1 + omega (b - A x1)
+// / dg, x1 = omega b / dg + x_coarse[aggregate]
+__global__ void __launch_bounds__(256) k_mg_up(const MgPair P)
 {
     if (P.cg.scal[kDone] != 0.0) return;
     const MgLevel &F = P.f, &C = P.c;
-    const unsigned n = F.n, plane = (unsigned)F.nr * (unsigned)F.nth;
     const float *idg = F.idg, *b = F.b, *xc = C.x;
     auto x1 = [&](unsigned i, int k, int j, int l) {
         return fmaf(kMgOmega * idg[i], b[i], xc[((unsigned)(l >> P.sp) * C.nth + (j >> P.st)) * C.nr + (k >> P.sr)]);
     };
-    KSum rz;
-    MG_LOOP(c, n)
+    MG_LOOP(c, F.n)
     {
         int k, j, l;
         cell_ijk(c, F.nr, F.nth, F.dnr, F.dnth, k, j, l);
         const float vc = x1(c, k, j, l);
-        float acc = F.s[c] * vc;
-        if (k + 1 < F.nr) acc = fmaf(F.w[c], vc - x1(c + 1, k + 1, j, l), acc);
-        if (k > 0) acc = fmaf(F.w[c - 1], vc - x1(c - 1, k - 1, j, l), acc);
-        if (j + 1 < F.nth) acc = fmaf(F.w[n + c], vc - x1(c + F.nr, k, j + 1, l), acc);
-        if (j > 0) acc = fmaf(F.w[n + c - F.nr], vc - x1(c - F.nr, k, j - 1, l), acc);
-        if (F.nph > 1) {
-            const int lb = l + 1 < F.nph ? l + 1 : 0, la = l > 0 ? l - 1 : F.nph - 1;
-            const unsigned cb = c + (unsigned)(lb - l) * plane, ca = c + (unsigned)(la - l) * plane;
-            acc = fmaf(F.w[2 * n + c], vc - x1(cb, k, j, lb), acc);
-            acc = fmaf(F.w[2 * n + ca], vc - x1(ca, k, j, la), acc);
-        }
-        const float xv = fmaf(kMgOmega * idg[c], b[c] - acc, vc);
-        F.x[c] = xv;
-        if (top) rz.add(b[c] * xv);
-    }
-    if (!top) return;
-    double tot;
-    if (grid_reduce<false>(P.cg, rz.value(), &tot)) {
-        double *sc = P.cg.scal;
-        if (init) {
-            sc[kRz] = tot;
-            sc[kRz0] = tot;
-            sc[kBeta] = 0.0;
-            sc[kDone] = tot > 0.0 ? 0.0 : 1.0;
-        } else {
-            sc[kBeta] = sc[kRz] > 0.0 ? tot / sc[kRz] : 0.0;
-            sc[kRz] = tot;
-            sc[kIters] += 1.0;
-            if (!(tot > kInnerDropMg * kInnerDropMg * sc[kRz0])) sc[kDone] = 1.0;
-        }
+        F.x[c] = fmaf(kMgOmega * idg[c], b[c] - flux_one(F.nr, F.nth, F.nph, F.n, F.s, F.w, x1, c, k, j, l, vc), vc);
     }
 }
 
-// Finest level with nr % 4 == 0: four cells of one ray per thread; the BF16 operator
-// in 64-bit loads. A_h v on the quad c .. c+3 at (k .. k+3, j, l), the value of the quad
-// at the same k of row (j', l') from vrow(c0, k, j', l') and of one cell from
-// vone(i, k', j, l).
-__device__ __forceinline__ float4 ldh4(const unsigned short *p)
+// The levels of at most kTailCells cells in one CTA, everything in shared memory: one launch in
+// place of two per level and the coarsest solve, whose few cells are all launch latency.
+struct MgTail {
+    MgLevel lv[kTailLevels];
+    int n_lv;
+    const double *scal;
+};
+
+size_t tail_smem(const MgTail &t)
 {
-    const uint2 u = *reinterpret_cast<const uint2 *>(p);
-    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
-                       __uint_as_float(u.y & 0xffff0000u));
+    size_t n = 0;
+    for (int i = 0; i < t.n_lv; ++i) n += t.lv[i].n;
+    return sizeof(float) * 8 * n;
 }
-__device__ __forceinline__ float ldh1(const unsigned short *p) { return __uint_as_float((unsigned)*p << 16); }
 
-template <class VR, class V1>
-__device__ __forceinline__ float4 apply_quad(const MgLevel &F, const HalfOp &h, const VR &vrow, const V1 &vone,
-                                             unsigned c, int k, int j, int l, float4 vc)
+__global__ void __launch_bounds__(1024) k_mg_tail(const __grid_constant__ MgTail T)
 {
-    const unsigned n = F.n, plane = (unsigned)F.nr * (unsigned)F.nth;
-    const float4 s = ldh4(h.s + c), wr = ldh4(h.w + c);
-    float4 acc = make_float4(s.x * vc.x, s.y * vc.y, s.z * vc.z, s.w * vc.w);
-    acc.x = fmaf(wr.x, vc.x - vc.y, acc.x);
-    acc.y = fmaf(wr.y, vc.y - vc.z, acc.y);
-    acc.z = fmaf(wr.z, vc.z - vc.w, acc.z);
-    acc.y = fmaf(wr.x, vc.y - vc.x, acc.y);
-    acc.z = fmaf(wr.y, vc.z - vc.y, acc.z);
-    acc.w = fmaf(wr.z, vc.w - vc.z, acc.w);
-    if (k + 4 < F.nr) acc.w = fmaf(wr.w, vc.w - vone(c + 4, k + 4, j, l), acc.w);
-    if (k > 0) acc.x = fmaf(ldh1(h.w + c - 1), vc.x - vone(c - 1, k - 1, j, l), acc.x);
-    auto face4 = [&](float4 w, float4 u) {
-        acc.x = fmaf(w.x, vc.x - u.x, acc.x);
-        acc.y = fmaf(w.y, vc.y - u.y, acc.y);
-        acc.z = fmaf(w.z, vc.z - u.z, acc.z);
-        acc.w = fmaf(w.w, vc.w - u.w, acc.w);
-    };
-    if (j + 1 < F.nth) face4(ldh4(h.w + n + c), vrow(c + F.nr, k, j + 1, l));
-    if (j > 0) face4(ldh4(h.w + n + c - F.nr), vrow(c - F.nr, k, j - 1, l));
-    if (F.nph > 1) {
-        const int lb = l + 1 < F.nph ? l + 1 : 0, la = l > 0 ? l - 1 : F.nph - 1;
-        const unsigned cb = c + (unsigned)(lb - l) * plane, ca = c + (unsigned)(la - l) * plane;
-        face4(ldh4(h.w + 2 * n + c), vrow(cb, k, j, lb));
-        face4(ldh4(h.w + 2 * n + ca), vrow(ca, k, j, la));
+    if (T.scal[kDone] != 0.0) return;
+    extern __shared__ float sm[];
+    // per level: s, w[3], 1/dg, b, x as in memory (one run of 7 n floats over the levels), then
+    // n floats y: residuals
+    unsigned n7 = 0;
+    for (int i = 0; i < T.n_lv; ++i) n7 += 7 * T.lv[i].n;
+    const float *src = T.lv[0].s;
+    for (unsigned c = threadIdx.x; c < n7; c += 8 * blockDim.x) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (c + u * blockDim.x < n7) v[u] = src[c + u * blockDim.x];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (c + u * blockDim.x < n7) sm[c + u * blockDim.x] = v[u];
     }
-    return acc;
+    __syncthreads();
+    float *o = sm, *y = sm + n7;
+    for (int i = 0; i + 1 < T.n_lv; ++i) {  // down
+        const MgLevel &F = T.lv[i], &C = T.lv[i + 1];
+        const float *id = o + 4 * F.n, *b = o + 5 * F.n;
+        auto x0 = [&](unsigned q, int, int, int) { return kMgOmega * id[q] * b[q]; };
+        for (unsigned c = threadIdx.x; c < F.n; c += blockDim.x) {
+            int k, j, l;
+            cell_ijk(c, F.nr, F.nth, F.dnr, F.dnth, k, j, l);
+            y[c] = b[c] - flux_one(F.nr, F.nth, F.nph, F.n, o, o + F.n, x0, c, k, j, l, x0(c, 0, 0, 0));
+        }
+        __syncthreads();
+        o += 7 * F.n;
+        const int sr = F.nr > 1, st = F.nth > 1, sp = F.nph > 1;
+        for (unsigned cc = threadIdx.x; cc < C.n; cc += blockDim.x) {
+            int K, J, L;
+            cell_ijk(cc, C.nr, C.nth, C.dnr, C.dnth, K, J, L);
+            float sum = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int dk = q & 1, dj = (q >> 1) & 1, dl = q >> 2;
+                const int k = (K << sr) + dk, j = (J << st) + dj, l = (L << sp) + dl;
+                if (dk <= sr && k < F.nr && dj <= st && j < F.nth && dl <= sp && l < F.nph)
+                    sum += y[((unsigned)l * F.nth + j) * F.nr + k];
+            }
+            o[5 * C.n + cc] = sum;
+        }
+        __syncthreads();
+    }
+    {  // the coarsest level (at most kMgCoarsest cells, one per thread): damped Jacobi sweeps from
+       // zero, the row of the operator in registers, x and y in turn
+        const MgLevel &L = T.lv[T.n_lv - 1];
+        const unsigned n = L.n, c = threadIdx.x;
+        const unsigned warps = (n + 31) / 32;
+        if (threadIdx.x < 32 * warps) {
+            const bool in = c < n;
+            float *x = o + 6 * n;
+            const float *w = o + n;
+            const unsigned plane = (unsigned)L.nr * (unsigned)L.nth;
+            float wv[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, dia = 0.0f, g = 0.0f, bb = 0.0f, v = 0.0f;
+            unsigned nb[6] = {c, c, c, c, c, c};
+            if (in) {
+                int k, j, l;
+                cell_ijk(c, L.nr, L.nth, L.dnr, L.dnth, k, j, l);
+                if (k + 1 < L.nr) { wv[0] = w[c]; nb[0] = c + 1; }
+                if (k > 0) { wv[1] = w[c - 1]; nb[1] = c - 1; }
+                if (j + 1 < L.nth) { wv[2] = w[n + c]; nb[2] = c + L.nr; }
+                if (j > 0) { wv[3] = w[n + c - L.nr]; nb[3] = c - L.nr; }
+                if (L.nph > 1) {
+                    nb[4] = l + 1 < L.nph ? c + plane : c - (unsigned)l * plane;
+                    nb[5] = l > 0 ? c - plane : c + (unsigned)(L.nph - 1) * plane;
+                    wv[4] = w[2 * n + c];
+                    wv[5] = w[2 * n + nb[5]];
+                }
+                dia = o[c];
+                g = kMgOmega * o[4 * n + c];
+                bb = o[5 * n + c];
+                v = g * bb;
+                x[c] = v;
+            }
+            float *cur = x, *nxt = y;
+            for (int t = 1; t < kMgCoarseSweeps; ++t) {
+                asm volatile("bar.sync 1, %0;" ::"r"(32 * warps) : "memory");
+                if (in) {
+                    float acc = dia * v;
+#pragma unroll
+                    for (int q = 0; q < 6; ++q) acc = fmaf(wv[q], v - cur[nb[q]], acc);
+                    v = fmaf(g, bb - acc, v);
+                    nxt[c] = v;
+                }
+                float *h = cur;
+                cur = nxt;
+                nxt = h;
+            }
+            asm volatile("bar.sync 1, %0;" ::"r"(32 * warps) : "memory");
+            if (in) x[c] = v;
+        }
+        __syncthreads();
+    }
+    for (int i = T.n_lv - 2; i >= 0; --i) {  // up
+        const MgLevel &F = T.lv[i], &C = T.lv[i + 1];
+        const float *xc = o + 6 * C.n;
+        o -= 7 * F.n;
+        const float *id = o + 4 * F.n, *b = o + 5 * F.n;
+        const int sr = F.nr > 1, st = F.nth > 1, sp = F.nph > 1;
+        auto x1 = [&](unsigned q, int k, int j, int l) {
+            return fmaf(kMgOmega * id[q], b[q], xc[((unsigned)(l >> sp) * C.nth + (j >> st)) * C.nr + (k >> sr)]);
+        };
+        float *xo = i == 0 ? T.lv[0].x : o + 6 * F.n;
+        for (unsigned c = threadIdx.x; c < F.n; c += blockDim.x) {
+            int k, j, l;
+            cell_ijk(c, F.nr, F.nth, F.dnr, F.dnth, k, j, l);
+            const float vc = x1(c, k, j, l);
+            xo[c] = fmaf(kMgOmega * id[c], b[c] - flux_one(F.nr, F.nth, F.nph, F.n, o, o + F.n, x1, c, k, j, l, vc), vc);
+        }
+        __syncthreads();
+    }
+    if (T.n_lv == 1)
+        for (unsigned c = threadIdx.x; c < T.lv[0].n; c += blockDim.x) T.lv[0].x[c] = sm[6 * T.lv[0].n + c];
 }
 
-// k_mg_down on the finest level: one thread per pair of coarse cells (K0, K0 + 1)
-// of one coarse row, i.e. the four-cell quads of the fine rows in the aggregate.
-// (Five CTAs per SM: 48 registers and a few bytes of spill measured 1.2 % faster per
-// FLD step than four CTAs at 54 registers; the same for k_mg_up4.)
-__global__ void __launch_bounds__(256, 5) k_mg_down4(const MgPair P)
+// k_mg_down on the finest level with nr % 4 == 0: four threads per pair of coarse cells (K0,
+// K0 + 1) of one coarse row, each a four-cell quad of one of the aggregate's fine rows, summed by
+// shuffles; the BF16 operator in 64-bit loads. (One thread per pair walked the four rows one
+// after the other: 8.9 us on 64x32x64, where 32 CTAs held the level; 4.5 us now, and 46 us on
+// 256x128x256 either way.)
+__global__ void __launch_bounds__(256) k_mg_down4(const MgPair P)
 {
     if (P.cg.scal[kDone] != 0.0) return;
     const MgLevel &F = P.f, &C = P.c;
     const unsigned short *idg = P.h.idg;
     const float *b = F.b;
-    auto vrow = [=](unsigned c0, int, int, int) {
-        const float4 d = ldh4(idg + c0), bb = ld4(b + c0);
+    const LineOp &ln = P.ln;
+    auto vrow = [&](unsigned c0, int k, int j, int l) {
+        if (ln.has(j)) return ld4(ln.x + ln.at(F.nr, k, j, l));
+        const float4 d = ldo4(idg + c0), bb = ld4(b + c0);
         return make_float4(kMgOmega * d.x * bb.x, kMgOmega * d.y * bb.y, kMgOmega * d.z * bb.z, kMgOmega * d.w * bb.w);
     };
-    auto vone = [=](unsigned i, int, int, int) { return kMgOmega * ldh1(idg + i) * b[i]; };
-    const unsigned nq = (unsigned)(F.nr / 4) * (unsigned)C.nth * (unsigned)C.nph;
-    for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < nq; t += gridDim.x * blockDim.x) {
-        const unsigned qr = (unsigned)(F.nr / 4);
-        const unsigned rest = t / qr;
-        const int m = (int)(t - rest * qr);
-        const int J = (int)(rest % (unsigned)C.nth), L = (int)(rest / (unsigned)C.nth);
-        const int k = 4 * m;
+    auto vone = [&](unsigned i, int k, int j, int l) {
+        return ln.has(j) ? ln.x[ln.at(F.nr, k, j, l)] : kMgOmega * ldo1(idg + i) * b[i];
+    };
+    const unsigned qr = (unsigned)(F.nr / 4), nq = qr * (unsigned)C.nth * (unsigned)C.nph;
+    // a warp holds 8 consecutive quads of the four rows: 128 bytes per row
+    const int dj = (threadIdx.x >> 3) & 1, dl = (threadIdx.x >> 4) & 1;
+    const unsigned step = (gridDim.x * blockDim.x) >> 2;
+    for (unsigned t0 = (blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) >> 2; t0 < nq; t0 += step) {
+        const unsigned t = t0 + (threadIdx.x & 7);
         float lo = 0.0f, hi = 0.0f;
-        for (int l = L << P.sp; l < min((L + 1) << P.sp, F.nph); ++l)
-            for (int j = J << P.st; j < min((J + 1) << P.st, F.nth); ++j) {
+        unsigned cc = 0u;
+        if (t < nq) {
+            const unsigned rest = t / qr;
+            const int m = (int)(t - rest * qr);
+            const int J = (int)(rest % (unsigned)C.nth), L = (int)(rest / (unsigned)C.nth);
+            const int k = 4 * m, l = (L << P.sp) + dl, j = (J << P.st) + dj;
+            cc = ((unsigned)L * C.nth + J) * C.nr + 2 * m;
+            if (dl <= P.sp && l < F.nph && dj <= P.st && j < F.nth) {
                 const unsigned c = ((unsigned)l * F.nth + j) * F.nr + k;
                 const float4 vc = vrow(c, k, j, l), bb = ld4(b + c);
-                const float4 ax = apply_quad(F, P.h, vrow, vone, c, k, j, l, vc);
-                lo += (bb.x - ax.x) + (bb.y - ax.y);
-                hi += (bb.z - ax.z) + (bb.w - ax.w);
+                const float4 ax = flux_quad(F.nr, F.nth, F.nph, F.n, P.h.s, P.h.w, vrow, vone, c, k, j, l, vc);
+                lo = (bb.x - ax.x) + (bb.y - ax.y);
+                hi = (bb.z - ax.z) + (bb.w - ax.w);
             }
-        const unsigned cc = ((unsigned)L * C.nth + J) * C.nr + 2 * m;
-        C.b[cc] = lo;
-        C.b[cc + 1] = hi;
+        }
+        for (int o = 8; o < 32; o <<= 1) {
+            lo += __shfl_xor_sync(0xffffffffu, lo, o);
+            hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        }
+        if (t < nq && (threadIdx.x & 24) == 0) *reinterpret_cast<float2 *>(C.b + cc) = make_float2(lo, hi);
     }
 }
 
-// k_mg_up on the finest level (top), four cells per thread
-__global__ void __launch_bounds__(256, 5) k_mg_up4(const MgPair P, int init)
+// The finest level's prolongation and second smoothing step, z = M^-1 r, and r.z, which closes
+// the CG step: as k_mg_up, four cells per thread and the BF16 operator where nr % 4 == 0 (Q). Of
+// the line rows it leaves x1 in z and the residual b - A x1 to k_line_post. (Residual and line
+// solve in blocks of their own beside the streaming ones: 140 us on 256x128x256 against 44 + 22.)
+template <bool Q>
+__global__ void __launch_bounds__(256, Q ? 5 : 6) k_mg_up0(const MgPair P)
 {
     if (P.cg.scal[kDone] != 0.0) return;
     const MgLevel &F = P.f, &C = P.c;
-    const unsigned short *idg = P.h.idg;
+    using T = typename std::conditional<Q, unsigned short, float>::type;
+    const T *os, *ow, *idg;
+    if constexpr (Q) {
+        os = P.h.s;
+        ow = P.h.w;
+        idg = P.h.idg;
+    } else {
+        os = F.s;
+        ow = F.w;
+        idg = F.idg;
+    }
     const float *b = F.b, *xc = C.x;
-    const int st = P.st, sp = P.sp, cnr = C.nr, cnth = C.nth;
+    const int sr = P.sr, st = P.st, sp = P.sp, cnr = C.nr, cnth = C.nth;
+    const LineOp &ln = P.ln;
     auto crow = [=](int j, int l) { return ((unsigned)(l >> sp) * cnth + (j >> st)) * cnr; };
-    auto vrow = [=](unsigned c0, int k, int j, int l) {
-        const unsigned K0 = crow(j, l) + (k >> 1);
-        const float2 x2 = make_float2(xc[K0], xc[K0 + 1]);
-        const float4 d = ldh4(idg + c0), bb = ld4(b + c0);
-        return make_float4(fmaf(kMgOmega * d.x, bb.x, x2.x), fmaf(kMgOmega * d.y, bb.y, x2.x),
-                           fmaf(kMgOmega * d.z, bb.z, x2.y), fmaf(kMgOmega * d.w, bb.w, x2.y));
-    };
-    auto vone = [=](unsigned i, int k, int j, int l) {
-        return fmaf(kMgOmega * ldh1(idg + i), b[i], xc[crow(j, l) + (k >> 1)]);
+    auto vone = [&](unsigned i, int k, int j, int l) {
+        const float cv = xc[crow(j, l) + (k >> sr)];
+        return ln.has(j) ? ln.x[ln.at(F.nr, k, j, l)] + cv : fmaf(kMgOmega * ldo1(idg + i), b[i], cv);
     };
     KSum rz;
-    for (unsigned c = 4u * (blockIdx.x * blockDim.x + threadIdx.x); c < F.n; c += 4u * gridDim.x * blockDim.x) {
-        int k, j, l;
-        cell_ijk(c, F.nr, F.nth, F.dnr, F.dnth, k, j, l);
-        const float4 vc = vrow(c, k, j, l);
-        const float4 ax = apply_quad(F, P.h, vrow, vone, c, k, j, l, vc);
-        const float4 d = ldh4(idg + c), bb = ld4(b + c);
-        const float4 z = make_float4(fmaf(kMgOmega * d.x, bb.x - ax.x, vc.x), fmaf(kMgOmega * d.y, bb.y - ax.y, vc.y),
-                                     fmaf(kMgOmega * d.z, bb.z - ax.z, vc.z), fmaf(kMgOmega * d.w, bb.w - ax.w, vc.w));
-        st4(F.x + c, z);
-        rz.add(bb.x * z.x);
-        rz.add(bb.y * z.y);
-        rz.add(bb.z * z.z);
-        rz.add(bb.w * z.w);
+    for_cells<Q>(P.cg, 0u, [&](unsigned c, int k, int j, int l) {
+        if constexpr (Q) {
+            auto vrow = [&](unsigned c0, int k, int j, int l) {
+                const float2 x2 = *reinterpret_cast<const float2 *>(xc + crow(j, l) + (k >> 1));
+                if (ln.has(j)) {
+                    const float4 x0 = ld4(ln.x + ln.at(F.nr, k, j, l));
+                    return make_float4(x0.x + x2.x, x0.y + x2.x, x0.z + x2.y, x0.w + x2.y);
+                }
+                const float4 d = ldo4(idg + c0), bb = ld4(b + c0);
+                return make_float4(fmaf(kMgOmega * d.x, bb.x, x2.x), fmaf(kMgOmega * d.y, bb.y, x2.x),
+                                   fmaf(kMgOmega * d.z, bb.z, x2.y), fmaf(kMgOmega * d.w, bb.w, x2.y));
+            };
+            const float4 vc = vrow(c, k, j, l);
+            const float4 ax = flux_quad(F.nr, F.nth, F.nph, F.n, os, ow, vrow, vone, c, k, j, l, vc);
+            const float4 bb = ld4(b + c);
+            const float4 res = make_float4(bb.x - ax.x, bb.y - ax.y, bb.z - ax.z, bb.w - ax.w);
+            if (ln.has(j)) {
+                st4(F.x + c, vc);
+                st4(ln.res + ln.at(F.nr, k, j, l), res);
+                return;
+            }
+            const float4 d = ldo4(idg + c);
+            const float4 z = make_float4(fmaf(kMgOmega * d.x, res.x, vc.x), fmaf(kMgOmega * d.y, res.y, vc.y),
+                                         fmaf(kMgOmega * d.z, res.z, vc.z), fmaf(kMgOmega * d.w, res.w, vc.w));
+            st4(F.x + c, z);
+            rz.add(bb.x * z.x);
+            rz.add(bb.y * z.y);
+            rz.add(bb.z * z.z);
+            rz.add(bb.w * z.w);
+        } else {
+            const float vc = vone(c, k, j, l);
+            const float res = b[c] - flux_one(F.nr, F.nth, F.nph, F.n, os, ow, vone, c, k, j, l, vc);
+            if (ln.has(j)) {
+                F.x[c] = vc;
+                ln.res[ln.at(F.nr, k, j, l)] = res;
+                return;
+            }
+            const float z = fmaf(kMgOmega * ldo1(idg + c), res, vc);
+            F.x[c] = z;
+            rz.add(b[c] * z);
+        }
+    });
+    if (ln.nl > 0) {  // k_line_post sums these partials with its own
+        const KSum t = block_reduce(rz);
+        if (threadIdx.x == 0) P.cg.part[blockIdx.x] = t.value();
+        return;
     }
     double tot;
-    if (grid_reduce<false>(P.cg, rz.value(), &tot)) {
-        double *sc = P.cg.scal;
-        if (init) {
-            sc[kRz] = tot;
-            sc[kRz0] = tot;
-            sc[kBeta] = 0.0;
-            sc[kDone] = tot > 0.0 ? 0.0 : 1.0;
-        } else {
-            sc[kBeta] = sc[kRz] > 0.0 ? tot / sc[kRz] : 0.0;
-            sc[kRz] = tot;
-            sc[kIters] += 1.0;
-            if (!(tot > kInnerDropMg * kInnerDropMg * sc[kRz0])) sc[kDone] = 1.0;
-        }
-    }
+    if (grid_reduce(P.cg, rz, &tot)) close_step(P.cg, tot);
+}
+
+// z = x1 + omega T^-1 (b - A x1) of the line rows, and their share of r.z (after the partials of
+// k_mg_up0, rows_partials of them)
+template <bool SM>
+__global__ void __launch_bounds__(512, 2) k_line_post(const CgArgs a, const LineOp L, int rows_partials)
+{
+    if (a.scal[kDone] != 0.0) return;
+    KSum rz;
+    line_solve<SM>(L, a, L.res, [&](unsigned, unsigned i) { return L.res[i]; }, [](unsigned, float) {},
+                   [&](unsigned c, unsigned, float2 &e) { e = make_float2(a.z[c], a.r[c]); },
+                   [&](unsigned c, unsigned, float x, float2 e) {
+                       const float z = fmaf(kMgOmega, x, e.x);
+                       a.z[c] = z;
+                       rz.add(e.y * z);
+                   });
+    double tot;
+    if (grid_reduce(a, rz, &tot, rows_partials)) close_step(a, tot);
 }
 
 #undef MG_LOOP
-
-// CG steps of the multigrid path (the preconditioned residual z comes from k_mg_up)
-// r = b - A x, d = 0, p = 0
-__global__ void __launch_bounds__(256) k_cg_residual_mg(const CgArgs a)
-{
-    FLD_CELLS(c)
-    {
-        a.r[c] = a.b[c] - apply_flux(a, a.x, c);
-        a.d[c] = 0.0f;
-        a.p[c] = 0.0f;
-    }
-}
-
-// d += alpha p, r -= alpha q (four cells per thread; n % 4 == 0)
-__global__ void __launch_bounds__(256) k_cg_update_mg4(const CgArgs a)
-{
-    if (a.scal[kDone] != 0.0) return;
-    const float alpha = (float)a.scal[kAlpha];
-    for (unsigned c = 4u * (blockIdx.x * blockDim.x + threadIdx.x); c < (unsigned)a.n; c += 4u * gridDim.x * blockDim.x) {
-        const float4 p = ld4(a.p + c), q = ld4(a.q + c);
-        float4 d = ld4(a.d + c), r = ld4(a.r + c);
-        d = make_float4(fmaf(alpha, p.x, d.x), fmaf(alpha, p.y, d.y), fmaf(alpha, p.z, d.z), fmaf(alpha, p.w, d.w));
-        r = make_float4(fmaf(-alpha, q.x, r.x), fmaf(-alpha, q.y, r.y), fmaf(-alpha, q.z, r.z),
-                        fmaf(-alpha, q.w, r.w));
-        st4(a.d + c, d);
-        st4(a.r + c, r);
-    }
-}
-
-__global__ void __launch_bounds__(256) k_cg_update_mg(const CgArgs a)
-{
-    if (a.scal[kDone] != 0.0) return;
-    const float alpha = (float)a.scal[kAlpha];
-    FLD_CELLS(c)
-    {
-        a.d[c] = fmaf(alpha, a.p[c], a.d[c]);
-        a.r[c] = fmaf(-alpha, a.q[c], a.r[c]);
-    }
-}
-
-// p = z + beta p (z: the finest level's multigrid result)
-__global__ void __launch_bounds__(256) k_cg_direction_mg4(const CgArgs a, const float *z)
-{
-    if (a.scal[kDone] != 0.0) return;
-    const float beta = (float)a.scal[kBeta];
-    for (unsigned c = 4u * (blockIdx.x * blockDim.x + threadIdx.x); c < (unsigned)a.n; c += 4u * gridDim.x * blockDim.x) {
-        const float4 zz = ld4(z + c), p = ld4(a.p + c);
-        st4(a.p + c, make_float4(fmaf(beta, p.x, zz.x), fmaf(beta, p.y, zz.y), fmaf(beta, p.z, zz.z),
-                                 fmaf(beta, p.w, zz.w)));
-    }
-}
-
-__global__ void __launch_bounds__(256) k_cg_direction_mg(const CgArgs a, const float *z)
-{
-    if (a.scal[kDone] != 0.0) return;
-    const float beta = (float)a.scal[kBeta];
-    FLD_CELLS(c) a.p[c] = fmaf(beta, a.p[c], z[c]);
-}
-
-#undef FLD_CELLS
 
 int rosseland_nodes(const CtxInfo &in, const std::vector<double> &t_nodes, double *kr_host, float *lkr_dev,
                     cudaStream_t st, std::string &err)
@@ -1124,6 +1498,31 @@ FldGeo geo_view(const float *gp, int nr, int nth, int nph)
     return g;
 }
 
+// largest dynamic shared memory of the step's kernels: the line kernels' 32 rings of
+// kLineSmemPhi cells; a tail of 2048 + 1024 + 512 cells (one direction only) takes 112 KB
+constexpr size_t kMaxFldSmem = sizeof(float) * 32 * kLineSmemPhi;
+
+// segments a ring of nph cells is cut into (k_line_*: one warp each)
+int line_segments(int nph) { return std::max(4, std::min(kLineMaxSeg, nph / 8)); }
+
+// share of the diagonal the phi faces of row j hold where D is uniform, at the middle radius
+std::vector<double> phi_shares(const CtxInfo &in)
+{
+    const int nth = in.ntheta, nph = in.nphi, k = in.nr / 2;
+    const double *ri = in.r_if_h, *ti = in.theta_if_h;
+    const double dph = (in.phi_if_h[nph] - in.phi_if_h[0]) / nph;
+    const double rc = 0.5 * (ri[k] + ri[k + 1]), dr = ri[k + 1] - ri[k], dr2 = dr * rc;
+    std::vector<double> share(nth);
+    for (int j = 0; j < nth; ++j) {
+        const double th = 0.5 * (ti[j] + ti[j + 1]), dth = ti[j + 1] - ti[j];
+        const double p = 2.0 * dth * dr2 / (rc * fabs(sin(th)) * dph);
+        const double t = dph * (sin(ti[j]) + sin(ti[j + 1])) * dr2 / (rc * dth);
+        const double r = in.nr > 1 ? 2.0 * dph * (cos(ti[j]) - cos(ti[j + 1])) * rc * rc / dr : 0.0;
+        share[j] = p / (p + t + r);
+    }
+    return share;
+}
+
 double radiation_constant()
 {
     const double sigma = 2.0 * pow(kPi, 5) * pow(kKB, 4) / (15.0 * kH * kH * kH * kC * kC);
@@ -1137,13 +1536,15 @@ void fld_free(FldState *s)
     if (!s) return;
     cudaFree(s->buf);
     cudaFree(s->mg_buf);
+    cudaFree(s->line_buf);
     cudaFree(s->part);
     cudaFree(s->scal);
     cudaFree(s->bad);
     cudaFree(s->count);
     cudaFree(s->geo);
     cudaFree(s->lkr);
-    if (s->burst) cudaGraphExecDestroy(s->burst);
+    if (s->loop) cudaGraphExecDestroy(s->loop);
+    cudaFreeHost(s->scal_h);
     if (s->ev_in) cudaEventDestroy(s->ev_in);
     if (s->gs) cudaStreamDestroy(s->gs);
     delete s;
@@ -1205,13 +1606,14 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
         cudaFree(fs->buf);
         fs->buf = nullptr;
         fs->cap = 0;
-        if (cudaMalloc(&fs->buf, sizeof(float) * 18 * (size_t)n) != cudaSuccess) {
+        if (cudaMalloc(&fs->buf, sizeof(float) * (14 * (size_t)n + (5 * (size_t)n + 1) / 2)) != cudaSuccess) {
             cudaGetLastError();
             return ctx_fail(ctx, RT_ERR_NO_MEMORY, "FLD workspace");
         }
         fs->cap = n;
     }
-    const int grid_max = 8 * nsm;  // 256-thread CTAs resident per SM are at most 8
+    // at most 16 resident CTAs per SM (128 threads and more), and one CTA per 32 rings before them
+    const int grid_max = 16 * nsm + nth * ((nr + 31) / 32);
     if (fs->part_cap < grid_max) {
         cudaFree(fs->part);
         fs->part = nullptr;
@@ -1226,11 +1628,14 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
         if (cudaMalloc(&fs->scal, sizeof(double) * kNScal) != cudaSuccess ||
             cudaMalloc(&fs->bad, sizeof(unsigned)) != cudaSuccess ||
             cudaMalloc(&fs->count, sizeof(unsigned)) != cudaSuccess ||
+            cudaMallocHost(&fs->scal_h, sizeof(double) * (kNScal + 1)) != cudaSuccess ||
             cudaMemset(fs->count, 0, sizeof(unsigned)) != cudaSuccess) {
             cudaGetLastError();
             cudaFree(fs->scal);
             cudaFree(fs->bad);
             cudaFree(fs->count);
+            cudaFreeHost(fs->scal_h);
+            fs->scal_h = nullptr;
             fs->scal = nullptr;
             fs->bad = fs->count = nullptr;
             return ctx_fail(ctx, RT_ERR_NO_MEMORY, "FLD scalars");
@@ -1263,6 +1668,22 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
             return ctx_fail(ctx, RT_ERR_NO_MEMORY, "FLD multigrid levels");
         }
     }
+    if (!fs->lines_set) {  // the rows smoothed by phi lines: a run at each theta end (LineOp)
+        fs->line_j0 = 0;
+        fs->line_j1 = nth;
+        if (fs->mg_dims.size() > 3 && nph >= kLineMinPhi) {
+            const std::vector<double> share = phi_shares(in);
+            while (fs->line_j0 < nth && share[fs->line_j0] > kLineShare) ++fs->line_j0;
+            while (fs->line_j1 > fs->line_j0 && share[fs->line_j1 - 1] > kLineShare) --fs->line_j1;
+        }
+        const size_t rows = (size_t)(fs->line_j0 + nth - fs->line_j1) * nr;
+        const size_t S = line_segments(nph);
+        if (rows > 0 && cudaMalloc(&fs->line_buf, sizeof(float) * rows * (5 * (size_t)nph + S * S)) != cudaSuccess) {
+            cudaGetLastError();
+            return ctx_fail(ctx, RT_ERR_NO_MEMORY, "FLD line smoother");
+        }
+        fs->lines_set = true;
+    }
     if (!fs->lkr_valid || fs->lkr_fp != in.table_fingerprint) {
         if (!fs->lkr && cudaMalloc(&fs->lkr, sizeof(float) * kRossNodes) != cudaSuccess) {
             cudaGetLastError();
@@ -1281,6 +1702,7 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
     const double a_rad = radiation_constant();
     float *F = fs->buf, *tc = F + n, *b0 = tc + n, *w = b0 + n, *sv = w + 3 * n, *idg = sv + n, *b = idg + n;
     float *d = b + n, *r = d + n, *p = r + n, *q = p + n, *z = q + n;
+    float *x = tc, *pbuf[2] = {p, F};  // tc and F are free once the face kernel has run
     unsigned short *hs = reinterpret_cast<unsigned short *>(z + n), *hw = hs + n, *hidg = hw + 3 * n;
 
     FldCellArgs ca;
@@ -1315,6 +1737,8 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
     fa.hs = hs;
     fa.hw = hw;
     fa.hidg = hidg;
+    fa.e = e_old;
+    fa.x = x;
     fa.n = n;
     CgArgs cg;
     cg.nr = nr;
@@ -1327,11 +1751,11 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
     cg.s = sv;
     cg.idg = idg;
     cg.b = b;
-    cg.x = e_new;
+    cg.x = x;
     cg.d = d;
     cg.r = r;
-    cg.p = p;
     cg.q = q;
+    cg.z = z;
     cg.part = fs->part;
     cg.scal = fs->scal;
     cg.count = fs->count;
@@ -1376,156 +1800,160 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
         pairs[i].cg = cg;
         pairs[i].h = HalfOp{hs, hw, hidg};
     }
-    auto work_grid = [&](const void *kern, unsigned cells) {
+    // phi lines of the finest level
+    LineOp ln{0, nth, 0, 0, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    const int nl = fs->line_j0 + nth - fs->line_j1;
+    const bool lines = use_mg && nl > 0;
+    if (lines) {
+        const size_t rows = (size_t)nl * nr;
+        ln.j0 = fs->line_j0;
+        ln.j1 = fs->line_j1;
+        ln.nl = nl;
+        ln.seg = line_segments(nph);
+        ln.blocks = nl * ((nr + 31) / 32);
+        ln.m = fs->line_buf;
+        ln.vl = ln.m + rows * nph;
+        ln.vr = ln.vl + rows * nph;
+        ln.x = ln.vr + rows * nph;
+        ln.res = ln.x + rows * nph;
+        ln.inv = ln.res + rows * nph;
+    }
+    if (use_mg) pairs[0].ln = ln;
+    // the levels of the one-CTA tail
+    MgTail tail{};
+    int t0 = n_lv;
+    if (use_mg) {
+        for (t0 = 1; lv[t0].n > kTailCells || n_lv - t0 > kTailLevels;) ++t0;
+        for (int i = t0; i < n_lv; ++i) tail.lv[tail.n_lv++] = lv[i];
+        tail.scal = fs->scal;
+    }
+
+    // grids of one full wave: the CTAs resident per SM (from each kernel's registers) times the
+    // SM count, capped by the work
+    const bool quads = nr % 4 == 0;  // four cells per thread where a ray holds a multiple of four
+    auto wave = [&](const void *kern, int threads, size_t smem, long long work) {
         int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess || per_sm < 1)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem) != cudaSuccess || per_sm < 1)
             per_sm = 1;
-        return (int)std::max(1LL, std::min<long long>((cells + 255) / 256, (long long)per_sm * nsm));
+        return (int)std::max(1LL, std::min<long long>((work + threads - 1) / threads, (long long)per_sm * nsm));
     };
-    // the finest pair in four-cell form where the rays hold a multiple of four cells
-    const bool quad0 = nr % 4 == 0 && use_mg;
+    const long long work = quads ? n / 4 : n;
+    const int t_line = lines ? 32 * ln.seg : 256;
+    const bool ring_sm = nph <= kLineSmemPhi;
+    const size_t sm_line = lines && ring_sm ? sizeof(float) * t_line * (size_t)(nph / ln.seg) : 0;
+    const size_t sm_tail = use_mg ? tail_smem(tail) : 0;
+    using LevelFn = void (*)(const MgPair);
+    const LevelFn up0 = quads ? k_mg_up0<true> : k_mg_up0<false>;
+    const LevelFn down0 = quads ? k_mg_down4 : lines ? k_mg_down<true> : k_mg_down<false>;
+    const auto residual = quads ? (ring_sm ? k_it_residual<true, true> : k_it_residual<true, false>)
+                                : (ring_sm ? k_it_residual<false, true> : k_it_residual<false, false>);
+    const auto line_post = ring_sm ? k_line_post<true> : k_line_post<false>;
+    const auto apply = quads ? k_it_apply<true> : k_it_apply<false>;
+    const auto flush = quads ? k_it_flush<true> : k_it_flush<false>;
+    // (one limit for all contexts: another thread's smaller step must not lower it)
+    auto big_smem = [](const void *kern, size_t bytes) {
+        return bytes <= 48 * 1024 ||
+               (bytes <= kMaxFldSmem && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                             (int)kMaxFldSmem) == cudaSuccess);
+    };
+    if (!big_smem((const void *)residual, sm_line) || !big_smem((const void *)line_post, sm_line) ||
+        !big_smem((const void *)k_mg_tail, sm_tail))
+        return ctx_fail(ctx, RT_ERR_CUDA, "FLD shared memory");
+    const int g_res = ln.blocks + wave((const void *)residual, t_line, sm_line, work);
+    const int g_up0 = wave((const void *)up0, 256, 0, work);
+    const int g_app = wave((const void *)apply, 256, 0, work), g_flu = wave((const void *)flush, 256, 0, work);
+    const int g_jac = wave((const void *)k_it_jacobi, 256, 0, n);
     std::vector<int> g_down(n_lv, 1), g_up(n_lv, 1);
     for (int i = 0; i + 1 < n_lv; ++i) {
-        g_down[i] = (i == 0 && quad0) ? work_grid((const void *)k_mg_down4, lv[1].n / 2)
-                                      : work_grid((const void *)k_mg_down, lv[i + 1].n);
-        g_up[i] = (i == 0 && quad0) ? work_grid((const void *)k_mg_up4, lv[0].n / 4)
-                                    : work_grid((const void *)k_mg_up, lv[i].n);
+        g_down[i] = wave(i == 0 ? (const void *)down0 : (const void *)k_mg_down<false>, 256, 0,
+                         i == 0 && quads ? 2LL * lv[1].n : 8LL * lv[i + 1].n);
+        g_up[i] = wave((const void *)k_mg_up, 256, 0, lv[i].n);
     }
-    auto mg_apply = [&](int init) {
-        if (quad0) k_mg_down4<<<g_down[0], 256, 0, st>>>(pairs[0]);
-        else k_mg_down<<<g_down[0], 256, 0, st>>>(pairs[0]);
-        for (int i = 1; i + 1 < n_lv; ++i) k_mg_down<<<g_down[i], 256, 0, st>>>(pairs[i]);
-        k_mg_coarsest<<<1, 256, 0, st>>>(lv[n_lv - 1], fs->scal);
-        for (int i = n_lv - 2; i >= 1; --i) k_mg_up<<<g_up[i], 256, 0, st>>>(pairs[i], 0, init);
-        if (quad0) k_mg_up4<<<g_up[0], 256, 0, st>>>(pairs[0], init);
-        else k_mg_up<<<g_up[0], 256, 0, st>>>(pairs[0], 1, init);
+    // one iteration; p goes from pbuf[i & 1] to the other buffer
+    auto iteration = [&](int i) {
+        const float *pc = pbuf[i & 1];
+        flush<<<g_flu, 256, 0, st>>>(cg, pc);
+        residual<<<g_res, t_line, sm_line, st>>>(cg, ln);
+        if (use_mg) {
+            down0<<<g_down[0], 256, 0, st>>>(pairs[0]);
+            for (int v = 1; v < t0; ++v) k_mg_down<false><<<g_down[v], 256, 0, st>>>(pairs[v]);
+            k_mg_tail<<<1, 1024, sm_tail, st>>>(tail);
+            for (int v = t0 - 1; v >= 1; --v) k_mg_up<<<g_up[v], 256, 0, st>>>(pairs[v]);
+            up0<<<g_up0, 256, 0, st>>>(pairs[0]);
+            if (lines) line_post<<<ln.blocks, t_line, sm_line, st>>>(cg, ln, g_up0);
+        } else {
+            k_it_jacobi<<<g_jac, 256, 0, st>>>(cg);
+        }
+        apply<<<g_app, 256, 0, st>>>(cg, pc, pbuf[(i + 1) & 1]);
     };
+    if (!fs->loop && !fs->no_graph) {  // the loop's graph
+        cudaGraph_t graph = nullptr, body = nullptr, end = nullptr;
+        cudaGraphConditionalHandle h{};
+        cudaGraphNode_t node = nullptr;
+        cudaGraphNodeParams par = {};
+        bool cap = cudaGraphCreate(&graph, 0) == cudaSuccess &&
+                   cudaGraphConditionalHandleCreate(&h, graph, 1, cudaGraphCondAssignDefault) == cudaSuccess;
+        if (cap) {
+            par.type = cudaGraphNodeTypeConditional;
+            par.conditional.handle = h;
+            par.conditional.type = cudaGraphCondTypeWhile;
+            par.conditional.size = 1;
+            cap = cudaGraphAddNode(&node, graph, nullptr, nullptr, 0, &par) == cudaSuccess;
+        }
+        if (cap) {
+            body = par.conditional.phGraph_out[0];
+            cap = cudaStreamBeginCaptureToGraph(st, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
+                  cudaSuccess;
+        }
+        if (cap) {
+            for (int i = 0; i < kUnroll; ++i) iteration(i);
+            k_it_loop<<<1, 1, 0, st>>>(fs->scal, h);
+            cap = cudaStreamEndCapture(st, &end) == cudaSuccess;
+        }
+        cap = cap && cudaGraphInstantiate(&fs->loop, graph, 0) == cudaSuccess;
+        if (graph) cudaGraphDestroy(graph);
+        if (!cap) {
+            cudaGetLastError();
+            fs->loop = nullptr;
+            fs->no_graph = true;
+        }
+    }
 
-    auto sync_read = [&](double *h_sc, unsigned *h_bad) {
-        bool ok = cudaGetLastError() == cudaSuccess &&
-                  cudaMemcpyAsync(h_sc, fs->scal, sizeof(double) * kNScal, cudaMemcpyDeviceToHost, st) == cudaSuccess;
-        if (ok && h_bad) ok = cudaMemcpyAsync(h_bad, fs->bad, sizeof(unsigned), cudaMemcpyDeviceToHost, st) == cudaSuccess;
-        return ok && cudaStreamSynchronize(st) == cudaSuccess;
+    auto sync_read = [&]() {
+        return cudaGetLastError() == cudaSuccess &&
+               cudaMemcpyAsync(fs->scal_h, fs->scal, sizeof(double) * kNScal, cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+               cudaMemcpyAsync(fs->scal_h + kNScal, fs->bad, sizeof(unsigned), cudaMemcpyDeviceToHost, st) ==
+                   cudaSuccess &&
+               cudaStreamSynchronize(st) == cudaSuccess;
     };
-    double h_sc[kNScal];
-    unsigned h_bad = 0;
-    bool ok = cudaMemsetAsync(fs->bad, 0, sizeof(unsigned), st) == cudaSuccess &&
-              cudaMemsetAsync(fs->scal, 0, sizeof(double) * kNScal, st) == cudaSuccess;
+    bool ok = cudaMemsetAsync(fs->bad, 0, sizeof(unsigned), st) == cudaSuccess;
     k_fld_cell<<<grid, 256, 0, st>>>(ca);
     k_fld_faces<<<grid, 256, 0, st>>>(fa);
     for (int i = 0; i + 1 < n_lv; ++i) {  // coarse operators of this step
-        k_mg_coarsen<<<work_grid((const void *)k_mg_coarsen, lv[i + 1].n), 256, 0, st>>>(pairs[i]);
-        k_mg_diag<<<work_grid((const void *)k_mg_diag, lv[i + 1].n), 256, 0, st>>>(lv[i + 1]);
+        k_mg_coarsen<<<wave((const void *)k_mg_coarsen, 256, 0, lv[i + 1].n), 256, 0, st>>>(pairs[i]);
+        k_mg_diag<<<wave((const void *)k_mg_diag, 256, 0, lv[i + 1].n), 256, 0, st>>>(lv[i + 1]);
     }
-    ok = ok && sync_read(h_sc, &h_bad);
-    if (!ok) return ctx_fail(ctx, RT_ERR_CUDA, std::string("FLD set-up: ") + cudaGetErrorString(cudaGetLastError()));
+    if (lines) k_line_setup<<<ln.blocks, t_line, 0, st>>>(ln, cg);
+    k_it_start<<<1, 1, 0, st>>>(fs->scal, fs->bad, fs->count, tol, (double)max_iter);
+    if (fs->loop) {
+        ok = ok && cudaGraphLaunch(fs->loop, st) == cudaSuccess;
+    } else {
+        for (double left = max_iter + 4.0 * kUnroll; ok && left > 0.0; left -= kUnroll) {
+            for (int i = 0; i < kUnroll; ++i) iteration(i);
+            ok = sync_read();
+            if (ok && fs->scal_h[kDone] != 0.0) break;
+        }
+    }
+    k_it_store<<<grid, 256, 0, st>>>(x, e_new, n, fs->bad);
+    ok = ok && sync_read();
+    if (!ok) return ctx_fail(ctx, RT_ERR_CUDA, std::string("FLD step: ") + cudaGetErrorString(cudaGetLastError()));
+    unsigned h_bad = 0;
+    memcpy(&h_bad, fs->scal_h + kNScal, sizeof(unsigned));
     if (h_bad)
         return ctx_fail(ctx, RT_ERR_NONFINITE_INPUT,
                         "FLD input holds rho < 0, T <= 0, E_old < 0, q_abs < 0 or a NaN/Inf");
-    if (cudaMemcpyAsync(e_new, e_old, sizeof(float) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return ctx_fail(ctx, RT_ERR_CUDA, "FLD start value");
-
-    // refinement passes; the inner iterations go in bursts of kBurst, whose launches
-    // return at once after the device flagged convergence (8 measured 1 % faster per
-    // step than 16 with multigrid: fewer idle launches at the end of a pass)
-    constexpr int kBurst = 8;
-    int iters = 0, passes = 0;
-    double corr = INFINITY;
-    bool done = false;
-    // four cells per thread where a ray holds a multiple of four cells
-    const bool quads = nr % 4 == 0;
-    // grids of one full wave: the CTAs resident per SM (from each kernel's registers)
-    // times the SM count, capped by the work
-    auto wave = [&](const void *kern) {
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess || per_sm < 1)
-            per_sm = 1;
-        const long long work = ((quads ? n / 4 : n) + 255) / 256;
-        return (int)std::max(1LL, std::min<long long>(work, (long long)per_sm * nsm));
-    };
-    const int g_res = quads ? wave((const void *)k_cg_residual4) : wave((const void *)k_cg_residual);
-    const int g_app = quads ? wave((const void *)k_cg_apply4) : wave((const void *)k_cg_apply);
-    const int g_upd = quads ? wave((const void *)k_cg_update4) : wave((const void *)k_cg_update);
-    const int g_dir = quads ? wave((const void *)k_cg_direction4) : wave((const void *)k_cg_direction);
-    const int g_acc = wave((const void *)k_cg_accumulate);
-    // one inner iteration: q = A p, the updates, z = M^-1 r and r.z, the new direction
-    auto iteration = [&]() {
-        if (use_mg) {
-            if (quads) {
-                k_cg_apply4<<<g_app, 256, 0, st>>>(cg);
-                k_cg_update_mg4<<<g_upd, 256, 0, st>>>(cg);
-            } else {
-                k_cg_apply<<<g_app, 256, 0, st>>>(cg);
-                k_cg_update_mg<<<g_upd, 256, 0, st>>>(cg);
-            }
-            mg_apply(0);
-            if (quads) k_cg_direction_mg4<<<g_dir, 256, 0, st>>>(cg, z);
-            else k_cg_direction_mg<<<g_dir, 256, 0, st>>>(cg, z);
-        } else if (quads) {
-            k_cg_apply4<<<g_app, 256, 0, st>>>(cg);
-            k_cg_update4<<<g_upd, 256, 0, st>>>(cg);
-            k_cg_direction4<<<g_dir, 256, 0, st>>>(cg);
-        } else {
-            k_cg_apply<<<g_app, 256, 0, st>>>(cg);
-            k_cg_update<<<g_upd, 256, 0, st>>>(cg);
-            k_cg_direction<<<g_dir, 256, 0, st>>>(cg);
-        }
-    };
-    while (!done) {
-        if (cudaMemsetAsync(fs->scal + kDone, 0, sizeof(double), st) != cudaSuccess)
-            return ctx_fail(ctx, RT_ERR_CUDA, "FLD pass start");
-        if (use_mg) {
-            k_cg_residual_mg<<<g_res, 256, 0, st>>>(cg);
-            mg_apply(1);
-            if (quads) k_cg_direction_mg4<<<g_dir, 256, 0, st>>>(cg, z);
-            else k_cg_direction_mg<<<g_dir, 256, 0, st>>>(cg, z);
-        } else if (quads) {
-            k_cg_residual4<<<g_res, 256, 0, st>>>(cg);
-        } else {
-            k_cg_residual<<<g_res, 256, 0, st>>>(cg);
-        }
-        bool inner_done = false;
-        while (!inner_done && iters < max_iter) {
-            const int burst = std::min(kBurst, max_iter - iters);
-            if (burst == kBurst && !fs->no_graph && (!fs->burst || fs->burst_x != e_new || fs->burst_buf != fs->buf)) {
-                // (re)capture the burst: its launches point at e_new and the workspace
-                if (fs->burst) cudaGraphExecDestroy(fs->burst);
-                fs->burst = nullptr;
-                cudaGraph_t graph = nullptr;
-                bool cap = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-                if (cap) {
-                    for (int i = 0; i < kBurst; ++i) iteration();
-                    cap = cudaStreamEndCapture(st, &graph) == cudaSuccess && graph;
-                }
-                if (cap) cap = cudaGraphInstantiate(&fs->burst, graph, 0) == cudaSuccess;
-                if (graph) cudaGraphDestroy(graph);
-                if (!cap) {  // run the bursts as plain launches from now on
-                    cudaGetLastError();
-                    if (fs->burst) cudaGraphExecDestroy(fs->burst);
-                    fs->burst = nullptr;
-                    fs->no_graph = true;
-                }
-                fs->burst_x = e_new;
-                fs->burst_buf = fs->buf;
-            }
-            if (burst == kBurst && fs->burst && !fs->no_graph) {
-                if (cudaGraphLaunch(fs->burst, st) != cudaSuccess)
-                    return ctx_fail(ctx, RT_ERR_CUDA, "FLD graph launch");
-            } else {
-                for (int i = 0; i < burst; ++i) iteration();
-            }
-            if (!sync_read(h_sc, nullptr))
-                return ctx_fail(ctx, RT_ERR_CUDA, std::string("FLD iteration: ") + cudaGetErrorString(cudaGetLastError()));
-            iters = (int)h_sc[kIters];
-            inner_done = h_sc[kDone] != 0.0;
-        }
-        k_cg_accumulate<<<g_acc, 256, 0, st>>>(cg);
-        if (!sync_read(h_sc, nullptr))
-            return ctx_fail(ctx, RT_ERR_CUDA, std::string("FLD refinement: ") + cudaGetErrorString(cudaGetLastError()));
-        ++passes;
-        corr = h_sc[kCorr];
-        done = corr < tol || iters >= max_iter || isinf(corr);
-    }
+    const int iters = (int)fs->scal_h[kIters], passes = (int)fs->scal_h[kPasses];
+    const double corr = fs->scal_h[kCorr];
     if (stats) {
         stats->levels = use_mg ? n_lv : 1;
         stats->iterations = iters;
