@@ -405,8 +405,8 @@ int rt_planck_mean_opacity(rt_ctx *ctx, double t, double *kappa_p);
  *           field (erg cm^-3), or NULL for E_R = 0;
  *   t_dust  device, same layout, receives T (K); 0 where a_rad = E_R = 0.
  * kappa_P(T) is tabulated for the context's table on 1 K .. 1e5 K (1024 points of
- * ln T, cubic interpolation) and held constant outside; the root is found by
- * Newton's method on ln T in FP32. Asynchronous on the context's stream (the first
+ * ln T, cubic interpolation) and held constant outside; the root is found in FP32
+ * (from a table where E_R = 0, by Halley and Newton steps on ln T with E_R). Asynchronous on the context's stream (the first
  * call per table builds the table and synchronises). */
 int rt_dust_temperature(rt_ctx *ctx, const float *a_rad, const float *e_rad, float *t_dust);
 
