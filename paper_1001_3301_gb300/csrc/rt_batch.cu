@@ -108,7 +108,10 @@ __global__ void __launch_bounds__(W * 32, MINB) k_batch_ray(const __grid_constan
     __shared__ unsigned s_next;
     extern __shared__ __align__(16) unsigned char smem[];
     const int warp = threadIdx.x >> 5;
-    float *const s_kap = reinterpret_cast<float *>(smem);
+    // the warps' stages first (their place must not depend on the grid), then its bin tables
+    float *const s_stage = reinterpret_cast<float *>(smem) + warp * ray_stage_len(C);
+    float *const s_kap = reinterpret_cast<float *>(smem) + W * ray_stage_len(C);
+    static_assert(W * ray_stage_len(C) % 4 == 0, "the bin tables stay 16-byte aligned");
     float4 *s_nu = nullptr, *s_mom = nullptr;
     if (threadIdx.x == 0) s_next = atomicAdd(bp.work, 1u);
     __syncthreads();
@@ -154,9 +157,21 @@ __global__ void __launch_bounds__(W * 32, MINB) k_batch_ray(const __grid_constan
         const unsigned units = bp.grid_tile_begin[cur + 1] - bp.grid_tile_begin[cur];
         const unsigned w0 = (c - bp.chunk_begin[cur]) * bp.chunk_slots;
         const unsigned w1 = w0 + bp.chunk_slots < units ? w0 + bp.chunk_slots : units;
-        if (G == 8) ray_slots<C, W, MODE, 8>(s_p, w0 + warp, w1, W, rs, s_kap, s_nu, s_mom, eabs, eesc);
-        else if (G == 16) ray_slots<C, W, MODE, 16>(s_p, w0 + warp, w1, W, rs, s_kap, s_nu, s_mom, eabs, eesc);
-        else ray_slots<C, W, MODE, 32>(s_p, w0 + warp, w1, W, rs, s_kap, s_nu, s_mom, eabs, eesc);
+        const bool vec = ray_vec(s_p, C);
+        auto trace = [&](auto g) {
+            constexpr int GG = decltype(g)::value;
+            if constexpr (ray_staged(C, GG)) {
+                if (!vec) {
+                    ray_slots<C, W, MODE, GG, 1, false, false, false, true>(s_p, w0 + warp, w1, W, rs, s_kap, s_nu, s_mom,
+                                                                            eabs, eesc, s_stage);
+                    return;
+                }
+            }
+            ray_slots<C, W, MODE, GG>(s_p, w0 + warp, w1, W, rs, s_kap, s_nu, s_mom, eabs, eesc, s_stage);
+        };
+        if (G == 8) trace(std::integral_constant<int, 8>());
+        else if (G == 16) trace(std::integral_constant<int, 16>());
+        else trace(std::integral_constant<int, 32>());
         __syncthreads();  // s_next holds the next chunk
         c = s_next;
     }
@@ -304,9 +319,11 @@ int plan(rt_batch *b, const BatchShape *s)
     const long long T = 32LL * s->w * s->c;
     size_t smem = 0;
     for (const rt::CtxView &v : b->views)
-        smem = std::max(smem, ray ? rt::ray_bin_smem(v.args.nnu_pad) + 16 : tile_smem(v.args, *s));
-    if (smem > 48 * 1024)
-        RT_BCK(b, cudaFuncSetAttribute(s->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        smem = std::max(smem, ray ? rt::ray_bin_smem(v.args.nnu_pad) + 16 + sizeof(float) * s->w * rt::ray_stage_len(s->c)
+                                  : tile_smem(v.args, *s));
+    if (smem > 24 * 1024)  // beyond 48 KB with the static part
+        RT_BCK(b, cudaFuncSetAttribute(s->kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)std::max<size_t>(smem, 96 * 1024)));
     int nsm = 0, per_sm = 0;
     RT_BCK(b, cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->dev));
     RT_BCK(b, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, s->kern, s->w * 32, smem));

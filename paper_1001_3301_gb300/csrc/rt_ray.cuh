@@ -88,11 +88,31 @@ __device__ __forceinline__ float ex_lg2(float x)
     return y;
 }
 
-// Ask L2 for `bytes` bytes from p (16-byte aligned, a multiple of 16): a hint with
+// Ask L2 for n floats from p, less what lies outside whole 16-byte units: a hint with
 // no completion to wait for.
-__device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
+__device__ __forceinline__ void prefetch_l2(const float *p, unsigned n)
 {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+    const size_t a = (reinterpret_cast<size_t>(p) + 15) & ~size_t(15);
+    const size_t e = (reinterpret_cast<size_t>(p) + 4 * (size_t)n) & ~size_t(15);
+    if (e > a)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((unsigned)(e - a)) : "memory");
+}
+
+// Fields whose rays do not start on vector boundaries (nr not a multiple of the vector, or
+// unaligned arrays) pass through shared memory: the warp copies its cells with consecutive lanes
+// on consecutive words, one chunk ahead, and each lane reads its own run from there. Straight loads
+// put the lanes C words apart, a sector each (301x128x128, 79 bins, tau550 = 0.3, C = 12: 47 -> 33 us;
+// 450x64x64, C = 16: 29 -> 15; 999x64x64, chunked: 58 -> 40). With few cells per lane, or short rays
+// of which a warp holds several, the straight loads are as good (101x128x128, C = 8: 21.2 us
+// against 21.9 staged), hence the line of ray_staged.
+// Floats per warp: two buffers of two arrays of 32 C cells, skewed against bank conflicts.
+__host__ __device__ constexpr int ray_stage_len(int c) { return 4 * 33 * c; }
+__host__ __device__ constexpr bool ray_staged(int c, int g) { return c >= 12 || (c == 8 && g == 32); }
+__host__ __device__ constexpr bool ray_vec(const TraceArgs &p, int c)
+{
+    const int v = c % 4 == 0 ? 4 : 2;
+    return p.nr % v == 0 && ((reinterpret_cast<size_t>(p.rho) | reinterpret_cast<size_t>(p.tdust) |
+                              reinterpret_cast<size_t>(p.q) | reinterpret_cast<size_t>(p.a)) % (4 * v) == 0);
 }
 
 // One lane's series in v = s2 u: Q(v) = sum_{k=1..K} F_k v^k. A cell with column u
@@ -261,11 +281,12 @@ __device__ __forceinline__ void ray_tables_mc(const TraceArgs &p, float2 *s_dr, 
 // weight b(T). LUT: the absorbed power of the cells comes from the lookup table of
 // TraceArgs::lut (the per-bin sum only in warp-slots that hold a flagged cell).
 // MC: the chunked form; s_dr_mc / s_gqa_mc hold the radial constants of every chunk,
-// [chunk][j / 2][lane in the segment] (ray_tables_mc).
-template <int C, int W, int MODE, int G, int P = 1, bool TW = false, bool LUT = false, bool MC = false>
+// [chunk][j / 2][lane in the segment] (ray_tables_mc). ST: the fields pass through s_stage, the
+// warp's ray_stage_len(C) floats.
+template <int C, int W, int MODE, int G, int P = 1, bool TW = false, bool LUT = false, bool MC = false, bool ST = false>
 __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin, unsigned wr_end, unsigned step,
                                           const RayShared<C, P> &rs, const float *s_kap, const float4 *s_nu,
-                                          const float4 *s_mom, KahanSum &eabs, KahanSum &eesc,
+                                          const float4 *s_mom, KahanSum &eabs, KahanSum &eesc, float *s_stage,
                                           const float2 *s_dr_mc = nullptr, const float4 *s_gqa_mc = nullptr)
 {
     static_assert(MODE != RT_FP64, "the FP64 mode uses the tile kernel");
@@ -299,14 +320,32 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
     const int nr = p.nr;
     const int nch = MC ? (nr + G * C - 1) / (G * C) : 1;  // chunks per ray
     // vector access needs every lane start and the field bases 4V-byte aligned
-    const bool vec = (nr % V == 0) &&
-                     ((reinterpret_cast<size_t>(p.rho) | reinterpret_cast<size_t>(p.tdust) |
-                       reinterpret_cast<size_t>(p.q) | reinterpret_cast<size_t>(p.a)) % (4 * V) == 0);
-    // a warp-slot's fields are R consecutive rays: one contiguous run per field
-    const bool pf = (nr % 4 == 0) &&
-                    ((reinterpret_cast<size_t>(p.rho) | reinterpret_cast<size_t>(p.tdust)) % 16 == 0);
+    const bool vec = !ST && ray_vec(p, C);
+    const int s_idx0 = seg * (G * C) + (lane % G) * C;  // the lane's first cell in the stage
+    float *s_one = s_stage, *s_two = s_stage + 33 * C;  // this chunk's buffers
+    // the warp's cells of one chunk, run by run (a segment's cells are one run of memory):
+    // f(index in the stage, index in the fields)
+    auto each_run = [&](unsigned wr, int ch, auto f) {
+#pragma unroll
+        for (int s = 0; s < R; ++s) {
+            const unsigned r = wr * R + s;
+            const int k0 = (ch * G + half * 32) * C, len = r < p.nrays ? min(G * C, nr - k0) : 0;
+            const size_t m0 = (size_t)r * nr + k0;
+            for (int i = lane; i < len; i += 32) f(skew(s * (G * C) + i), m0 + i);
+        }
+    };
+    auto stage_in = [&](unsigned wr, int ch, float *one, float *two) {
+        each_run(wr, ch, [&](int i, size_t m) {
+            cp_async4(one + i, p.rho + m);
+            cp_async4(two + i, p.tdust + m);
+        });
+    };
     const int na = p.n_active;
     const float2 tiny2 = f2(FLT_MIN);
+    if constexpr (ST) {
+        __syncwarp();  // a previous range of slots may still be leaving the buffers
+        if (wr_begin < wr_end) stage_in(wr_begin, 0, s_one, s_two);
+    }
 
     for (unsigned wr = wr_begin; wr < wr_end; wr += step) {
         const unsigned ray = wr * R + seg;
@@ -321,7 +360,23 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
 
         // the fields, straight from HBM (or from L2, where the prefetch got there first)
         float2 rho2[C / 2], td2[C / 2];
-        if (vec && nv == C) {
+        if constexpr (ST) {
+            cp_async_wait_all();
+            __syncwarp();
+            // cells past the ray's end: no density, no dust (their column is 0 with any t_sub)
+#pragma unroll
+            for (int j = 0; j < C; j += 2) {
+                const int i0 = skew(s_idx0 + j), i1 = skew(s_idx0 + j + 1);
+                rho2[j / 2] = make_float2(j < nv ? s_one[i0] : 0.0f, j + 1 < nv ? s_one[i1] : 0.0f);
+                td2[j / 2] = make_float2(j < nv ? s_two[i0] : INFINITY, j + 1 < nv ? s_two[i1] : INFINITY);
+            }
+            // the next chunk into the other buffers (their outputs left before the barrier)
+            const unsigned wn = ch + 1 < nch ? wr : wr + step;
+            if (wn < wr_end) {
+                const bool first = s_one == s_stage;
+                stage_in(wn, ch + 1 < nch ? ch + 1 : 0, first ? s_stage + 66 * C : s_stage, first ? s_stage + 99 * C : s_stage + 33 * C);
+            }
+        } else if (vec && nv == C) {
 #pragma unroll
             for (int j = 0; j < C; j += V) {
                 if constexpr (V == 4) {
@@ -337,7 +392,7 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
                 }
             }
         } else {
-            // cells past the ray's end: no density, no dust (their column is 0 with any t_sub)
+            // the last lanes of a ray
 #pragma unroll
             for (int j = 0; j < C; j += 2) {
                 rho2[j / 2] = make_float2(j < nv ? __ldg(p.rho + base + j) : 0.0f,
@@ -350,24 +405,24 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
         // first warp asks for the whole ray); in the chunked form each segment's first
         // lane asks for its ray's next chunk (the first chunk of its next ray after the
         // last), the same distance ahead as one slot of the one-chunk form
-        if constexpr (MC) {
-            if (pf && lane % G == 0) {
+        if constexpr (ST) {
+        } else if constexpr (MC) {
+            if (lane % G == 0) {
                 const bool last = ch + 1 == nch;
                 const unsigned rn = last ? (wr + step) * R + seg : ray;
                 const int k0 = last ? 0 : (ch + 1) * G * C;
                 if ((!last || wr + step < wr_end) && rn < p.nrays) {
-                    const unsigned bytes = (unsigned)min(G * C, nr - k0) * 4u;
-                    prefetch_l2(p.rho + (size_t)rn * nr + k0, bytes);
-                    prefetch_l2(p.tdust + (size_t)rn * nr + k0, bytes);
+                    const unsigned cells = (unsigned)min(G * C, nr - k0);
+                    prefetch_l2(p.rho + (size_t)rn * nr + k0, cells);
+                    prefetch_l2(p.tdust + (size_t)rn * nr + k0, cells);
                 }
             }
-        } else if (pf && lane == 0 && half == 0 && wr + step < wr_end) {
+        } else if (lane == 0 && half == 0 && wr + step < wr_end) {
             const unsigned r0 = (wr + step) * R;
             if (r0 < p.nrays) {
                 const unsigned nrs = p.nrays - r0 < (unsigned)R ? p.nrays - r0 : (unsigned)R;
-                const unsigned bytes = nrs * (unsigned)nr * 4u;
-                prefetch_l2(p.rho + (size_t)r0 * nr, bytes);
-                prefetch_l2(p.tdust + (size_t)r0 * nr, bytes);
+                prefetch_l2(p.rho + (size_t)r0 * nr, nrs * (unsigned)nr);
+                prefetch_l2(p.tdust + (size_t)r0 * nr, nrs * (unsigned)nr);
             }
         }
 
@@ -602,6 +657,22 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
                     *reinterpret_cast<float2 *>(p.a + base + j) = acc[j / 2];
                 }
             }
+        } else if constexpr (ST) {
+            __syncwarp();  // every lane has read its inputs
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                const int i = skew(s_idx0 + j);
+                s_one[i] = (j & 1) ? qv[j / 2].y : qv[j / 2].x;
+                s_two[i] = (j & 1) ? acc[j / 2].y : acc[j / 2].x;
+            }
+            __syncwarp();
+            each_run(wr, ch, [&](int i, size_t m) {
+                p.q[m] = s_one[i];
+                p.a[m] = s_two[i];
+            });
+            const bool first = s_one == s_stage;
+            s_one = first ? s_stage + 66 * C : s_stage;
+            s_two = s_one + 33 * C;
         } else {
 #pragma unroll
             for (int j = 0; j < C; ++j) {
@@ -618,7 +689,7 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
 
 // The kernel over all rays of one grid (persistent CTAs striding over the warp-slots),
 // then the CTA's energy partial.
-template <int C, int W, int MODE, int MINB, int G, int P, bool TW, bool LUT, bool MC>
+template <int C, int W, int MODE, int MINB, int G, int P, bool TW, bool LUT, bool MC, bool ST>
 __global__ void __launch_bounds__(W * 32, MINB) k_ray(const TraceArgs p)
 {
     using ESum = KahanSum;
@@ -632,6 +703,8 @@ __global__ void __launch_bounds__(W * 32, MINB) k_ray(const TraceArgs p)
     // chunked form: the radial constants of every chunk after the bin tables
     float2 *s_dr_mc = reinterpret_cast<float2 *>(s_mom + 2 * p.nnu_pad);
     float4 *s_gqa_mc = reinterpret_cast<float4 *>(s_dr_mc + (MC ? ray_chunk_pairs(C, G, p.nr) : 0));
+    // and the warps' stages where the fields need them
+    float *s_stage = reinterpret_cast<float *>(s_gqa_mc + (MC ? ray_chunk_pairs(C, G, p.nr) : 0)) + warp * (ST ? ray_stage_len(C) : 0);
     __shared__ ESum s_red[W][2];
     ray_tables<C, W, P>(p, G, rs, s_kap, s_nu, s_mom);
     if constexpr (MC) ray_tables_mc<C, W, G>(p, s_dr_mc, s_gqa_mc);
@@ -642,8 +715,8 @@ __global__ void __launch_bounds__(W * 32, MINB) k_ray(const TraceArgs p)
     eesc.zero();
     const unsigned slots = (p.nrays + R - 1) / R;
     constexpr int WG = W / P;  // ray groups per CTA
-    ray_slots<C, W, MODE, G, P, TW, LUT, MC>(p, blockIdx.x * WG + warp / P, slots, gridDim.x * WG, rs, s_kap, s_nu,
-                                             s_mom, eabs, eesc, s_dr_mc, s_gqa_mc);
+    ray_slots<C, W, MODE, G, P, TW, LUT, MC, ST>(p, blockIdx.x * WG + warp / P, slots, gridDim.x * WG, rs, s_kap, s_nu,
+                                             s_mom, eabs, eesc, s_stage, s_dr_mc, s_gqa_mc);
 
     for (int o = 16; o > 0; o >>= 1) {
         eabs.add(eabs.shfl_xor(o));
@@ -658,14 +731,20 @@ __global__ void __launch_bounds__(W * 32, MINB) k_ray(const TraceArgs p)
     }
 }
 
-template <int C, int W, int MODE, int MINB, int G, int P, bool TW, bool LUT, bool MC = false>
-cudaError_t launch_ray_g(const TraceArgs &a, cudaStream_t stream, unsigned *grid_out, unsigned max_grid)
+template <int C, int W, int MODE, int MINB, int G, int P, bool TW, bool LUT, bool MC, bool ST>
+cudaError_t launch_ray_st(const TraceArgs &a, cudaStream_t stream, unsigned *grid_out, unsigned max_grid)
 {
     constexpr int R = 32 / G;
-    const size_t smem = ray_bin_smem(a.nnu_pad) + 16 + (MC ? (size_t)ray_chunk_pairs(C, G, a.nr) * (8 + 16) : 0);
-    auto kern = k_ray<C, W, MODE, MINB, G, P, TW, LUT, MC>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = ray_bin_smem(a.nnu_pad) + 16 + (MC ? (size_t)ray_chunk_pairs(C, G, a.nr) * (8 + 16) : 0) +
+                        (ST ? sizeof(float) * W * ray_stage_len(C) : 0);
+    auto kern = k_ray<C, W, MODE, MINB, G, P, TW, LUT, MC, ST>;
+    // beyond 48 KB with the static part (at most 24 KB); one limit for every caller, so that another
+    // thread's smaller launch cannot lower it (the largest: the chunked form's radial constants of
+    // kMaxChunkedNr cells, 49 KB, the bin tables, 7 KB, and the stages, 34 KB)
+    constexpr size_t kMaxSmem = 96 * 1024;
+    if (smem > 24 * 1024) {
+        if (smem > kMaxSmem) return cudaErrorInvalidValue;
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem);
         if (e != cudaSuccess) return e;
     }
     int dev = 0, nsm = 0, per_sm = 0;
@@ -682,6 +761,15 @@ cudaError_t launch_ray_g(const TraceArgs &a, cudaStream_t stream, unsigned *grid
     kern<<<grid, W * 32, smem, stream>>>(a);
     *grid_out = grid;
     return cudaGetLastError();
+}
+
+template <int C, int W, int MODE, int MINB, int G, int P, bool TW, bool LUT, bool MC = false>
+cudaError_t launch_ray_g(const TraceArgs &a, cudaStream_t stream, unsigned *grid_out, unsigned max_grid)
+{
+    if constexpr (ray_staged(C, G)) {
+        if (!ray_vec(a, C)) return launch_ray_st<C, W, MODE, MINB, G, P, TW, LUT, MC, true>(a, stream, grid_out, max_grid);
+    }
+    return launch_ray_st<C, W, MODE, MINB, G, P, TW, LUT, MC, false>(a, stream, grid_out, max_grid);
 }
 
 }  // namespace

@@ -11,20 +11,9 @@ namespace {
 // radial table staged in shared memory up to this many cells per ray
 constexpr int kRtabSmemMax = 1024;
 
-// Shared-memory index with one padding word per 32: lanes that own C consecutive
-// cells read at stride C, which this skew spreads over distinct banks.
-__device__ __forceinline__ int skew(int i) { return i + (i >> 5); }
 // (rounded up to 4 floats so the float4 tables after the buffers stay 16-byte aligned)
 template <int T>
 constexpr int skewed_len() { return (T + T / 32 + 1 + 3) & ~3; }
-
-__device__ __forceinline__ void cp_async4(void *smem_dst, const void *gmem_src)
-{
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 
 // energy sums of the tile kernel: compensated FP32 (the FP64 pipe of this part is
 // far narrower than its FP32 pipes), plain FP64 in the FP64 mode
