@@ -187,37 +187,10 @@ int all_shapes(const rt_ctx *c, Shape *out, int max_out)
     return n;
 }
 
-Shape default_shape(const rt_ctx *c)
+// the widest tile that still gives every SM several tiles; on a small grid the one with the most
+// tiles, then the smaller
+Shape default_tile(const rt_ctx *c)
 {
-    const bool tw = use_tw(c);
-    if (c->n_t > 0 && !tw) {  // temperature-dependent table: the fewest cells per lane that hold a ray
-        Shape ts[16];
-        const int n = use_r2(c) ? rt::tdep2_shapes(c->rk, c->nr, ts, 16) : rt::tdep_shapes(c->nr, ts, 16);
-        int bi = -1;
-        for (int i = 0; i < n; ++i)
-            if (bi < 0 || ts[i].cells_per_lane < ts[bi].cells_per_lane ||
-                (ts[i].cells_per_lane == ts[bi].cells_per_lane && ts[i].min_blocks > ts[bi].min_blocks))
-                bi = i;
-        return bi >= 0 ? ts[bi] : Shape{rt::kKindRay, 0, 0, 0};
-    }
-    {
-        std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_tune_cache.find(std::make_tuple(c->precision, c->nr, c->nrays, c->sc_h.nnu_pad, table_kind(c)));
-        if (it != g_tune_cache.end()) return it->second;
-    }
-    // Prefer the warp-per-ray kernel with the fewest cells per lane when the rays
-    // fill at least 3/4 of the G C cells of their lane segment; else the widest tile
-    // that still gives every SM several tiles.
-    if (c->precision != RT_FP64) {
-        Shape rs[32];
-        const int nrs = tw ? rt::ray_shapes_tw(c->precision, c->nr, rs, 32) : rt::ray_shapes(c->precision, c->nr, rs, 32);
-        int bi = -1;
-        for (int i = 0; i < nrs; ++i)
-            if (4 * c->nr >= 3 * rt::ray_cells_held(rs[i].cells_per_lane, c->nr) &&
-                (bi < 0 || rs[i].cells_per_lane < rs[bi].cells_per_lane))
-                bi = i;
-        if (bi >= 0) return rs[bi];
-    }
     Shape cand[32];
     const int n = rt::trace_shapes(c->precision, cand, 32);
     Shape best = cand[0];
@@ -237,6 +210,53 @@ Shape default_shape(const rt_ctx *c)
         }
     }
     return best;
+}
+
+Shape default_shape(const rt_ctx *c)
+{
+    const bool tw = use_tw(c);
+    if (c->n_t > 0 && !tw) {  // temperature-dependent table: the fewest cells per lane that hold a ray,
+                              // and of its register caps the wider (the bin-pair form: 256x128x128,
+                              // full rank, 347 -> 306 us; 100x64x64 71 -> 57)
+        Shape ts[16];
+        const int n = use_r2(c) ? rt::tdep2_shapes(c->rk, c->nr, ts, 16) : rt::tdep_shapes(c->nr, ts, 16);
+        int bi = -1;
+        for (int i = 0; i < n; ++i)
+            if (bi < 0 || ts[i].cells_per_lane < ts[bi].cells_per_lane ||
+                (ts[i].cells_per_lane == ts[bi].cells_per_lane && ts[i].min_blocks < ts[bi].min_blocks))
+                bi = i;
+        return bi >= 0 ? ts[bi] : Shape{rt::kKindRay, 0, 0, 0};
+    }
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto it = g_tune_cache.find(std::make_tuple(c->precision, c->nr, c->nrays, c->sc_h.nnu_pad, table_kind(c)));
+        if (it != g_tune_cache.end()) return it->second;
+    }
+    // the warp-per-ray kernels where they serve the grid (a separable temperature table needs
+    // them: the tile kernel has no column weight), else tiles
+    if (c->precision != RT_FP64) {
+        Shape rs;
+        if (rt::ray_default(c->precision, c->nr, c->nrays, tw, &rs)) return rs;
+    }
+    return default_tile(c);
+}
+
+// The shape the surrogate's training fields are traced with: a rule of the grid alone, so that
+// the network that a set of fields and a seed give does not depend on the shape in use (the
+// shapes differ in the rounding of their last bits, which training amplifies).
+Shape training_shape(const rt_ctx *c)
+{
+    if (c->precision != RT_FP64) {
+        Shape rs[32];
+        const int n = rt::ray_shapes(c->precision, c->nr, rs, 32);
+        int bi = -1;
+        for (int i = 0; i < n; ++i)
+            if (4 * c->nr >= 3 * rt::ray_cells_held(rs[i].cells_per_lane, c->nr) &&
+                (bi < 0 || rs[i].cells_per_lane < rs[bi].cells_per_lane))
+                bi = i;
+        if (bi >= 0) return rs[bi];
+    }
+    return default_tile(c);
 }
 
 int finalize(rt_ctx *c)
@@ -513,6 +533,12 @@ unsigned long long &ctx_temp_fingerprint(rt_ctx *c) { return c->temp_fp; }
 FldState *&ctx_fld(rt_ctx *c) { return c->fld; }
 
 int ctx_fail(rt_ctx *c, int status, const std::string &msg) { return fail(c, status, msg); }
+
+int trace_training(rt_ctx *c, const float *rho, const float *td, float *q, float *a)
+{
+    const int st = check_call(c, rho, td, q, a);
+    return st == RT_OK ? trace(c, rho, td, q, a, training_shape(c)) : st;
+}
 }  // namespace rt
 
 extern "C" {

@@ -182,6 +182,9 @@ int ray_shapes(int precision, int nr, Shape *out, int max_out);  // ray kernel, 
 int ray_shapes_tw(int precision, int nr, Shape *out, int max_out);
 // ray-kernel shapes compiled with the lookup-table comparator
 int ray_shapes_lut(int precision, int nr, Shape *out, int max_out);
+// the warp-per-ray (or chunked) shape of a context that was not autotuned (tw: with the column
+// weight); false: the tile kernel
+bool ray_default(int precision, int nr, long long nrays, bool tw, Shape *out);
 // shapes of the chunked ray kernel (8 C < nr <= kMaxChunkedNr), rt_ray_mc.cu
 int ray_shapes_mc(int precision, int nr, Shape *out, int max_out);
 cudaError_t launch_ray_mc_shape(int precision, Shape s, const TraceArgs &args, cudaStream_t stream,
@@ -264,6 +267,8 @@ struct FldState;
 FldState *&ctx_fld(rt_ctx *c);
 void fld_free(FldState *s);
 int ctx_fail(rt_ctx *c, int status, const std::string &msg);
+// rt_irradiate on one of the surrogate's training fields, in a shape that depends on the grid alone
+int trace_training(rt_ctx *c, const float *rho, const float *td, float *q, float *a);
 
 // Set-up kernels (rt_setup.cu)
 // order_dev (may be null) receives the original index of every kappa-sorted bin

@@ -80,6 +80,48 @@ int ray_shapes_lut(int precision, int nr, Shape *out, int max_out)
     return n;
 }
 
+// The warp-per-ray shape of a context that was not autotuned; false where the tile kernel serves it
+// better (rays beyond 512 cells, few of them) or no such shape applies. Timed over 79 bins,
+// tau550 = 0.1 to 100, nr 64 to 4096, 32 to 131072 rays:
+//   - a lane's fixed work and the whole-warp decisions want many cells per lane, masked lanes want
+//     few: the cost is cells held / nr, weighted per shape (256x128x256, tau550 = 10: C = 8 62 us,
+//     C = 16 65, C = 4 with two warps per ray 99; 384x128x128, tau550 = 1: C = 12 32 us, C = 6 with
+//     two warps 48, C = 16 46);
+//   - grids that do not give every SM two warps are latency-bound: the fewest cells per lane
+//     (64x32x1: C = 2 7.3 us, C = 8 7.5, C = 16 9.3);
+//   - longer rays: the chunked form, which needs some 1500 rays to fill the SMs (1024x128x16:
+//     31 us against the tiles' 58; 1024x16x16: tiles 22 us).
+bool ray_default(int precision, int nr, long long nrays, bool tw, Shape *out)
+{
+    Shape s[32];
+    const int n = tw ? ray_shapes_tw(precision, nr, s, 32) : ray_shapes(precision, nr, s, 32);
+    if (n < 1) {
+        if (tw || precision == RT_FP64 || nrays < 1536) return false;
+        const int m = ray_shapes_mc(precision, nr, s, 32);
+        for (int i = 0; i < m; ++i)
+            if (s[i].cells_per_lane == 16 && s[i].min_blocks == 4) {
+                *out = s[i];
+                return true;
+            }
+        return false;
+    }
+    auto weight = [](int c) { return c <= 2 ? 2.1 : c <= 4 ? 1.3 : c <= 6 ? 1.35 : c <= 12 ? 1.0 : 1.07; };
+    int bi = 0;
+    double best = 0.0;
+    for (int i = 0; i < n; ++i) {
+        const int c = s[i].cells_per_lane, held = ray_cells_held(c, nr);
+        double cost = (double)held / nr * weight(c) * (held > 32 * c ? 1.15 : 1.0);  // two warps per ray
+        if (nrays * held < 304LL * 32 * c) cost = 100.0 + c;
+        // of one shape's register caps the first but for the two of C = 16 (4 CTAs per SM)
+        if (i == 0 || cost < best || (cost == best && c == 16 && s[bi].cells_per_lane == 16)) {
+            best = cost;
+            bi = i;
+        }
+    }
+    *out = s[bi];
+    return true;
+}
+
 cudaError_t launch_ray_shape(int precision, Shape s, const TraceArgs &args, cudaStream_t stream,
                              unsigned *grid_out, unsigned max_grid)
 {

@@ -88,14 +88,11 @@ __device__ __forceinline__ float ex_lg2(float x)
     return y;
 }
 
-// Ask L2 for n floats from p, less what lies outside whole 16-byte units: a hint with
+// Ask L2 for `bytes` bytes from p (16-byte aligned, a multiple of 16): a hint with
 // no completion to wait for.
-__device__ __forceinline__ void prefetch_l2(const float *p, unsigned n)
+__device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes)
 {
-    const size_t a = (reinterpret_cast<size_t>(p) + 15) & ~size_t(15);
-    const size_t e = (reinterpret_cast<size_t>(p) + 4 * (size_t)n) & ~size_t(15);
-    if (e > a)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((unsigned)(e - a)) : "memory");
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 // Fields whose rays do not start on vector boundaries (nr not a multiple of the vector, or
@@ -274,6 +271,31 @@ __device__ __forceinline__ void ray_tables_mc(const TraceArgs &p, float2 *s_dr, 
     }
 }
 
+// The warp's cells of chunk ch of warp-slot wr, run by run (a segment's cells are one run of
+// memory): f(index in the stage, index in the fields)
+template <int C, int G, class F>
+__device__ __forceinline__ void each_run(const TraceArgs &p, unsigned wr, int ch, int half, int lane, const F &f)
+{
+    constexpr int R = 32 / G;
+#pragma unroll
+    for (int s = 0; s < R; ++s) {
+        const unsigned r = wr * R + s;
+        const int k0 = (ch * G + half * 32) * C, len = r < p.nrays ? min(G * C, p.nr - k0) : 0;
+        const size_t m0 = (size_t)r * p.nr + k0;
+        for (int i = lane; i < len; i += 32) f(skew(s * (G * C) + i), m0 + i);
+    }
+}
+
+// their density and temperature, on their way to the buffers at `one` and one + 33 C
+template <int C, int G>
+__device__ __forceinline__ void stage_in(const TraceArgs &p, unsigned wr, int ch, int half, int lane, float *one)
+{
+    each_run<C, G>(p, wr, ch, half, lane, [&](int i, size_t m) {
+        cp_async4(one + i, p.rho + m);
+        cp_async4(one + 33 * C + i, p.tdust + m);
+    });
+}
+
 // Warp-slots wr = wr_begin, wr_begin + step, ... (< wr_end) of grid p, R = 32 / G rays
 // each (or, with P > 1, one ray per group of P consecutive warps, which all walk the
 // same slots); the lanes' energy sums are added to eabs / eesc. TW: the table is a
@@ -321,30 +343,15 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
     const int nch = MC ? (nr + G * C - 1) / (G * C) : 1;  // chunks per ray
     // vector access needs every lane start and the field bases 4V-byte aligned
     const bool vec = !ST && ray_vec(p, C);
-    const int s_idx0 = seg * (G * C) + (lane % G) * C;  // the lane's first cell in the stage
-    float *s_one = s_stage, *s_two = s_stage + 33 * C;  // this chunk's buffers
-    // the warp's cells of one chunk, run by run (a segment's cells are one run of memory):
-    // f(index in the stage, index in the fields)
-    auto each_run = [&](unsigned wr, int ch, auto f) {
-#pragma unroll
-        for (int s = 0; s < R; ++s) {
-            const unsigned r = wr * R + s;
-            const int k0 = (ch * G + half * 32) * C, len = r < p.nrays ? min(G * C, nr - k0) : 0;
-            const size_t m0 = (size_t)r * nr + k0;
-            for (int i = lane; i < len; i += 32) f(skew(s * (G * C) + i), m0 + i);
-        }
-    };
-    auto stage_in = [&](unsigned wr, int ch, float *one, float *two) {
-        each_run(wr, ch, [&](int i, size_t m) {
-            cp_async4(one + i, p.rho + m);
-            cp_async4(two + i, p.tdust + m);
-        });
-    };
+    // a warp-slot's fields are R consecutive rays: one contiguous run per field
+    const bool pf = (nr % 4 == 0) &&
+                    ((reinterpret_cast<size_t>(p.rho) | reinterpret_cast<size_t>(p.tdust)) % 16 == 0);
     const int na = p.n_active;
     const float2 tiny2 = f2(FLT_MIN);
+    int stage_buf = 0;  // ST: the buffers of this chunk
     if constexpr (ST) {
         __syncwarp();  // a previous range of slots may still be leaving the buffers
-        if (wr_begin < wr_end) stage_in(wr_begin, 0, s_one, s_two);
+        if (wr_begin < wr_end) stage_in<C, G>(p, wr_begin, 0, half, lane, s_stage);
     }
 
     for (unsigned wr = wr_begin; wr < wr_end; wr += step) {
@@ -364,18 +371,17 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
             cp_async_wait_all();
             __syncwarp();
             // cells past the ray's end: no density, no dust (their column is 0 with any t_sub)
+            const float *one = s_stage + stage_buf * (66 * C), *two = one + 33 * C;
 #pragma unroll
             for (int j = 0; j < C; j += 2) {
-                const int i0 = skew(s_idx0 + j), i1 = skew(s_idx0 + j + 1);
-                rho2[j / 2] = make_float2(j < nv ? s_one[i0] : 0.0f, j + 1 < nv ? s_one[i1] : 0.0f);
-                td2[j / 2] = make_float2(j < nv ? s_two[i0] : INFINITY, j + 1 < nv ? s_two[i1] : INFINITY);
+                const int i0 = skew(seg * (G * C) + (lane % G) * C + j), i1 = skew(seg * (G * C) + (lane % G) * C + j + 1);
+                rho2[j / 2] = make_float2(j < nv ? one[i0] : 0.0f, j + 1 < nv ? one[i1] : 0.0f);
+                td2[j / 2] = make_float2(j < nv ? two[i0] : INFINITY, j + 1 < nv ? two[i1] : INFINITY);
             }
             // the next chunk into the other buffers (their outputs left before the barrier)
             const unsigned wn = ch + 1 < nch ? wr : wr + step;
-            if (wn < wr_end) {
-                const bool first = s_one == s_stage;
-                stage_in(wn, ch + 1 < nch ? ch + 1 : 0, first ? s_stage + 66 * C : s_stage, first ? s_stage + 99 * C : s_stage + 33 * C);
-            }
+            if (wn < wr_end)
+                stage_in<C, G>(p, wn, ch + 1 < nch ? ch + 1 : 0, half, lane, s_stage + (stage_buf ^ 1) * (66 * C));
         } else if (vec && nv == C) {
 #pragma unroll
             for (int j = 0; j < C; j += V) {
@@ -407,22 +413,23 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
         // last), the same distance ahead as one slot of the one-chunk form
         if constexpr (ST) {
         } else if constexpr (MC) {
-            if (lane % G == 0) {
+            if (pf && lane % G == 0) {
                 const bool last = ch + 1 == nch;
                 const unsigned rn = last ? (wr + step) * R + seg : ray;
                 const int k0 = last ? 0 : (ch + 1) * G * C;
                 if ((!last || wr + step < wr_end) && rn < p.nrays) {
-                    const unsigned cells = (unsigned)min(G * C, nr - k0);
-                    prefetch_l2(p.rho + (size_t)rn * nr + k0, cells);
-                    prefetch_l2(p.tdust + (size_t)rn * nr + k0, cells);
+                    const unsigned bytes = (unsigned)min(G * C, nr - k0) * 4u;
+                    prefetch_l2(p.rho + (size_t)rn * nr + k0, bytes);
+                    prefetch_l2(p.tdust + (size_t)rn * nr + k0, bytes);
                 }
             }
-        } else if (lane == 0 && half == 0 && wr + step < wr_end) {
+        } else if (pf && lane == 0 && half == 0 && wr + step < wr_end) {
             const unsigned r0 = (wr + step) * R;
             if (r0 < p.nrays) {
                 const unsigned nrs = p.nrays - r0 < (unsigned)R ? p.nrays - r0 : (unsigned)R;
-                prefetch_l2(p.rho + (size_t)r0 * nr, nrs * (unsigned)nr);
-                prefetch_l2(p.tdust + (size_t)r0 * nr, nrs * (unsigned)nr);
+                const unsigned bytes = nrs * (unsigned)nr * 4u;
+                prefetch_l2(p.rho + (size_t)r0 * nr, bytes);
+                prefetch_l2(p.tdust + (size_t)r0 * nr, bytes);
             }
         }
 
@@ -659,20 +666,19 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
             }
         } else if constexpr (ST) {
             __syncwarp();  // every lane has read its inputs
+            float *one = s_stage + stage_buf * (66 * C), *two = one + 33 * C;
 #pragma unroll
             for (int j = 0; j < C; ++j) {
-                const int i = skew(s_idx0 + j);
-                s_one[i] = (j & 1) ? qv[j / 2].y : qv[j / 2].x;
-                s_two[i] = (j & 1) ? acc[j / 2].y : acc[j / 2].x;
+                const int i = skew(seg * (G * C) + (lane % G) * C + j);
+                one[i] = (j & 1) ? qv[j / 2].y : qv[j / 2].x;
+                two[i] = (j & 1) ? acc[j / 2].y : acc[j / 2].x;
             }
             __syncwarp();
-            each_run(wr, ch, [&](int i, size_t m) {
-                p.q[m] = s_one[i];
-                p.a[m] = s_two[i];
+            each_run<C, G>(p, wr, ch, half, lane, [&](int i, size_t m) {
+                p.q[m] = one[i];
+                p.a[m] = two[i];
             });
-            const bool first = s_one == s_stage;
-            s_one = first ? s_stage + 66 * C : s_stage;
-            s_two = s_one + 33 * C;
+            stage_buf ^= 1;
         } else {
 #pragma unroll
             for (int j = 0; j < C; ++j) {

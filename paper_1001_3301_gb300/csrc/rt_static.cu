@@ -98,19 +98,11 @@ int fail(int status, const std::string &msg)
     return status;
 }
 
-// Warp-per-ray kernel when the rays fill 3/4 of the cells its lanes hold, else an 8-cell tile.
-rt::Shape pick_shape(int precision, int nr)
+// The warp-per-ray kernels where they serve the grid, else an 8-cell tile.
+rt::Shape pick_shape(int precision, int nr, long long nrays)
 {
     rt::Shape s[32];
-    if (precision != RT_FP64) {
-        const int n = rt::ray_shapes(precision, nr, s, 32);
-        int bi = -1;
-        for (int i = 0; i < n; ++i)
-            if (4 * nr >= 3 * rt::ray_cells_held(s[i].cells_per_lane, nr) &&
-                (bi < 0 || s[i].cells_per_lane < s[bi].cells_per_lane))
-                bi = i;
-        if (bi >= 0) return s[bi];
-    }
+    if (precision != RT_FP64 && rt::ray_default(precision, nr, nrays, false, &s[0])) return s[0];
     const int n = rt::trace_shapes(precision, s, 32);
     for (int i = 0; i < n; ++i)
         if (s[i].cells_per_lane == 8 && s[i].warps == 4) return s[i];
@@ -189,7 +181,7 @@ extern "C" int rt_irradiate_static(const rt_grid_desc *g, double t_star, double 
     RT_SCK(cudaStreamSynchronize(stream));
 
     // the tracer (one launch: the limits keep nrays (nr + 1) below the 31-bit range)
-    const rt::Shape shape = pick_shape(g->precision, g->nr);
+    const rt::Shape shape = pick_shape(g->precision, g->nr, nrays);
     rt::TraceArgs args;
     args.rho = rho;
     args.tdust = t_dust;

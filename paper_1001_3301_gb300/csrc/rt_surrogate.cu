@@ -1511,7 +1511,7 @@ int rt_surrogate_train(rt_ctx *ctx, const rt_train_cfg *cfg, const float *const 
     // pass 0: eligible cells of every grid (the exact tracer judges each cell)
     long long eligible = 0;
     for (int gi = 0; gi < ngrids && rc == RT_OK; ++gi) {
-        rc = rt_irradiate(ctx, rho[gi], t_dust[gi], q, a, nullptr);
+        rc = trace_training(ctx, rho[gi], t_dust[gi], q, a);
         if (rc != RT_OK) break;
         ca.pass = 0;
         ca.rho = rho[gi];
@@ -1553,7 +1553,7 @@ int rt_surrogate_train(rt_ctx *ctx, const rt_train_cfg *cfg, const float *const 
         }
         cudaMemsetAsync(base, 0, sizeof(long long) * 2, st);
         for (int gi = 0; gi < ngrids && rc == RT_OK; ++gi) {
-            rc = rt_irradiate(ctx, rho[gi], t_dust[gi], q, a, nullptr);
+            rc = trace_training(ctx, rho[gi], t_dust[gi], q, a);
             if (rc != RT_OK) break;
             ca.rho = rho[gi];
             ca.tdust = t_dust[gi];
