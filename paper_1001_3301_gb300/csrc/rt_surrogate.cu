@@ -522,7 +522,29 @@ __global__ void k_moments(const float *Y, long long n, double *out)
 // ---------------------------------------------------------------------------
 constexpr int kInfThreads = 256;
 constexpr uint32_t kSmW2 = 0, kSmH1hi = 32768, kSmH1lo = 65536, kSmW1 = 98304;
+constexpr uint32_t kTmemCols = 256;  // the two layers' accumulators, 128 columns each (two CTAs per SM)
 constexpr uint32_t kSmDyn = 106496;  // the feature rows (8 KB) alias the start of H1lo
+
+// SiLU of two pre-activations, both reciprocals from one: 1 / s0 = s1 / (s0 s1). MUFU is what
+// bounds the network (ex2 at 32 and rcp at 16 per SM and clock), and a pair this way takes 2 of one
+// and 1 of the other instead of 2 and 2; the rest runs packed. e^-z is cut at 2^62 (z = -43, where
+// SiLU is below 1e-17) so that the product stays finite.
+__device__ __forceinline__ float2 silu_pair(float2 z)
+{
+    const float2 t = __fmul2_rn(z, f2(-1.4426950408889634f));
+    const float2 s = __fadd2_rn(make_float2(sur::ex2f(fminf(t.x, 62.0f)), sur::ex2f(fminf(t.y, 62.0f))), f2(1.0f));
+    const float r = sur::rcpf(s.x * s.y);
+    return __fmul2_rn(z, __fmul2_rn(make_float2(s.y, s.x), f2(r)));
+}
+
+// SiLU of two first-layer pre-activations, as (hi, lo) BF16 pairs that sum to it
+__device__ __forceinline__ void act1_pair_infer(float z0, float z1, uint32_t &hi, uint32_t &lo)
+{
+    const float2 h = silu_pair(make_float2(z0, z1));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(hi) : "f"(h.y), "f"(h.x));
+    const float2 d = __fadd2_rn(h, make_float2(-__uint_as_float(hi << 16), -__uint_as_float(hi & 0xffff0000u)));
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(lo) : "f"(d.y), "f"(d.x));
+}
 
 struct SurNet {
     const uint4 *w1t;  // [512] 16-byte groups: W1b^T in the K-major tensor-core layout (128 x 32)
@@ -532,7 +554,7 @@ struct SurNet {
     sur::FeatConst fc;
 };
 
-struct MlpSmem {
+struct alignas(16) MlpSmem {
     float b2[kHid], w3[kHid];
     float part[2][kHid];
     uint64_t bar;
@@ -549,7 +571,7 @@ __device__ void mlp_load(unsigned char *dsm, MlpSmem &S, const SurNet &net)
         S.w3[tid] = net.master[sur::kOffW3 + tid];
     }
     if ((tid >> 5) == 0) {
-        umma::tmem_alloc(&S.taddr, 128);
+        umma::tmem_alloc(&S.taddr, kTmemCols);
         umma::tmem_relinquish();
     }
     if (tid == 0) umma::mbar_init(&S.bar, 1);
@@ -563,7 +585,7 @@ __device__ void mlp_release(MlpSmem &S)
 {
     umma::fence_before_sync();
     __syncthreads();
-    if ((threadIdx.x >> 5) == 0) umma::tmem_dealloc(S.taddr, 128);
+    if ((threadIdx.x >> 5) == 0) umma::tmem_dealloc(S.taddr, kTmemCols);
 }
 
 // The network on 128 rows: threads 0..127 supply row r = tid's features; y is
@@ -601,6 +623,8 @@ __device__ bool mlp_tile(unsigned char *dsm, MlpSmem &S, uint32_t &phase, const 
     fence_after_sync();
 
     const uint32_t lane_addr = taddr + ((uint32_t)((warp & 3) * 32) << 16);
+    // the second layer's products start on the first half of the columns (K slices 2 c2 and 4 + 2 c2
+    // of 16 columns, on) while the epilogue works on the rest
 #pragma unroll
     for (int c2 = 0; c2 < 2; ++c2) {
         const int col0 = 64 * half + 32 * c2;
@@ -610,40 +634,48 @@ __device__ bool mlp_tile(unsigned char *dsm, MlpSmem &S, uint32_t &phase, const 
         for (int j8 = 0; j8 < 4; ++j8) {
             uint32_t hi[4], lo[4];
 #pragma unroll
-            for (int p = 0; p < 4; ++p) sur::act1_pair(v[8 * j8 + 2 * p], v[8 * j8 + 2 * p + 1], hi[p], lo[p]);
+            for (int p = 0; p < 4; ++p) act1_pair_infer(v[8 * j8 + 2 * p], v[8 * j8 + 2 * p + 1], hi[p], lo[p]);
             const uint32_t off = kmajor_offset(r, col0 + 8 * j8, 128);
             *reinterpret_cast<uint4 *>(dsm + kSmH1hi + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
             *reinterpret_cast<uint4 *>(dsm + kSmH1lo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
-    }
-    fence_async_smem();
-    fence_before_sync();
-    __syncthreads();
-    if (tid == 0) {
-        fence_after_sync();
-        for (int s = 0; s < 8; ++s)
-            mma_bf16(taddr, desc_kmajor(smem_u32(dsm + kSmH1hi + s * 4096)),
-                     desc_kmajor(smem_u32(dsm + kSmW2 + s * 4096)), idesc, s > 0 ? 1u : 0u);
-        for (int s = 0; s < 8; ++s)
-            mma_bf16(taddr, desc_kmajor(smem_u32(dsm + kSmH1lo + s * 4096)),
-                     desc_kmajor(smem_u32(dsm + kSmW2 + s * 4096)), idesc, 1u);
-        mma_commit(&S.bar);
+        fence_async_smem();
+        fence_before_sync();
+        __syncthreads();
+        if (tid == 0) {
+            fence_after_sync();
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int sl = 4 * (q >> 1) + 2 * c2 + (q & 1);
+                const uint64_t bd = desc_kmajor(smem_u32(dsm + kSmW2 + sl * 4096));
+                mma_bf16(taddr + 128u, desc_kmajor(smem_u32(dsm + kSmH1hi + sl * 4096)), bd, idesc, c2 + q > 0 ? 1u : 0u);
+                mma_bf16(taddr + 128u, desc_kmajor(smem_u32(dsm + kSmH1lo + sl * 4096)), bd, idesc, 1u);
+            }
+            if (c2 == 1) mma_commit(&S.bar);
+        }
     }
     ok = mbar_wait_bounded(&S.bar, phase, kMaxPolls);
     phase ^= 1u;
     if (!__syncthreads_and(ok)) return false;
     fence_after_sync();
 
-    float part = 0.0f;
+    float2 part2 = f2(0.0f);
 #pragma unroll
     for (int c2 = 0; c2 < 2; ++c2) {
         const int col0 = 64 * half + 32 * c2;
         float v[32];
-        tmem_ld32(lane_addr + (uint32_t)col0, v);
+        tmem_ld32(lane_addr + 128u + (uint32_t)col0, v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) part = fmaf(sur::silu(v[j] + S.b2[col0 + j]), S.w3[col0 + j], part);
+        for (int j = 0; j < 32; j += 4) {
+            const float4 b = *reinterpret_cast<const float4 *>(S.b2 + col0 + j);
+            const float4 w = *reinterpret_cast<const float4 *>(S.w3 + col0 + j);
+            part2 = __ffma2_rn(silu_pair(__fadd2_rn(make_float2(v[j], v[j + 1]), make_float2(b.x, b.y))),
+                               make_float2(w.x, w.y), part2);
+            part2 = __ffma2_rn(silu_pair(__fadd2_rn(make_float2(v[j + 2], v[j + 3]), make_float2(b.z, b.w))),
+                               make_float2(w.z, w.w), part2);
+        }
     }
-    S.part[half][r] = part;
+    S.part[half][r] = part2.x + part2.y;
     fence_before_sync();
     __syncthreads();
     y = S.part[0][r] + S.part[1][r] + b3;
@@ -686,17 +718,45 @@ __global__ void __launch_bounds__(kInfThreads, 1) k_sur_eval(const SurNet net, c
     mlp_release(S);
 }
 
-// exact per-bin sum of one cell (Eqs. 17, 31-32; the rho -> 0 limit for dN == 0):
-// acc = sum_i 2^(nk_i N + lf_i) (1 - e^{-kappa_i dN}), and sum_i kappa_i 2^(...)
-__device__ __forceinline__ void exact_cell(const float2 *s_nu, const float *s_kap, int na, float n_in, float dn,
-                                           float &acc, float &acc0)
+// The exact sums of a warp's cells (Eqs. 17, 31-32; the rho -> 0 limit for dN == 0) over the bins
+// of one of two halves: acc = sum_i 2^(nk_i N + lf_i) (1 - e^{-kappa_i dN}) and, where dN = 0,
+// acc0 = sum_i kappa_i 2^(...). The bins thin up to the warp's largest column are one power series
+// (set-up rows, as in the tracer; first half), the others alternate between the halves, with the
+// 8-term series below kappa dN = 1/2 (first omitted term 1e-8 of the value) and 1 - ex2 above (ex2
+// error amplified at most 1.6-fold). (One thread per cell over every bin with expm1f took 680 us of
+// the 256x128x128 grid's 1590.)
+__device__ __forceinline__ void exact_cells(const float2 *s_nu, const float *s_kap, const float *rows, int na,
+                                            int half, int lane, bool need, float n_in, float dn, float &acc, float &acc0)
 {
-    acc = 0.0f;
-    acc0 = 0.0f;
-    for (int i = 0; i < na; ++i) {
-        const float e = sur::ex2f(fmaf(s_nu[i].x, n_in, s_nu[i].y));
-        if (dn > 0.0f) acc = fmaf(e, -expm1f(s_nu[i].x * dn * (float)kLn2), acc);
-        else acc0 = fmaf(e, s_kap[i], acc0);
+    acc = acc0 = 0.0f;
+    const float top = need ? n_in + dn : 0.0f;  // (a negative or NaN column, invalid input, counts as 0)
+    const float nmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(top, 0.0f))));
+    int bt = 0;
+    for (int c0 = 0; c0 < na; c0 += 32) {
+        const int i = c0 + lane;
+        bt += __popc(__ballot_sync(0xffffffffu, i < na && -s_nu[i].x * nmax <= kThinY));
+    }
+    const bool any_zero = __any_sync(0xffffffffu, need && dn == 0.0f);
+    if (half == 0 && bt > 0) {
+        const float *row = rows + bt * kThinStride;
+        const float s = __ldg(row), c = s * n_in, a = fmaf(s, dn, c);
+        float dd = __ldg(row + kThinTerms), pc = fmaf(dd, c, __ldg(row + kThinTerms - 1));
+#pragma unroll
+        for (int k = kThinTerms - 2; k >= 1; --k) {
+            dd = fmaf(dd, a, pc);
+            pc = fmaf(pc, c, __ldg(row + k));
+        }
+        acc0 = s * fmaf(dd, a, pc);
+        acc = dn * acc0;
+    }
+    for (int i = bt + half; i < na; i += 2) {
+        const float2 e = s_nu[i];
+        const float g = sur::ex2f(fmaf(e.x, n_in, e.y)), y = e.x * dn;
+        float t = (float)taylor_coeff(7);
+#pragma unroll
+        for (int k = 6; k >= 0; --k) t = fmaf(t, y, (float)taylor_coeff(k));
+        acc = fmaf(g, y > -0.72134752f ? y * t : 1.0f - sur::ex2f(y), acc);
+        if (any_zero) acc0 = fmaf(g, s_kap[i], acc0);
     }
 }
 
@@ -726,6 +786,12 @@ struct SurRayArgs {
 // of the ray-major field, in order, carrying the column density of a ray that
 // continues into the next tile. Per tile: masked column dN (Eq. 19), segmented
 // compensated scan -> N_in, features, the network, gate or judge, outputs.
+// Bound by latency between barriers: two CTAs per SM (126 registers; the two accumulators take 256
+// of the 512 TMEM columns), issue 47 %, MUFU 38 %, tensor pipe 19 % busy. 256x128x128 cells, gated:
+// 1590 -> 677 us, of which the network 607 us (was ~910): one reciprocal per two sigmoids (MUFU was
+// first), packed activations, the second layer's columns accumulated beside the first's so that its
+// MMA slices start while the first's epilogue runs on, the next tile's fields loaded ahead, and
+// exact_cells by both halves.
 __global__ void __launch_bounds__(kInfThreads, 2) k_sur_ray(const __grid_constant__ SurRayArgs p)
 {
     extern __shared__ __align__(1024) unsigned char dsm[];
@@ -735,6 +801,7 @@ __global__ void __launch_bounds__(kInfThreads, 2) k_sur_ray(const __grid_constan
     __shared__ uint32_t s_trust[kTrustWords];
     __shared__ KahanSum s_wv[4], s_next, s_red[8];
     __shared__ int s_wf[4];
+    __shared__ float2 s_cell[kHid], s_ex[2][kHid];  // (N_in, dN) of the cells the network does not answer; their sums
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, r = tid & 127;
     for (int i = tid; i < p.nnu_pad; i += kInfThreads) {
         s_nu[i] = make_float2(p.nu[i].nk, p.nu[i].lf);
@@ -779,6 +846,16 @@ __global__ void __launch_bounds__(kInfThreads, 2) k_sur_ray(const __grid_constan
     eesc.zero();
     double st_dust = 0, st_fb = 0, st_judged = 0, st_sum = 0, st_max = 0;
 
+    // the fields of the next tile are loaded while the network works on this one
+    float rho_n = 0.0f, td_n = 0.0f;
+    auto fetch = [&](unsigned tile) {
+        const unsigned c = tile * 128u + (unsigned)r;
+        if (tid < 128 && tile < t_end && c < p.ncells) {
+            rho_n = p.rho[c];
+            td_n = p.tdust[c];
+        }
+    };
+    fetch(t_begin);
     for (unsigned tile = t_begin; tile < t_end; ++tile) {
         const unsigned cell = tile * 128u + (unsigned)r;
         const bool valid = tid < 128 && cell < p.ncells;
@@ -789,12 +866,13 @@ __global__ void __launch_bounds__(kInfThreads, 2) k_sur_ray(const __grid_constan
         if (valid) {
             ray = p.nrdiv.div(cell);
             k = cell - ray * p.nr;
-            rho = p.rho[cell];
-            td = p.tdust[cell];
+            rho = rho_n;
+            td = td_n;
             g = __ldg(p.rtab + k);
             dust = td <= p.t_sub;
             d = dust ? rho * g.x : 0.0f;
         }
+        fetch(tile + 1u);
         const bool bad = valid && (!(rho >= 0.0f && rho <= FLT_MAX) || td != td);
         if (__any_sync(0xffffffffu, bad) && lane == 0) atomicMax(p.bad_input, p.seq);
         const bool head = !valid || k == 0u;
@@ -840,6 +918,39 @@ __global__ void __launch_bounds__(kInfThreads, 2) k_sur_ray(const __grid_constan
         }
         carry = s_next;  // written before the network's barriers
 
+        // the gate, and the exact sums of the cells outside it (all threads: two per cell)
+        bool need = false;
+        if (p.mode == 0 && dust) {
+            // an empty column (log2 0 = -inf) falls into bin 0
+            const float u = fmaxf(sur::lg2f(k550 * n_in), kTrustU0 - 1.0f);
+            const float w = fmaxf(sur::lg2f(k550 * d), kTrustV0 - 1.0f);
+            const int iu = max(0, (int)floorf((u - kTrustU0) * (1.0f / kTrustDU)));
+            const int iv = max(0, (int)floorf((w - kTrustV0) * (1.0f / kTrustDV)));
+            need = true;
+            if (iu < kTrustBins && iv < kTrustBins) {
+                const int b = iu * kTrustBins + iv;
+                need = !((s_trust[b >> 5] >> (b & 31)) & 1u);
+            }
+        }
+        float ex_acc = 0.0f, ex_acc0 = 0.0f;
+        if (__syncthreads_or(need)) {
+            if (tid < 128) s_cell[r] = make_float2(n_in, need ? fmaxf(d, 0.0f) : -1.0f);
+            __syncthreads();
+            const float2 c = s_cell[r];
+            if (__any_sync(0xffffffffu, c.y >= 0.0f)) {
+                float e1, e0;
+                const bool mine = c.y >= 0.0f;
+                exact_cells(s_nu, s_kap, p.kap + kKapTable, p.n_active, tid >> 7, lane, mine, mine ? c.x : 0.0f,
+                            mine ? c.y : 0.0f, e1, e0);
+                s_ex[tid >> 7][r] = make_float2(e1, e0);
+            }
+            __syncthreads();
+            if (need) {
+                ex_acc = s_ex[0][r].x + s_ex[1][r].x;
+                ex_acc0 = s_ex[0][r].y + s_ex[1][r].y;
+            }
+        }
+
         if (valid) {
             const float dom = __ldg(p.domega32 + ray);
             float qv = 0.0f, av = 0.0f, acc = 0.0f;
@@ -851,25 +962,11 @@ __global__ void __launch_bounds__(kInfThreads, 2) k_sur_ray(const __grid_constan
                 av = g.z * gg * k550;
                 bool use_exact = false;
                 float qx = 0.0f, ax = 0.0f;
-                if (p.mode == 0) {
-                    // an empty column (log2 0 = -inf) falls into bin 0
-                    const float u = fmaxf(sur::lg2f(k550 * n_in), kTrustU0 - 1.0f);
-                    const float w = fmaxf(sur::lg2f(k550 * d), kTrustV0 - 1.0f);
-                    const int iu = max(0, (int)floorf((u - kTrustU0) * (1.0f / kTrustDU)));
-                    const int iv = max(0, (int)floorf((w - kTrustV0) * (1.0f / kTrustDV)));
-                    bool trusted = false;
-                    if (iu < kTrustBins && iv < kTrustBins) {
-                        const int b = iu * kTrustBins + iv;
-                        trusted = (s_trust[b >> 5] >> (b & 31)) & 1u;
-                    }
-                    if (!trusted) {
-                        float e1, e0;
-                        exact_cell(s_nu, s_kap, p.n_active, n_in, d, e1, e0);
-                        acc = e1;
-                        qx = g.y * e1;
-                        ax = g.z * (d > 0.0f ? __fdividef(e1, d) : e0);
-                        use_exact = true;
-                    }
+                if (need) {
+                    acc = ex_acc;
+                    qx = g.y * ex_acc;
+                    ax = g.z * (d > 0.0f ? __fdividef(ex_acc, d) : ex_acc0);
+                    use_exact = true;
                 } else if (p.mode == 1) {
                     qx = p.q_ref[cell];
                     ax = p.a_ref[cell];
@@ -893,12 +990,18 @@ __global__ void __launch_bounds__(kInfThreads, 2) k_sur_ray(const __grid_constan
             p.q[cell] = qv;
             p.a[cell] = av;
             eabs.add(acc * dom);
-            if (k == p.nr - 1u) {  // the ray leaves the grid: escaping power (Eqs. 33-35)
-                const float ntot = incl.value();
-                float s = 0.0f;
-                for (int i = 0; i < p.n_active; ++i) s += sur::ex2f(fmaf(s_nu[i].x, ntot, s_nu[i].y));
-                eesc.add(s * dom);
-            }
+        }
+        // rays that leave the grid: escaping power (Eqs. 33-35), the warp's lanes sharing the bins
+        unsigned ends = __ballot_sync(0xffffffffu, valid && k == p.nr - 1u);
+        while (ends) {
+            const int src = __ffs(ends) - 1;
+            ends &= ends - 1u;
+            const float ntot = __shfl_sync(0xffffffffu, incl.value(), src);
+            const unsigned ray_e = __shfl_sync(0xffffffffu, ray, src);
+            float s = 0.0f;
+            for (int i = lane; i < p.n_active; i += 32) s += sur::ex2f(fmaf(s_nu[i].x, ntot, s_nu[i].y));
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) eesc.add(s * __ldg(p.domega32 + ray_e));
         }
     }
 

@@ -307,3 +307,31 @@ def test_gain_over_exact_tracer(trained, torch):
           f"{st['n_fallback'] / max(st['n_dust'], 1):.3f}, max rel err {rel.max():.2e}")
     assert rel.max() < 2 * TOL
     tr.close()
+
+
+@pytest.mark.parametrize("nr,ntheta,nphi,n_nu,tau", [
+    (3, 16, 5, 4, 1.0), (33, 12, 3, 5, 100.0), (127, 9, 3, 33, 1.0), (129, 8, 3, 78, 1e-3),
+    (64, 16, 2, 79, 1e4), (300, 5, 1, 79, 30.0)])
+def test_exact_cells_over_bins_and_columns(torch, nr, ntheta, nphi, n_nu, tau):
+    """A network whose every answer is wrong leaves the cells to the exact sums: columns from
+    all-thin (one power series) to opaque, odd and even bin counts over the two halves, rays that
+    end inside and across the tiles of 128 cells, empty and sublimated cells. Bound as for the other
+    fallback test, 2e-5; the energy balance (escaping part included) to 1e-5, as the wrong answers
+    (e^-60) of the cells below the mask leave out less than 1e-12 of L* each."""
+    w = synth.disk3d(nr, ntheta, nphi, n_nu=n_nu, tau550=tau, seed=nr)
+    rng = np.random.default_rng(nr)
+    rho, td = w.rho32().copy(), w.tdust32().copy()
+    rho[rng.random(rho.shape) < 0.1] = 0.0
+    td[rng.random(td.shape) < 0.1] = w.t_sub + 50.0
+    tr = _tracer(w)
+    tr.surrogate_set_params(_random_params(3).flat(), -60.0, 1.0)
+    q, a, st = tr.irradiate_surrogate(torch.from_numpy(rho).cuda(), torch.from_numpy(td).cuda(),
+                                      err_tol=TOL, validate=0)
+    orc = _parity.oracle_for(w, rho=rho, tdust=td)
+    mq, _ = _parity.masks(w, orc, rho=rho, tdust=td)
+    assert mq.any() and st["n_fallback"] >= mq.sum()
+    qn, an = q.double().cpu().numpy(), a.double().cpu().numpy()
+    assert np.abs(qn[mq] / orc.q_abs[mq] - 1).max() < 2e-5
+    assert np.abs(an[mq] / orc.a_rad[mq] - 1).max() < 2e-5
+    assert abs(st["rel_err"]) < 1e-5
+    tr.close()
