@@ -215,11 +215,10 @@ Shape default_tile(const rt_ctx *c)
 Shape default_shape(const rt_ctx *c)
 {
     const bool tw = use_tw(c);
-    if (c->n_t > 0 && !tw) {  // temperature-dependent table: the fewest cells per lane that hold a ray,
-                              // and of its register caps the wider (the bin-pair form: 256x128x128,
-                              // full rank, 347 -> 306 us; 100x64x64 71 -> 57)
+    if (c->n_t > 0 && !tw && !use_r2(c)) return rt::tdep_default(c->nr, c->nrays, c->sc_h.n_active);
+    if (c->n_t > 0 && !tw) {  // a low-rank table: the fewest cells per lane that hold a ray
         Shape ts[16];
-        const int n = use_r2(c) ? rt::tdep2_shapes(c->rk, c->nr, ts, 16) : rt::tdep_shapes(c->nr, ts, 16);
+        const int n = rt::tdep2_shapes(c->rk, c->nr, ts, 16);
         int bi = -1;
         for (int i = 0; i < n; ++i)
             if (bi < 0 || ts[i].cells_per_lane < ts[bi].cells_per_lane ||

@@ -205,6 +205,7 @@ cudaError_t launch_build_lut(const NuEntry *nu, const DevScalars *sc, double kre
 
 // Tracer with temperature-dependent opacity tables (rt_tdep.cu)
 int tdep_shapes(int nr, Shape *out, int max_out);
+Shape tdep_default(int nr, long long nrays, int n_active);
 cudaError_t launch_tdep(Shape s, const TraceArgs &args, const float2 *kt2, const float *tg, int n_t,
                         cudaStream_t stream, unsigned *grid_out);
 cudaError_t launch_build_tdep(int n_active, int nnu_pad, int n_t, const double *kappa_t, const int *order,

@@ -318,6 +318,244 @@ __global__ void __launch_bounds__(W * 32, MINB) k_ray_tdep(const TraceArgs p, co
     }
 }
 
+// ---------------------------------------------------------------------------
+// the bins across the lanes
+// ---------------------------------------------------------------------------
+// Eight lanes per ray (four rays per warp): lane l of a ray owns the bin pairs l, 8 + l, 16 + l, ..
+// and walks outwards in chunks of 8 cells: every bin's optical depth is a running sum in its own
+// lane, so no bin needs a warp scan, and the table rows of a cell are read by the lanes of its ray
+// as consecutive 16-byte words, whatever the temperatures (with the cells across the lanes, lanes
+// in different temperature intervals collide in the banks). A slot (8 pairs with consecutive
+// opacities) takes one class per chunk, from its largest opacity and the chunk's largest column.
+// The running sums start at lf, so that hi + lo is the exponent itself (a Kahan pair, one
+// compensated addition per chunk; inside the chunk a plain partial sum of at most 8 terms).
+constexpr int kBinLanes = 8, kBinCells = 8;  // (the lanes of a ray also hold one cell of the chunk each)
+
+// Slots [m0, m1) of one class over the chunk's cells: rows of (kappa_2p(T_j), kappa_2p+1(T_j),
+// kappa_2p(T_j+1), kappa_2p+1(T_j+1)) at kt + row[c] + the slot's offset; wt, wb the interpolation
+// weights times -rho dr log2 e, or times -log2 e for a zero-density dust cell (bit c of zm; ZERO:
+// the chunk holds one), whose sum is of g y alone (y = -kappa log2 e) and whose step does not enter
+// the column. The sums are of (1 - 2^y) / p0, p0 = -ln 2 the first Taylor coefficient: one term is y.
+template <int CLASS, bool ZERO>
+__device__ __forceinline__ void bins_chunk(int m0, int m1, const unsigned char *kt, unsigned char *state,
+                                           const int (&row)[kBinCells], const float2 (&wt)[kBinCells],
+                                           const float2 (&wb)[kBinCells], unsigned zm, float2 (&acc)[kBinCells])
+{
+    constexpr double p0 = taylor_coeff(0);
+    for (int m = m0; m < m1; ++m) {
+        float4 *sp = reinterpret_cast<float4 *>(state + m * (32 * (int)sizeof(float4)));
+        const float4 st = *sp;
+        const float2 hi = make_float2(st.x, st.y);
+        float2 part = make_float2(st.z, st.w);
+#pragma unroll
+        for (int c = 0; c < kBinCells; ++c) {
+            const float4 k = *reinterpret_cast<const float4 *>(kt + (row[c] + m * (kBinLanes * (int)sizeof(float4))));
+            const float2 y = __ffma2_rn(make_float2(k.z, k.w), wt[c], __fmul2_rn(make_float2(k.x, k.y), wb[c]));
+            const float2 g = ex2_approx2(__fadd2_rn(hi, part));
+            float2 om = y;  // (1 - 2^y) / p0
+            if constexpr (CLASS > 1) {
+                constexpr int N = CLASS <= 5 ? CLASS : 5;
+                float2 pl = f2((float)(taylor_coeff(N - 1) / p0));
+#pragma unroll
+                for (int k2 = N - 2; k2 >= 0; --k2) pl = __ffma2_rn(pl, y, f2((float)(taylor_coeff(k2) / p0)));
+                om = __fmul2_rn(y, pl);
+            }
+            if constexpr (CLASS == 6) {
+                const float2 big = __ffma2_rn(ex2_approx2(y), f2((float)(-1.0 / p0)), f2((float)(1.0 / p0)));
+                if (!(y.x > -kYSplit)) om.x = big.x;
+                if (!(y.y > -kYSplit)) om.y = big.y;
+            }
+            if constexpr (ZERO) {
+                const bool z = (zm >> c) & 1u;
+                if (z) om = y;
+                part = __ffma2_rn(y, f2(z ? 0.0f : 1.0f), part);
+            } else {
+                part = __fadd2_rn(part, y);
+            }
+            acc[c] = __ffma2_rn(g, om, acc[c]);
+        }
+        const float2 t = __fadd2_rn(hi, part);
+        const float2 rest = __ffma2_rn(__ffma2_rn(hi, f2(-1.0f), t), f2(-1.0f), part);
+        *sp = make_float4(t.x, t.y, rest.x, rest.y);
+    }
+}
+
+// every slot over the chunk, class by class (lane m holds the largest |nk| of slot m; live: the
+// slots before the first one whose exponents have all gone under)
+template <bool ZERO>
+__device__ __forceinline__ void bins_slots(int live, float km, float dmax, const unsigned char *kt,
+                                           unsigned char *state, const int (&row)[kBinCells],
+                                           const float2 (&wt)[kBinCells], const float2 (&wb)[kBinCells], unsigned zm,
+                                           float2 (&acc)[kBinCells])
+{
+    const float ym = km * dmax;
+    const int b1 = min(live, __popc(__ballot_sync(0xffffffffu, ym < kYT1)));
+    const int b2 = min(live, __popc(__ballot_sync(0xffffffffu, ym < kYT2)));
+    const int b3 = min(live, __popc(__ballot_sync(0xffffffffu, ym < kYT3)));
+    const int b5 = min(live, __popc(__ballot_sync(0xffffffffu, ym < kYSplit)));
+    bins_chunk<1, ZERO>(0, b1, kt, state, row, wt, wb, zm, acc);
+    bins_chunk<2, ZERO>(b1, b2, kt, state, row, wt, wb, zm, acc);
+    bins_chunk<3, ZERO>(b2, b3, kt, state, row, wt, wb, zm, acc);
+    bins_chunk<5, ZERO>(b3, b5, kt, state, row, wt, wb, zm, acc);
+    bins_chunk<6, ZERO>(b5, live, kt, state, row, wt, wb, zm, acc);
+}
+
+// Bound by issue (110 M warp instructions for 4.2 M cells x 79 bins, 60 % of the issue slots with 16
+// warps per SM) and by latency beside the slots: 256x128x128 cells, 79 bins, 24 temperatures 306 ->
+// 186 us, the cells-across-lanes form above spending 17 instructions per (cell, bin) where this one
+// spends 11, and 64x256x256 567 -> 164. Tried and slower: 16 or 32 lanes per ray (254, 397 us), the
+// chunk's weights in shared memory with 20-28 warps per SM (231-295), sub-chunks of 4 cells (186-208).
+template <int W, int MINB>
+__global__ void __launch_bounds__(W * 32, MINB) k_ray_tdep_bins(const TraceArgs p, const TdepTab t, int nslot)
+{
+    constexpr int L = kBinLanes, R = 32 / L;  // rays per warp
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, l = lane % L;
+    const int nr = p.nr, nt = t.n_t, np = nslot * L;  // bin pairs with padding
+    __shared__ float s_tg[kMaxTdepPoints], s_idt[kMaxTdepPoints];
+    __shared__ KahanSum s_red[W][2];
+    extern __shared__ __align__(16) unsigned char smem[];
+    float4 *s_kt = reinterpret_cast<float4 *>(smem);       // [n_t][np]
+    float4 *s_st = s_kt + nt * np;                         // [W][nslot][32] running pairs (hi, hi, lo, lo)
+    float2 *s_lf = reinterpret_cast<float2 *>(s_st + W * nslot * 32);  // [np]
+    const int na = p.n_active;
+    for (int i = tid; i < nt * np; i += W * 32) {
+        const int j = i / np, q = i - j * np;
+        const float2 a = 2 * q < na ? t.kt2[2 * q * nt + j] : make_float2(0.0f, 0.0f);
+        const float2 b = 2 * q + 1 < na ? t.kt2[(2 * q + 1) * nt + j] : make_float2(0.0f, 0.0f);
+        s_kt[i] = make_float4(a.x, b.x, a.y, b.y);
+    }
+    for (int q = tid; q < np; q += W * 32)  // (no flux: an exponent that gives 0 and stays finite)
+        s_lf[q] = make_float2(2 * q < na ? fmaxf(p.nu[2 * q].lf, -1e4f) : -1e4f,
+                              2 * q + 1 < na ? fmaxf(p.nu[2 * q + 1].lf, -1e4f) : -1e4f);
+    for (int i = tid; i < nt; i += W * 32) {
+        s_tg[i] = t.tg[i];
+        s_idt[i] = i + 1 < nt ? 1.0f / (t.tg[i + 1] - t.tg[i]) : 0.0f;
+    }
+    __syncthreads();
+
+    float4 *state = s_st + warp * nslot * 32 + lane;  // the lane's own, slot by slot
+    // the largest |nk| of slot `lane` (at most 8 slots; lanes behind them: never in a class)
+    const float km = lane < nslot ? -p.nu[min(2 * L * (lane + 1), na) - 1].nk : INFINITY;
+    KahanSum eabs, eesc;
+    eabs.zero();
+    eesc.zero();
+    for (unsigned w0 = (blockIdx.x * W + warp) * R; w0 < p.nrays; w0 += gridDim.x * W * R) {
+        const unsigned ray = w0 + lane / L;
+        const bool live = ray < p.nrays;
+        const size_t base = (size_t)ray * nr;
+        const float w = live ? __ldg(p.domega32 + ray) : 0.0f;
+        for (int m = 0; m < nslot; ++m) {
+            const float2 lf = s_lf[m * L + l];
+            state[m * 32] = make_float4(lf.x, lf.y, 0.0f, 0.0f);
+        }
+        int nlive = nslot;
+        bool bad = false;
+        float rho_n = 0.0f, td_n = 0.0f;
+        if (live && l < nr) {
+            rho_n = __ldg(p.rho + base + l);
+            td_n = __ldg(p.tdust + base + l);
+        }
+        for (int c0 = 0; c0 < nr; c0 += kBinCells) {
+            const int k = c0 + l;
+            const bool in = live && k < nr;
+            const float rho = rho_n, td = td_n;
+            float4 geo = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (in) {
+                geo = __ldg(&p.rtab[k]);
+                bad |= !(rho >= 0.0f && rho <= FLT_MAX) || (td != td);
+            }
+            if (live && k + kBinCells < nr) {  // the next chunk's
+                rho_n = __ldg(p.rho + base + k + kBinCells);
+                td_n = __ldg(p.tdust + base + k + kBinCells);
+            }
+            const bool dust = in && td <= p.t_sub;
+            const float d = dust ? rho * geo.x : 0.0f;
+            const bool zero = dust && d == 0.0f;
+            const float dmax = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(d, 0.0f))));
+            const unsigned zall = __ballot_sync(0xffffffffu, zero);
+            float sum = 0.0f;
+            if (dmax > 0.0f || zall) {
+                // bracketing temperature points; two non-negative terms, no cancellation
+                // where a row falls towards zero
+                int j = 0;
+                for (int s = 16; s > 0; s >>= 1)
+                    if (j + s < nt - 1 && s_tg[j + s] <= td) j += s;
+                const float f = zero ? -(float)kLog2e : -(float)kLog2e * d;
+                const float wu = f * fminf(fmaxf((td - s_tg[j]) * s_idt[j], 0.0f), 1.0f);
+                const float wl = f * fminf(fmaxf((s_tg[j + 1] - td) * s_idt[j], 0.0f), 1.0f);
+                const int rw = j * np * (int)sizeof(float4);  // (row of the cell's lower temperature)
+                int row[kBinCells];
+                float2 wt[kBinCells], wb[kBinCells], acc[kBinCells];
+#pragma unroll
+                for (int c = 0; c < kBinCells; ++c) {
+                    row[c] = __shfl_sync(0xffffffffu, rw, c, 8) + l * (int)sizeof(float4);
+                    wt[c] = f2(__shfl_sync(0xffffffffu, wu, c, 8));
+                    wb[c] = f2(__shfl_sync(0xffffffffu, wl, c, 8));
+                    acc[c] = f2(0.0f);
+                }
+                const unsigned zm = zall >> (lane & 24);
+                unsigned char *sb = reinterpret_cast<unsigned char *>(state);
+                if (zall) bins_slots<true>(nlive, km, dmax, smem, sb, row, wt, wb, zm, acc);
+                else bins_slots<false>(nlive, km, dmax, smem, sb, row, wt, wb, zm, acc);
+                // 2^-128 and below is flushed to zero and columns only grow: the last slots,
+                // of the largest opacities, drop out first
+                while (nlive > 0) {
+                    const float4 st = state[(nlive - 1) * 32];
+                    if (__any_sync(0xffffffffu, fmaxf(st.x, st.y) > -130.0f)) break;
+                    --nlive;
+                }
+                // lane l of the ray gets cell l: halve the cells, double the lanes summed
+                float v[kBinCells];
+#pragma unroll
+                for (int c = 0; c < kBinCells; ++c) v[c] = acc[c].x + acc[c].y;
+#pragma unroll
+                for (int h = 4; h > 0; h >>= 1) {
+                    const bool upper = lane & h;
+#pragma unroll
+                    for (int c = 0; c < h; ++c) {
+                        const float keep = upper ? v[c + h] : v[c], give = upper ? v[c] : v[c + h];
+                        v[c] = keep + __shfl_xor_sync(0xffffffffu, give, h);
+                    }
+                }
+                sum = v[0] * (float)taylor_coeff(0);
+            }
+            if (in) {
+                p.q[base + k] = zero ? 0.0f : geo.y * sum;
+                p.a[base + k] = geo.z * (zero ? sum : (d > 0.0f ? __fdividef(sum, d) : 0.0f));
+                if (!zero) eabs.add(sum * w);
+            }
+        }
+        if (__any_sync(0xffffffffu, bad) && lane == 0) atomicMax(p.bad_input, p.seq);
+        // the flux leaving the ray (Eq. 33)
+        float esc = 0.0f;
+        for (int m = 0; m < nslot; ++m) {
+            const float4 st = state[m * 32];
+            esc += ex2_approx(st.x + st.z) + ex2_approx(st.y + st.w);
+        }
+#pragma unroll
+        for (int o = 1; o < L; o <<= 1) esc += __shfl_xor_sync(0xffffffffu, esc, o);
+        if (l == 0) eesc.add(esc * w);
+    }
+
+    for (int o = 16; o > 0; o >>= 1) {
+        eabs.add(eabs.shfl_xor(o));
+        eesc.add(eesc.shfl_xor(o));
+    }
+    if (lane == 0) {
+        s_red[warp][0] = eabs;
+        s_red[warp][1] = eesc;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        KahanSum sa = s_red[0][0], se = s_red[0][1];
+        for (int w2 = 1; w2 < W; ++w2) {
+            sa.add(s_red[w2][0]);
+            se.add(s_red[w2][1]);
+        }
+        p.partials[blockIdx.x] = make_double2(to_double(sa), to_double(se));
+    }
+}
+
 // kt2[a][j] = (kappa[order[a]][j], kappa[order[a]][j + 1]) for the sorted active
 // bins; padding bins get zero opacity
 __global__ void k_build_tdep(int n_active, int nnu_pad, int n_t, const double *kappa_t, const int *order,
@@ -334,28 +572,52 @@ __global__ void k_build_tdep(int n_active, int nnu_pad, int n_t, const double *k
     kt2[idx] = make_float2((float)row[j], (float)row[j + 1 < n_t ? j + 1 : j]);
 }
 
-template <int C, int W, int MINB, bool PAIRS>
-cudaError_t launch_tdep_shape(const TraceArgs &a, const TdepTab &t, cudaStream_t stream, unsigned *grid_out)
+// persistent blocks of W warps, `rays` rays per warp and turn
+template <typename K, typename... Extra>
+cudaError_t launch_rays(K kern, int W, int rays, size_t smem, const TraceArgs &a, cudaStream_t stream,
+                        unsigned *grid_out, const Extra &...extra)
 {
-    const size_t smem = (size_t)a.nnu_pad * (16 + 4) + 16 + (size_t)(a.nnu_pad / 2) * t.n_t * sizeof(float4);
-    auto kern = k_ray_tdep<C, W, MINB, PAIRS>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int dev = 0, nsm = 0, per_sm = 0;
+    cudaError_t e = cudaSuccess;
+    if (smem > 40 * 1024) {  // the static part counts towards the 48 KB a launch has without asking
+        int most = 0;
+        e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        cudaFuncAttributes fa;
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+        if (e == cudaSuccess)  // one value for every caller: another thread's smaller call cannot lower it
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
         if (e != cudaSuccess) return e;
     }
-    int dev = 0, nsm = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     unsigned grid = (unsigned)nsm * (unsigned)per_sm;
-    const unsigned need = (a.nrays + W - 1) / W;
+    const unsigned need = (a.nrays + W * rays - 1) / (W * rays);
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    kern<<<grid, W * 32, smem, stream>>>(a, t);
+    kern<<<grid, W * 32, smem, stream>>>(a, extra...);
     *grid_out = grid;
     return cudaGetLastError();
+}
+
+template <int C, int W, int MINB, bool PAIRS>
+cudaError_t launch_tdep_shape(const TraceArgs &a, const TdepTab &t, cudaStream_t stream, unsigned *grid_out)
+{
+    const size_t smem = (size_t)a.nnu_pad * (16 + 4) + 16 + (size_t)(a.nnu_pad / 2) * t.n_t * sizeof(float4);
+    return launch_rays(k_ray_tdep<C, W, MINB, PAIRS>, W, 1, smem, a, stream, grid_out, t);
+}
+
+template <int W, int MINB>
+cudaError_t launch_tdep_bins(const TraceArgs &a, const TdepTab &t, cudaStream_t stream, unsigned *grid_out)
+{
+    constexpr int L = kBinLanes;
+    const int nslot = (a.n_active + 2 * L - 1) / (2 * L);
+    const size_t np = (size_t)nslot * L;
+    const size_t smem = np * t.n_t * sizeof(float4) + (size_t)W * nslot * 32 * sizeof(float4) + np * sizeof(float2);
+    return launch_rays(k_ray_tdep_bins<W, MINB>, W, 32 / L, smem, a, stream, grid_out, t, nslot);
 }
 
 struct TdepEntry {
@@ -363,11 +625,16 @@ struct TdepEntry {
     cudaError_t (*fn)(const TraceArgs &, const TdepTab &, cudaStream_t, unsigned *);
 };
 // the bin-pair form where its registers fit the cap without more than a few bytes of spill
+// the kernel with the bins across the lanes takes every ray length: it stands in every class of nr,
+// as (C, 4, 1)
+#define RT_TB(C) {C, 4, 1, &launch_tdep_bins<4, 4>}
 #define RT_TD(C, W, MB, PR) {C, W, MB, &launch_tdep_shape<C, W, MB, PR>}
 const TdepEntry kTdepShapes[] = {RT_TD(2, 4, 8, true),  RT_TD(4, 4, 8, false),  RT_TD(4, 4, 6, true),
                                  RT_TD(8, 4, 6, false), RT_TD(8, 4, 4, true),   RT_TD(16, 4, 3, false),
-                                 RT_TD(32, 4, 2, false)};
+                                 RT_TD(32, 4, 2, false),
+                                 RT_TB(2), RT_TB(4), RT_TB(8), RT_TB(16), RT_TB(32)};
 #undef RT_TD
+#undef RT_TB
 
 }  // namespace
 
@@ -382,6 +649,29 @@ int tdep_shapes(int nr, Shape *out, int max_out)
     for (const TdepEntry &s : kTdepShapes)
         if (s.c == c_fit && n < max_out) out[n++] = Shape{kKindRay, s.c, s.w, s.minb};
     return n;
+}
+
+// The shape without tuning. The bins across the lanes take a ray per 8 lanes and walk it serially
+// (1.5-2 us per 8 cells of a lone warp), so they need rays to fill the chip: from 2048 rays on with
+// 64 bins or more, from 4096 on with 32 to 63, and not with fewer (per chunk of 8 cells the kernel
+// spends as much beside the slots as 45 bins cost). us, cells across / bins across the lanes, full rank, 24 temperatures:
+//   79 bins: 256x64x32 52.2 / 51.7, 128x64x32 38 / 29, 512x64x32 110 / 95, 512x64x24 77 / 95,
+//            1000x64x32 211 / 179, 1000x64x16 112 / 178, 256x128x128 306 / 186, 64x256x256 567 / 164;
+//   32 bins: 256x64x48 37.5 / 43.9, 256x64x64 46.1 / 44.0, 256x128x128 135 / 119;
+//   128 bins: 256x64x32 77 / 63;  16 bins: 256x64x64 31.4 / 39.6, 100x64x64 19.4 / 19.3.
+// Below, of the register caps of the fewest cells per lane the wider (the bin-pair form:
+// 256x128x16 64.6 -> 51.9).
+Shape tdep_default(int nr, long long nrays, int n_active)
+{
+    Shape ts[16];
+    const int n = tdep_shapes(nr, ts, 16);
+    const bool bins = n_active >= 32 && nrays >= (n_active >= 64 ? 2048 : 4096);
+    Shape best{kKindRay, 0, 0, 0};
+    for (int i = 0; i < n; ++i) {
+        if ((ts[i].min_blocks == 1) != bins) continue;
+        if (best.cells_per_lane == 0 || ts[i].min_blocks < best.min_blocks) best = ts[i];
+    }
+    return best;
 }
 
 cudaError_t launch_tdep(Shape s, const TraceArgs &args, const float2 *kt2, const float *tg, int n_t,
