@@ -422,10 +422,9 @@ int trace(rt_ctx *c, const float *rho, const float *td, float *q, float *a, Shap
 
 int read_energy(rt_ctx *c, rt_energy *out)
 {
-    cudaError_t e = rt::launch_energy_reduce(c->partials, c->last_ntiles, c->sc, c->energy_d, c->stream);
+    cudaError_t e = rt::launch_energy_reduce(c->partials, c->last_ntiles, c->sc, c->energy_h, c->stream, c->bad,
+                                             c->bad_h);
     if (e != cudaSuccess) return cuda_fail(c, "energy reduce", e);
-    RT_CK(c, cudaMemcpyAsync(c->energy_h, c->energy_d, sizeof(rt_energy), cudaMemcpyDeviceToHost, c->stream));
-    RT_CK(c, cudaMemcpyAsync(c->bad_h, c->bad, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
     RT_CK(c, cudaStreamSynchronize(c->stream));
     *out = *c->energy_h;
     if (*c->bad_h == c->seq) return fail(c, RT_ERR_NONFINITE_INPUT, "input field holds NaN/Inf/negative density or NaN temperature");

@@ -286,7 +286,7 @@ cudaError_t launch_setup_geometry(int nr, int ntheta, int nphi, const double *r_
                                   double *domega, float *domega32, DevScalars *sc_dev,
                                   cudaStream_t stream);
 cudaError_t launch_energy_reduce(const double2 *partials, long long ntiles,
-                                 const DevScalars *sc_dev, rt_energy *out_dev,
-                                 cudaStream_t stream);
+                                 const DevScalars *sc_dev, rt_energy *out, cudaStream_t stream,
+                                 const unsigned *bad = nullptr, unsigned *bad_out = nullptr);
 
 }  // namespace rt

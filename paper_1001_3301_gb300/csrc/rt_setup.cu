@@ -223,17 +223,38 @@ __global__ void k_sum_domega(long long nrays, const double *domega, double t_sta
     }
 }
 
+// The energy balance from the launch's partials, and a copy of the validity word where bad is given
+// (a call that reads both back: out and bad_out then lie in page-locked host memory, which spares
+// the two copies that followed). One warp per 32 partials up to 1024 threads: on a small grid the
+// block's start and its barriers were the time (64x32 cells, the whole call 31.5 -> 22.8 us).
 __global__ void k_energy_reduce(const double2 *partials, long long ntiles, const DevScalars *sc,
-                                rt_energy *out)
+                                rt_energy *out, const unsigned *bad, unsigned *bad_out)
 {
-    __shared__ double s_red[32];
+    __shared__ double s_red[2][32];
     double sa = 0.0, se = 0.0;
     for (long long t = threadIdx.x; t < ntiles; t += blockDim.x) {
         sa += partials[t].x;
         se += partials[t].y;
     }
-    sa = block_sum(sa, s_red);
-    se = block_sum(se, s_red);
+    for (int o = 16; o > 0; o >>= 1) {
+        sa += __shfl_xor_sync(0xffffffffu, sa, o);
+        se += __shfl_xor_sync(0xffffffffu, se, o);
+    }
+    if (blockDim.x > 32) {
+        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        if (lane == 0) {
+            s_red[0][threadIdx.x >> 5] = sa;
+            s_red[1][threadIdx.x >> 5] = se;
+        }
+        __syncthreads();
+        if (threadIdx.x >= 32) return;
+        sa = lane < nw ? s_red[0][lane] : 0.0;
+        se = lane < nw ? s_red[1][lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) {
+            sa += __shfl_xor_sync(0xffffffffu, sa, o);
+            se += __shfl_xor_sync(0xffffffffu, se, o);
+        }
+    }
     if (threadIdx.x == 0) {
         const double scale = sc->r2 * sc->f_max;
         rt_energy e;
@@ -242,6 +263,7 @@ __global__ void k_energy_reduce(const double2 *partials, long long ntiles, const
         e.l_star = sc->l_grid;
         e.rel_err = (e.e_abs + e.e_esc) / e.l_star - 1.0;
         *out = e;
+        if (bad) *bad_out = *bad;
     }
 }
 
@@ -286,9 +308,11 @@ cudaError_t launch_setup_geometry(int nr, int ntheta, int nphi, const double *r_
 }
 
 cudaError_t launch_energy_reduce(const double2 *partials, long long ntiles,
-                                 const DevScalars *sc_dev, rt_energy *out_dev, cudaStream_t stream)
+                                 const DevScalars *sc_dev, rt_energy *out, cudaStream_t stream, const unsigned *bad,
+                                 unsigned *bad_out)
 {
-    k_energy_reduce<<<1, 1024, 0, stream>>>(partials, ntiles, sc_dev, out_dev);
+    const int threads = ntiles >= 1024 ? 1024 : ntiles <= 32 ? 32 : (int)((ntiles + 31) / 32) * 32;
+    k_energy_reduce<<<1, threads, 0, stream>>>(partials, ntiles, sc_dev, out, bad, bad_out);
     return cudaGetLastError();
 }
 
