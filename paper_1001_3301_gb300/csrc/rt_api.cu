@@ -995,13 +995,14 @@ int host_enqueue(rt_ctx *ctx, const float *rho, const float *t_dust, float *q_ab
         if (!ok) return cuda_fail(ctx, "host pipeline streams", cudaGetLastError());
         RT_CK(ctx, cudaEventRecord(ctx->ev_out, ctx->s_out));
     }
-    // ~2 M cells per chunk, copies of 8 MB per field, since the link moves small copies in both
+    // ~1.4-2 M cells per chunk, copies of 6-8 MB per field, since the link moves small copies in both
     // directions at once less efficiently (4 MB: 253 GB/s in total, 16 MB: 312 GB/s, one 256 MB copy
     // each way: 340 GB/s); below 8 M cells up to four chunks of >= 0.5 M cells, since there the first
     // copies in and the last ones out, which overlap nothing, weigh more (one chunk or ~2 M cells
     // each -> four, us: 1.6 M cells 169 -> 147, 2.1 M 213 -> 189, 3.1 M 302 -> 260, 4.2 M 333 -> 310,
-    // 6.3 M 450 -> 442; 8.4 M cells: four chunks 565, six 553-569, smaller end chunks 562-594)
-    int nch = ctx->ncells >= 1LL << 23 ? (int)std::min<long long>(kHostChunks, ctx->ncells >> 21)
+    // 6.3 M 450 -> 442, where six take 462; four -> six: 8.4 M cells 565 -> 521-553, 12 M 769 -> 764,
+    // 14 M 921 -> 907; smaller end chunks: 8.4 M cells 562-594)
+    int nch = ctx->ncells >= 1LL << 23 ? (int)std::min<long long>(kHostChunks, std::max<long long>(6, ctx->ncells >> 21))
                                        : (int)std::max<long long>(1, std::min<long long>(4, ctx->ncells >> 19));
     if (nch > ctx->nrays) nch = (int)ctx->nrays;
     long long bound = 0;
