@@ -26,6 +26,8 @@
 //
 //
 // The per-(cell, bin) arithmetic is described in rt_device.cuh.
+#include <algorithm>
+
 #include "rt_tile.cuh"
 
 namespace rt {
@@ -52,20 +54,29 @@ __global__ void __launch_bounds__(W * 32, MINB) k_trace(const TraceArgs p)
 // when there are fewer tiles. The FP64 mode launches one CTA per tile instead: a tile's
 // work depends on its columns (a midplane tile takes several times the mean) and is long
 // against the CTA's set-up, so the hardware's block scheduler balances the SMs, which
-// contiguous ranges left two thirds idle (128x64x64, 79 bins, tau550 = 1: 0.55 -> 0.26 ms).
+// contiguous ranges left two thirds idle (128x64x64, 79 bins, tau550 = 1: 0.55 -> 0.25 ms).
 // Returns the grid size (energy partials written).
 template <int C, int W, int MODE, int MINB>
 cudaError_t launch_shape(const TraceArgs &a, unsigned ntiles, cudaStream_t stream, unsigned *grid_out,
                          unsigned max_grid)
 {
-    const size_t smem = trace_smem_bytes<C, W, MODE>(a);
+    size_t smem = trace_smem_bytes<C, W, MODE>(a);
+    // FP64: at most three CTAs per SM, by their shared memory. Two or three fill the FP64 pipe (a warp
+    // instruction takes it 16 clocks), and with the tiles handed out as CTAs end, an SM that holds eight
+    // from the start keeps its expensive ones while others run dry. us, eight / three / two / one per SM:
+    // 128x64x64 249 / 217 / 218 / 259, 100x97x31 296 / 159 / 156 / 168, 512x256x32 913 / 913 / 929 / 1114.
+    if (MODE == RT_FP64) smem = std::max(smem, (size_t)(200 * 1024 / 3));
     auto kern = k_trace<C, W, MODE, MINB>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
     int dev = 0, nsm = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess && smem > 40 * 1024) {  // the static part counts towards the 48 KB a launch has without asking
+        int most = 0;
+        cudaFuncAttributes fa;
+        e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+        if (e == cudaSuccess)  // one value for every caller: another thread's smaller call cannot lower it
+            e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes);
+    }
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, W * 32, smem);
     if (e != cudaSuccess) return e;
