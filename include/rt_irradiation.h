@@ -238,7 +238,9 @@ int rt_get_bins(rt_ctx *ctx, double *f_bin);
  * automatic choice. Shapes that are not compiled in or do not fit the grid return
  * RT_ERR_INVALID_ARG. rt_get_tuning reports the shape in use; rt_list_tunings
  * writes the shapes that apply to this context's grid and precision (up to max of
- * them) into the four arrays and returns their number (negative status on error). */
+ * them) into the four arrays and returns their number (negative status on error).
+ * With a full-rank temperature table the shapes with min_blocks_per_sm 1 are the
+ * kernel with the bins across the lanes. */
 int rt_set_tuning(rt_ctx *ctx, int kind, int cells_per_lane, int warps_per_block,
                   int min_blocks_per_sm);
 int rt_get_tuning(const rt_ctx *ctx, int *kind, int *cells_per_lane, int *warps_per_block,
@@ -422,7 +424,7 @@ int rt_rosseland_mean_opacity(rt_ctx *ctx, double t, double *kappa_r);
 
 typedef struct rt_fld_stats {
     int iterations;      /* conjugate-gradient iterations taken, all passes */
-    int passes;          /* refinement passes */
+    int passes;          /* groups between two residual replacements */
     double rel_change;   /* max over cells of |correction| / |E'| of the last pass */
     int levels;          /* multigrid levels of the preconditioner (1: Jacobi) */
 } rt_fld_stats;

@@ -18,6 +18,9 @@
 // largest column, the remaining bins take the per-cell select between the 5-term
 // series and 1 - ex2 (kappa's smallest value need not follow the same order). A pair
 // takes the class of its upper bin, which holds for the lower one too.
+//
+// Where the rays fill the chip the bins go across the lanes instead (k_ray_tdep_bins below; the
+// line is in tdep_default).
 #include "rt_device.cuh"
 
 namespace rt {
