@@ -1859,9 +1859,10 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
     const auto line_post = ring_sm ? k_line_post<true> : k_line_post<false>;
     const auto apply = quads ? k_it_apply<true> : k_it_apply<false>;
     const auto flush = quads ? k_it_flush<true> : k_it_flush<false>;
-    // (one limit for all contexts: another thread's smaller step must not lower it)
+    // (one limit for all contexts: another thread's smaller step must not lower it; the kernels'
+    // static part, at most 6.7 KB, counts towards the 48 KB a launch has without asking)
     auto big_smem = [](const void *kern, size_t bytes) {
-        return bytes <= 48 * 1024 ||
+        return bytes <= 40 * 1024 ||
                (bytes <= kMaxFldSmem && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                              (int)kMaxFldSmem) == cudaSuccess);
     };
