@@ -1897,6 +1897,19 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
         apply<<<g_app, 256, 0, st>>>(cg, pc, pbuf[(i + 1) & 1]);
     };
     if (!fs->loop && !fs->no_graph) {  // the loop's graph
+        // (none of its launches may be refused: the kernel would be missing from the body)
+        bool fit = launch_fits((const void *)flush, 256, 0) && launch_fits((const void *)residual, t_line, sm_line) &&
+                   launch_fits((const void *)apply, 256, 0) && launch_fits((const void *)k_it_loop, 1, 0);
+        if (use_mg)
+            fit = fit && launch_fits((const void *)down0, 256, 0) && launch_fits((const void *)k_mg_down<false>, 256, 0) &&
+                  launch_fits((const void *)k_mg_tail, 1024, sm_tail) && launch_fits((const void *)k_mg_up, 256, 0) &&
+                  launch_fits((const void *)up0, 256, 0) &&
+                  (!lines || launch_fits((const void *)line_post, t_line, sm_line));
+        else
+            fit = fit && launch_fits((const void *)k_it_jacobi, 256, 0);
+        if (!fit) return ctx_fail(ctx, RT_ERR_CUDA, "FLD step: a kernel of the loop does not fit its launch");
+        cudaGetLastError();  // (an older call's error is none of these launches')
+        cudaError_t refused = cudaSuccess;
         cudaGraph_t graph = nullptr, body = nullptr, end = nullptr;
         cudaGraphConditionalHandle h{};
         cudaGraphNode_t node = nullptr;
@@ -1918,13 +1931,17 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
         if (cap) {
             for (int i = 0; i < kUnroll; ++i) iteration(i);
             k_it_loop<<<1, 1, 0, st>>>(fs->scal, h);
-            cap = cudaStreamEndCapture(st, &end) == cudaSuccess;
+            refused = cudaGetLastError();
+            cap = cudaStreamEndCapture(st, &end) == cudaSuccess && refused == cudaSuccess;
         }
         cap = cap && cudaGraphInstantiate(&fs->loop, graph, 0) == cudaSuccess;
         if (graph) cudaGraphDestroy(graph);
         if (!cap) {
             cudaGetLastError();
             fs->loop = nullptr;
+            // (the host-driven loop would have the same launch refused)
+            if (refused != cudaSuccess)
+                return ctx_fail(ctx, RT_ERR_CUDA, std::string("FLD loop: ") + cudaGetErrorString(refused));
             fs->no_graph = true;
         }
     }

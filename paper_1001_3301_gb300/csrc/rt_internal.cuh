@@ -271,6 +271,19 @@ int ctx_fail(rt_ctx *c, int status, const std::string &msg);
 // rt_irradiate on one of the surrogate's training fields, in a shape that depends on the grid alone
 int trace_training(rt_ctx *c, const float *rho, const float *td, float *q, float *a);
 
+// Whether a launch of `kern` with this block and dynamic shared memory is one it may have; asked
+// before launches are captured, as one that is refused in there is missing from the graph.
+inline bool launch_fits(const void *kern, int threads, size_t smem)
+{
+    cudaFuncAttributes fa;
+    if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    const size_t most = (size_t)fa.maxDynamicSharedSizeBytes, plain = 48 * 1024;
+    return threads <= fa.maxThreadsPerBlock && smem <= most && (most > plain || smem + fa.sharedSizeBytes <= plain);
+}
+
 // Set-up kernels (rt_setup.cu)
 // order_dev (may be null) receives the original index of every kappa-sorted bin
 cudaError_t launch_setup_bins(int n_nu, const double *nu_mid_dev, const double *kappa_dev,
