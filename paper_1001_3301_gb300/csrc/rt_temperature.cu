@@ -20,6 +20,7 @@
 // takes Newton steps only in the intervals where that check failed.
 #include <math.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -33,7 +34,7 @@ constexpr int kTempNodes = 1024;
 // node i at v = (v_org + i) 2^-e, v_org an integer, at most kTempInvNodes nodes.
 constexpr int kTempInvNodes = 2048;
 // the context's table buffer: lkp [kTempNodes]; 8 constants (X(y_lo), X(y_hi), 2^e,
-// v_org, the node count of the inverse table); then (16-byte aligned) the cubic
+// v_org, the node count of the inverse table, 1 / the step diffuse_temperature accepts); then (16-byte aligned) the cubic
 // coefficients of lkp [kTempNodes - 1], of the inverse table [kTempInvNodes - 1] and of lkp in
 // lg2 units [kTempNodes + 1], float4 each, and the inverse table's nodes while it is built
 constexpr int kTempConsts = kTempNodes;
@@ -136,7 +137,8 @@ __device__ __forceinline__ double inverse_node_x(double i, int v_org, int e, dou
 
 // the nodes: ym[i] = (y, dT/dt)
 __global__ void __launch_bounds__(128) k_inverse_nodes(const float *lkp, float *consts, double2 *ym, double y0,
-                                                       double y1, double ln_a, int e, int v_org, int n_inv)
+                                                       double y1, double ln_a, int e, int v_org, int n_inv,
+                                                       float per_step)
 {
     const double inv_dy = (kTempNodes - 1) / (y1 - y0);
     const double hx = ldexp(1.0, -e) * kLn2;
@@ -153,6 +155,7 @@ __global__ void __launch_bounds__(128) k_inverse_nodes(const float *lkp, float *
         consts[2] = (float)ldexp(1.0, e);
         consts[3] = (float)v_org;
         consts[4] = (float)n_inv;
+        consts[5] = per_step;
     }
 }
 
@@ -209,7 +212,7 @@ struct TempArgs {
     const float *e_rad;   // may be null (E_R = 0)
     float *t_out;
     const float *lkp;     // [kTempNodes] ln kappa_P on the uniform ln T grid
-    const float *consts;  // X(y_lo), X(y_hi), 2^e, v_org, node count of the inverse table
+    const float *consts;  // X(y_lo), X(y_hi), 2^e, v_org, node count of the inverse table, per_step
     const float4 *c_lkp;  // [kTempNodes - 1] cubic coefficients of lkp per interval
     const float4 *c_inv;  // [n_inv - 1] cubic coefficients of T on the v = lg2 a_rad grid
     int vec;              // a_rad, e_rad (if any) and t_out are 16-byte aligned
@@ -277,6 +280,7 @@ struct TempConsts {
     float l_lo, l_hi, v_scale, v_org, u_max;
     int k_max;
     float sat_scale, sat_org, u_top;  // lg2 a_rad to [0, 1] over the inverse table, and its last interval
+    float per_step;                   // 1 / the last step of ln T that diffuse_temperature accepts
 };
 
 // rcp.approx (relative error below 2^-22)
@@ -296,19 +300,77 @@ __device__ __forceinline__ float2 splat(float v) { return make_float2(v, v); }
 // Halley step on F(y) = 4 y + ln a - ln(E_R + a_rad / kappa_P), y = ln T, with F'' from L' alone
 // (the error it leaves is cubic but for L''), and a Newton step. F is the log of a ratio near 1,
 // so there is no cancellation, and the last step is applied to T itself: the rounding of ln T
-// (5e-7) does not reach the result. Where the last step is above 5e-4, or a value is beyond the
-// tables or the hardware functions' range, err says so and the cell takes the general solve.
+// (5e-7) does not reach the result. A last step above what the table's curvature allows
+// (accepted_step) is followed by further Newton steps of the thread's cells (diffuse_more: most
+// cells of a table whose mean has kinks need one); where a value is beyond the tables or the
+// hardware functions' range, or the steps do not settle, the cell takes the general solve.
 // What bounds it: issue slots. So the intervals come from a saturating multiply and an FMA
 // that rounds down to an integer (no conversions, no clamps; the lg2 kappa_P table has a constant
 // interval at either end in place of range tests), and the arithmetic runs on pairs of cells.
 // 8.4 M cells with E_R: 131 us for Newton steps from 300 K with accurate exp and log, 58 us for
-// these steps cell by cell, 49 us four cells at once (175 instructions per cell), 41 us (116).
+// these steps cell by cell, 49 us four cells at once (175 instructions per cell), 41 us (116);
+// further steps cost less than the general solve they spare (524 k cells, kappa(nu, T) linear
+// between 24 temperatures: 19 us with the cells beyond 5e-4 sent there, 14 us now).
+constexpr float kMagic = 12582912.0f;  // 1.5 2^23: adding it, rounding down, gives the floor
+constexpr int kMagicBits = 0x4b400000;
+
+template <bool HALLEY, int N>
+__device__ __forceinline__ void diffuse_step(const TempArgs &p, const TempConsts &k, const float (&ar)[N],
+                                             const float (&er)[N], float (&l)[N], float (&t_out)[N], float (&err)[N])
+{
+#pragma unroll
+    for (int c = 0; c < N; c += 2) {
+        // lg2 kappa_P and d ln kappa_P / dy: the interval, and the offset in it by FMA
+        float L[2], dL[2], T[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float x = l[c + i];
+            const float m = __fmaf_rd(__saturatef(fmaf(x, p.l_scale, p.l_org)), kTempLg2Top, kMagic);
+            // (node n of the table is entry n + 1)
+            const float t = fmaf(x, p.s_lo, fmaf(x, p.s_hi, -(m - (kMagic + 1.0f))));
+            const float4 q = __ldg(p.c_lg2 + (__float_as_int(m) - kMagicBits));
+            L[i] = fmaf(fmaf(fmaf(q.w, t, q.z), t, q.y), t, q.x);
+            dL[i] = fmaf(fmaf(3.0f * q.w, t, 2.0f * q.z), t, q.y);
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(T[i]) : "f"(x));
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(L[i]) : "f"(-L[i]));  // 1 / kappa_P
+        }
+        const float2 T2 = make_float2(T[0], T[1]), e2 = make_float2(er[c], er[c + 1]);
+        const float2 d2 = __fmul2_rn(make_float2(dL[0], dL[1]), splat(p.dl_dy));
+        const float2 src = __fmul2_rn(make_float2(ar[c], ar[c + 1]), make_float2(L[0], L[1]));
+        const float2 rhs = __fadd2_rn(e2, src);
+        const float2 tt = __fmul2_rn(T2, T2), t4 = __fmul2_rn(__fmul2_rn(splat(p.a), tt), tt);
+        const float2 den = __ffma2_rn(src, d2, __fmul2_rn(rhs, splat(4.0f)));
+        const float2 rt = make_float2(rcp_fast(t4.x), rcp_fast(t4.y));
+        const float2 rd = make_float2(rcp_fast(den.x), rcp_fast(den.y));
+        const float2 x = __ffma2_rn(rhs, rt, splat(-1.0f));  // rhs / (a T^4) - 1
+        // ln(1 + x): to 1e-4 at x = 0.3 (the first step), to rounding where the last step is
+        float2 f = splat(1.0f / 3.0f);
+        if (HALLEY) f = __ffma2_rn(x, __ffma2_rn(x, splat(0.2f), splat(-0.25f)), f);
+        f = __fmul2_rn(x, __ffma2_rn(x, __ffma2_rn(x, f, splat(-0.5f)), splat(1.0f)));
+        float2 dy = __fmul2_rn(f, __fmul2_rn(rhs, rd));
+        if (HALLEY) {
+            // dy (1 + F F'' / (2 F'^2))
+            const float2 sd = __fmul2_rn(__fmul2_rn(src, rd), d2);
+            const float2 ed = __fmul2_rn(__fmul2_rn(e2, rd), d2);
+            dy = __ffma2_rn(dy, __fmul2_rn(__fmul2_rn(f, splat(0.5f)), __fmul2_rn(sd, ed)), dy);
+            l[c] = fmaf(dy.x, 1.44269504088896340736f, l[c]);
+            l[c + 1] = fmaf(dy.y, 1.44269504088896340736f, l[c + 1]);
+        } else {
+            const float2 g = __ffma2_rn(__fmul2_rn(dy, splat(0.5f)), dy, dy);
+            const float2 r = __ffma2_rn(T2, g, T2);
+            t_out[c] = r.x;
+            t_out[c + 1] = r.y;
+            // (a NaN step gives err = NaN, which is not below 1)
+            err[c] = fabsf(dy.x) * k.per_step;
+            err[c + 1] = fabsf(dy.y) * k.per_step;
+        }
+    }
+}
+
 template <int N>
 __device__ __forceinline__ void diffuse_temperature(const TempArgs &p, const TempConsts &k, const float (&ar)[N],
                                                     const float (&er)[N], float (&t_out)[N], float (&err)[N])
 {
-    constexpr float kMagic = 12582912.0f;  // 1.5 2^23: adding it, rounding down, gives the floor
-    constexpr int kMagicBits = 0x4b400000;
     float l[N];
 #pragma unroll
     for (int c = 0; c < N; ++c) {
@@ -320,58 +382,37 @@ __device__ __forceinline__ void diffuse_temperature(const TempArgs &p, const Tem
         const float tc = fmaf(fmaf(fmaf(q.w, t, q.z), t, q.y), t, q.x), t2 = tc * tc;
         // beyond the inverse table t leaves [0, 1]; a_rad = 0 (t = -Inf) has no source
         const bool in = fabsf(t - 0.5f) < 0.501f;
-        l[c] = 0.25f * lg2_approx(fmaf(er[c], p.inv_a, in ? t2 * t2 : 0.0f));
-        err[c] = (in || ar[c] == 0.0f) && fabsf(l[c] - 8.0f) < 18.0f ? 0.0f : 2.0f;  // T in 1e-3 .. 6e7 K
+        const float l0 = 0.25f * lg2_approx(fmaf(er[c], p.inv_a, in ? t2 * t2 : 0.0f));
+        // T in 1e-3 .. 6e7 K (a NaN start gives a NaN step)
+        l[c] = (in || ar[c] == 0.0f) && fabsf(l0 - 8.0f) < 18.0f ? l0 : NAN;
+    }
+    diffuse_step<true, N>(p, k, ar, er, l, t_out, err);
+    diffuse_step<false, N>(p, k, ar, er, l, t_out, err);
+}
+
+// Further Newton steps from t_out while a cell is short of its step but near (0.1 in ln T; three
+// steps at most: quadratic from there), then the general solve of the rest.
+__device__ float cell_temperature_general(const TempArgs &p, const TempConsts &k, float ar, float er);
+
+template <int N>
+__device__ __forceinline__ void diffuse_more(const TempArgs &p, const TempConsts &k, const float (&ar)[N],
+                                             const float (&er)[N], float (&t_out)[N], float (&err)[N])
+{
+#pragma unroll 1
+    for (int it = 0; it < 3; ++it) {
+        bool more = false;
+        float l[N];
+#pragma unroll
+        for (int c = 0; c < N; ++c) {
+            more |= err[c] >= 1.0f && err[c] < 0.1f * k.per_step;
+            l[c] = lg2_approx(t_out[c]);
+        }
+        if (!more) break;
+        diffuse_step<false, N>(p, k, ar, er, l, t_out, err);
     }
 #pragma unroll
-    for (int it = 0; it < 2; ++it)
-#pragma unroll
-        for (int c = 0; c < N; c += 2) {
-            // lg2 kappa_P and d ln kappa_P / dy: the interval, and the offset in it by FMA
-            float L[2], dL[2], T[2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const float x = l[c + i];
-                const float m = __fmaf_rd(__saturatef(fmaf(x, p.l_scale, p.l_org)), kTempLg2Top, kMagic);
-                // (node n of the table is entry n + 1)
-                const float t = fmaf(x, p.s_lo, fmaf(x, p.s_hi, -(m - (kMagic + 1.0f))));
-                const float4 q = __ldg(p.c_lg2 + (__float_as_int(m) - kMagicBits));
-                L[i] = fmaf(fmaf(fmaf(q.w, t, q.z), t, q.y), t, q.x);
-                dL[i] = fmaf(fmaf(3.0f * q.w, t, 2.0f * q.z), t, q.y);
-                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(T[i]) : "f"(x));
-                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(L[i]) : "f"(-L[i]));  // 1 / kappa_P
-            }
-            const float2 T2 = make_float2(T[0], T[1]), e2 = make_float2(er[c], er[c + 1]);
-            const float2 d2 = __fmul2_rn(make_float2(dL[0], dL[1]), splat(p.dl_dy));
-            const float2 src = __fmul2_rn(make_float2(ar[c], ar[c + 1]), make_float2(L[0], L[1]));
-            const float2 rhs = __fadd2_rn(e2, src);
-            const float2 tt = __fmul2_rn(T2, T2), t4 = __fmul2_rn(__fmul2_rn(splat(p.a), tt), tt);
-            const float2 den = __ffma2_rn(src, d2, __fmul2_rn(rhs, splat(4.0f)));
-            const float2 rt = make_float2(rcp_fast(t4.x), rcp_fast(t4.y));
-            const float2 rd = make_float2(rcp_fast(den.x), rcp_fast(den.y));
-            const float2 x = __ffma2_rn(rhs, rt, splat(-1.0f));  // rhs / (a T^4) - 1
-            // ln(1 + x): to 1e-4 at x = 0.3 (the first step), to rounding where the last step is
-            float2 f = splat(1.0f / 3.0f);
-            if (it == 0) f = __ffma2_rn(x, __ffma2_rn(x, splat(0.2f), splat(-0.25f)), f);
-            f = __fmul2_rn(x, __ffma2_rn(x, __ffma2_rn(x, f, splat(-0.5f)), splat(1.0f)));
-            float2 dy = __fmul2_rn(f, __fmul2_rn(rhs, rd));
-            if (it == 0) {
-                // Halley: dy (1 + F F'' / (2 F'^2))
-                const float2 sd = __fmul2_rn(__fmul2_rn(src, rd), d2);
-                const float2 ed = __fmul2_rn(__fmul2_rn(e2, rd), d2);
-                dy = __ffma2_rn(dy, __fmul2_rn(__fmul2_rn(f, splat(0.5f)), __fmul2_rn(sd, ed)), dy);
-                l[c] = fmaf(dy.x, 1.44269504088896340736f, l[c]);
-                l[c + 1] = fmaf(dy.y, 1.44269504088896340736f, l[c + 1]);
-            } else {
-                const float2 g = __ffma2_rn(__fmul2_rn(dy, splat(0.5f)), dy, dy);
-                const float2 r = __ffma2_rn(T2, g, T2);
-                t_out[c] = r.x;
-                t_out[c + 1] = r.y;
-                // (a NaN step gives err = NaN, which is not below 1)
-                err[c] = fmaf(fabsf(dy.x), 2000.0f, err[c]);
-                err[c + 1] = fmaf(fabsf(dy.y), 2000.0f, err[c + 1]);
-            }
-        }
+    for (int c = 0; c < N; ++c)
+        if (!(err[c] < 1.0f)) t_out[c] = cell_temperature_general(p, k, ar[c], er[c]);
 }
 
 // T of one cell (Eq. 16): a T^4 = E_R + a_rad / kappa_P(T); 0 where both sources vanish.
@@ -415,11 +456,14 @@ __device__ __forceinline__ float cell_temperature_body(const TempArgs &p, const 
     // the general solve (what diffuse_temperature leaves):
     // Newton on F(y) = 4 y + ln a - ln(E_R + a_rad e^{-L}) from 300 K's opacity; it
     // converges quadratically: once a step is below 1e-5 the next one reaches the FP32
-    // resolution of ln T, so one more step ends the solve
+    // resolution of ln T, so one more step ends the solve. F grows with y, so each
+    // evaluation bounds the root from one side, and a step out of the bounds (a steep mean
+    // sends Newton back and forth) halves them instead.
     interp_c(p.c_lkp, k.l_lo, k.l_hi, 5.7037825f, p.y0, p.inv_dy, L, dL);
     y = 0.25f * (logf(er + ar * expf(-L)) - p.ln_a);
+    float y_lo = -100.0f, y_hi = 100.0f;  // (T of any float sources lies within e^(-20 .. 60))
     bool close = false;
-    for (int it = 0; it < 24; ++it) {
+    for (int it = 0; it < 48; ++it) {
         interp_c(p.c_lkp, k.l_lo, k.l_hi, y, p.y0, p.inv_dy, L, dL);
         const float src = ar * expf(-L);
         const float rhs = er + src;
@@ -427,6 +471,9 @@ __device__ __forceinline__ float cell_temperature_body(const TempArgs &p, const 
         const float fp = 4.0f + dL * __fdividef(src, rhs);
         float dy = -__fdividef(f, fmaxf(fp, 0.5f));
         dy = fminf(fmaxf(dy, -2.0f), 2.0f);
+        if (f < 0.0f) y_lo = y;
+        if (f > 0.0f) y_hi = y;
+        if (!close && fabsf(dy) >= 1e-5f && (y + dy <= y_lo || y + dy >= y_hi)) dy = 0.5f * (y_lo + y_hi) - y;
         y += dy;
         if (close) break;
         close = fabsf(dy) < 1e-5f;
@@ -439,8 +486,7 @@ __device__ __forceinline__ float cell_temperature(const TempArgs &p, const TempC
 {
     return cell_temperature_body<ER>(p, k, ar, er);
 }
-template <>
-__device__ __noinline__ float cell_temperature<true>(const TempArgs &p, const TempConsts &k, float ar, float er)
+__device__ __noinline__ float cell_temperature_general(const TempArgs &p, const TempConsts &k, float ar, float er)
 {
     return cell_temperature_body<true>(p, k, ar, er);
 }
@@ -461,12 +507,13 @@ __global__ void __launch_bounds__(256) k_dust_temperature(const TempArgs p)
     k.sat_scale = k.v_scale / k.u_max;
     k.sat_org = k.v_org / k.u_max;
     k.u_top = k.u_max - 0.001f;
+    k.per_step = ER ? __ldg(p.consts + 5) : 0.0f;
     const long long tid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long n4 = p.vec ? p.n / 4 : 0;
     // D quads in flight per thread: slot d holds the inputs of quad v + d stride, and is
     // refilled with quad v + (d + D) stride before quad v + d stride is solved (one with
-    // an E_R field: its Newton solve needs the registers)
+    // an E_R field: the steps of its four cells need the registers)
     constexpr int D = ER ? 1 : 2;
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     float4 an[D], en[D];
@@ -493,9 +540,8 @@ __global__ void __launch_bounds__(256) k_dust_temperature(const TempArgs p)
                 const float er[4] = {fmaxf(e4.x, 0.0f), fmaxf(e4.y, 0.0f), fmaxf(e4.z, 0.0f), fmaxf(e4.w, 0.0f)};
                 float t[4], err[4];
                 diffuse_temperature<4>(p, k, ar, er, t, err);
-#pragma unroll
-                for (int c = 0; c < 4; ++c)
-                    if (!(err[c] < 1.0f)) t[c] = cell_temperature<ER>(p, k, ar[c], er[c]);
+                if (!(err[0] < 1.0f && err[1] < 1.0f && err[2] < 1.0f && err[3] < 1.0f))
+                    diffuse_more<4>(p, k, ar, er, t, err);
                 t4 = make_float4(t[0], t[1], t[2], t[3]);
             } else {
                 t4.x = cell_temperature<ER>(p, k, a4.x, e4.x);
@@ -512,7 +558,8 @@ __global__ void __launch_bounds__(256) k_dust_temperature(const TempArgs p)
             const float ar[2] = {a0, a0}, er[2] = {e0, e0};
             float t[2], err[2];
             diffuse_temperature<2>(p, k, ar, er, t, err);
-            p.t_out[c] = err[0] < 1.0f ? t[0] : cell_temperature<ER>(p, k, a0, e0);
+            if (!(err[0] < 1.0f)) diffuse_more<2>(p, k, ar, er, t, err);
+            p.t_out[c] = t[0];
         } else {
             p.t_out[c] = cell_temperature<ER>(p, k, p.a_rad[c], 0.0f);
         }
@@ -557,6 +604,36 @@ int planck_means(const CtxInfo &in, const std::vector<double> &t_nodes, double *
     cudaFree(tg);
     cudaFree(kp);
     return ok ? RT_OK : RT_ERR_CUDA;
+}
+
+// The last Newton step of ln T after which diffuse_temperature takes a cell. A step dy leaves
+// F''/(2 F') dy^2, with F' = 4 + w L' and F'' = w L'' - w (1 - w) L'^2, 0 <= w <= 1 the source's
+// share: the largest |L''| and |L'| of the table's cubics bound that by kLeft. 5e-4 on means of
+// kappa(nu), 5e-5 to 1e-4 on tables whose kappa(T) is linear between 24 or 32 temperatures (kinks
+// in the mean: L'' in the hundreds; with 5e-4 there, one cell in a thousand was off by up to 2e-5).
+double accepted_step(const std::vector<float> &h)
+{
+    constexpr double kLeft = 1.5e-7;
+    const double per_y = (kTempNodes - 1) / (kTempLnHi - kTempLnLo);
+    double curve = 0.0, slope = 0.0, fall = 0.0;
+    for (int k = 0; k < kTempNodes - 1; ++k) {  // the cubics of k_hermite_coeffs
+        const double p0 = h[k], p1 = h[k + 1];
+        const double m0 = k > 0 ? 0.5 * (p1 - h[k - 1]) : p1 - p0;
+        const double m1 = k + 2 < kTempNodes ? 0.5 * (h[k + 2] - p0) : p1 - p0;
+        const double q2 = 3.0 * (p1 - p0) - 2.0 * m0 - m1, q3 = 2.0 * (p0 - p1) + m0 + m1;
+        curve = std::max({curve, fabs(2.0 * q2), fabs(2.0 * q2 + 6.0 * q3)});
+        for (double t : {0.0, 1.0, q3 != 0.0 ? -q2 / (3.0 * q3) : 0.0}) {
+            if (!(t >= 0.0 && t <= 1.0)) continue;
+            const double d = m0 + t * (2.0 * q2 + t * 3.0 * q3);
+            slope = std::max(slope, fabs(d));
+            fall = std::max(fall, -d);
+        }
+    }
+    curve *= per_y * per_y;
+    slope *= per_y;
+    fall *= per_y;
+    const double left = (curve + 0.25 * slope * slope) / (2.0 * std::max(4.0 - fall, 0.5));
+    return std::min(5e-4, std::max(1e-6, sqrt(kLeft / left)));  // (a NaN or infinite curve: 1e-6 or less)
 }
 
 }  // namespace
@@ -605,13 +682,11 @@ int rt_dust_temperature(rt_ctx *ctx, const float *a_rad, const float *e_rad, flo
         if (rc != RT_OK) return ctx_fail(ctx, rc, err);
         // the inverse table's grid in v = lg2 a_rad: the finest spacing 2^-e whose nodes
         // (whole steps from v_org) cover X(y_lo)..X(y_hi) within kTempInvNodes
-        float ends[2];
-        if (cudaMemcpyAsync(&ends[0], lkp, sizeof(float), cudaMemcpyDeviceToHost, in.stream) != cudaSuccess ||
-            cudaMemcpyAsync(&ends[1], lkp + kTempNodes - 1, sizeof(float), cudaMemcpyDeviceToHost, in.stream) !=
-                cudaSuccess ||
+        std::vector<float> h(kTempNodes);
+        if (cudaMemcpyAsync(h.data(), lkp, sizeof(float) * kTempNodes, cudaMemcpyDeviceToHost, in.stream) != cudaSuccess ||
             cudaStreamSynchronize(in.stream) != cudaSuccess)
-            return ctx_fail(ctx, RT_ERR_CUDA, "Planck-mean table ends");
-        const double v_lo = (4.0 * kTempLnLo + ends[0] + ln_a) / kLn2, v_hi = (4.0 * kTempLnHi + ends[1] + ln_a) / kLn2;
+            return ctx_fail(ctx, RT_ERR_CUDA, "Planck-mean table");
+        const double v_lo = (4.0 * kTempLnLo + h[0] + ln_a) / kLn2, v_hi = (4.0 * kTempLnHi + h[kTempNodes - 1] + ln_a) / kLn2;
         int e = 6, v_org = 0, n_inv = 0;
         for (; e >= 0; --e) {
             v_org = (int)floor(ldexp(v_lo, e));
@@ -621,7 +696,7 @@ int rt_dust_temperature(rt_ctx *ctx, const float *a_rad, const float *e_rad, flo
         if (e < 0 || n_inv < 2) return ctx_fail(ctx, RT_ERR_INVALID_ARG, "Planck mean outside the tabulated range");
         double2 *ym = reinterpret_cast<double2 *>(lkp + kTempInvYm);
         k_inverse_nodes<<<(n_inv + 127) / 128, 128, 0, in.stream>>>(lkp, lkp + kTempConsts, ym, kTempLnLo, kTempLnHi, ln_a,
-                                                                    e, v_org, n_inv);
+                                                                    e, v_org, n_inv, (float)(1.0 / accepted_step(h)));
         k_inverse_coeffs<<<(8 * (n_inv - 1) + 127) / 128, 128, 0, in.stream>>>(
             lkp, ym, reinterpret_cast<float4 *>(lkp + kTempCoefInv), kTempLnLo, kTempLnHi, ln_a, e, v_org, n_inv);
         k_hermite_coeffs<<<4, 256, 0, in.stream>>>(lkp, reinterpret_cast<float4 *>(lkp + kTempCoefLkp),
