@@ -6,7 +6,7 @@
 // (tiles weighted by the grid's bin count) is 1/G of the total, and walks it grid
 // segment by grid segment with the tile body of rt_tile.cuh, writing one energy
 // partial per (grid, CTA). A second small kernel reduces the partials of every
-// grid in FP64. Both kernels and the partials reset form a CUDA graph built once;
+// grid in FP64. Both kernels and a reset form a CUDA graph built once;
 // each run only replaces the field pointers in the tracer node and replays it.
 // Two kernel families: the tile body of rt_tile.cuh (any nr; work units are tiles,
 // split statically as above), and the warp-per-ray body of rt_ray.cuh (every grid
@@ -30,7 +30,8 @@ struct BatchParams {
     const TraceArgs *grids;          // [n] tables and sizes of every grid
     const unsigned *grid_tile_begin; // [n+1] first global work unit (tile or warp-slot) of every grid
     const unsigned *cta_begin;       // [G+1] first global work unit of every CTA
-    double2 *partials;               // [n * G] (absorbed, escaped) per grid and CTA
+    double2 *partials;               // (absorbed, escaped): [n * G] per grid and CTA, or [n_chunks * W]
+                                     // per chunk and warp (warp-per-ray kind)
     unsigned *work;                  // warp-per-ray kind: next chunk to hand out (zeroed per run)
     const unsigned *chunk_begin;     // [n+1] first chunk of every grid (warp-per-ray kind)
     unsigned n_chunks;               // chunks of all grids
@@ -97,8 +98,10 @@ __host__ __device__ __forceinline__ int ray_lanes_for(int nr, int C)
 // from one counter: the cost of a warp-slot depends on how many of its bins the
 // thin series takes, which only the fields decide, so a static split by bins would
 // leave CTAs idle. Chunk indices grow, so a CTA meets every grid at most once; it
-// stages the grid's descriptor and tables in shared memory when the grid changes
-// and writes one FP64 energy partial per (grid, CTA) when it leaves it. The next
+// stages the grid's descriptor and tables in shared memory when the grid changes.
+// Every warp writes one FP64 energy partial per chunk: which rays a partial holds is
+// then a matter of the plan alone, and the energies of a replay repeat bit for bit
+// whichever CTA took a chunk (a partial per CTA followed the hand-out). The next
 // chunk's index is fetched while the current one is traced.
 template <int C, int W, int MODE, int MINB>
 __global__ void __launch_bounds__(W * 32, MINB) k_batch_ray(const __grid_constant__ BatchParams bp)
@@ -117,9 +120,6 @@ __global__ void __launch_bounds__(W * 32, MINB) k_batch_ray(const __grid_constan
     __syncthreads();
     unsigned c = s_next;
     int cur = -1, G = 32;
-    KahanSum eabs, eesc;
-    eabs.zero();
-    eesc.zero();
     while (c < bp.n_chunks) {
         __syncthreads();  // every thread has read s_next
         if (threadIdx.x == 0) s_next = atomicAdd(bp.work, 1u);
@@ -130,11 +130,6 @@ __global__ void __launch_bounds__(W * 32, MINB) k_batch_ray(const __grid_constan
             else lo = mid + 1;
         }
         if (lo != cur) {
-            if (cur >= 0) {
-                block_energy<W>(eabs, eesc);
-                if (threadIdx.x == 0)
-                    bp.partials[(size_t)cur * gridDim.x + blockIdx.x] = make_double2(to_double(eabs), to_double(eesc));
-            }
             __syncthreads();  // everyone is done with the previous grid's tables
             if (threadIdx.x == 0) {
                 s_p = bp.grids[lo];
@@ -151,9 +146,10 @@ __global__ void __launch_bounds__(W * 32, MINB) k_batch_ray(const __grid_constan
             ray_tables<C, W>(s_p, G, rs, s_kap, s_nu, s_mom);
             __syncthreads();
             cur = lo;
-            eabs.zero();
-            eesc.zero();
         }
+        KahanSum eabs, eesc;
+        eabs.zero();
+        eesc.zero();
         const unsigned units = bp.grid_tile_begin[cur + 1] - bp.grid_tile_begin[cur];
         const unsigned w0 = (c - bp.chunk_begin[cur]) * bp.chunk_slots;
         const unsigned w1 = w0 + bp.chunk_slots < units ? w0 + bp.chunk_slots : units;
@@ -172,27 +168,31 @@ __global__ void __launch_bounds__(W * 32, MINB) k_batch_ray(const __grid_constan
         if (G == 8) trace(std::integral_constant<int, 8>());
         else if (G == 16) trace(std::integral_constant<int, 16>());
         else trace(std::integral_constant<int, 32>());
+        for (int o = 16; o > 0; o >>= 1) {
+            eabs.add(eabs.shfl_xor(o));
+            eesc.add(eesc.shfl_xor(o));
+        }
+        if ((threadIdx.x & 31) == 0)
+            bp.partials[(size_t)c * W + warp] = make_double2(to_double(eabs), to_double(eesc));
         __syncthreads();  // s_next holds the next chunk
         c = s_next;
     }
-    if (cur >= 0) {
-        block_energy<W>(eabs, eesc);
-        if (threadIdx.x == 0)
-            bp.partials[(size_t)cur * gridDim.x + blockIdx.x] = make_double2(to_double(eabs), to_double(eesc));
-    }
 }
 
-// One block per grid: FP64 sum of its partials and the energy bookkeeping of
-// rt_energy (the same formulas as the single-grid reduction).
-__global__ void k_batch_energy(const double2 *partials, unsigned G, const DevScalars *const *sc,
-                               rt_energy *out)
+// One block per grid: FP64 sum of its partials (`per` of them, or of each of its chunks where
+// chunk_begin is given) and the energy bookkeeping of rt_energy (the same formulas as the
+// single-grid reduction).
+__global__ void k_batch_energy(const double2 *partials, unsigned per, const unsigned *chunk_begin,
+                               const DevScalars *const *sc, rt_energy *out)
 {
     __shared__ double s_a[32], s_e[32];
     const int g = blockIdx.x;
+    const size_t b0 = (size_t)(chunk_begin ? chunk_begin[g] : (unsigned)g) * per;
+    const size_t b1 = (size_t)(chunk_begin ? chunk_begin[g + 1] : (unsigned)g + 1u) * per;
     double sa = 0.0, se = 0.0;
-    for (unsigned b = threadIdx.x; b < G; b += blockDim.x) {
-        sa += partials[(size_t)g * G + b].x;
-        se += partials[(size_t)g * G + b].y;
+    for (size_t b = b0 + threadIdx.x; b < b1; b += blockDim.x) {
+        sa += partials[b].x;
+        se += partials[b].y;
     }
     for (int o = 16; o > 0; o >>= 1) {
         sa += __shfl_xor_sync(0xffffffffu, sa, o);
@@ -369,11 +369,13 @@ int plan(rt_batch *b, const BatchShape *s)
     cb[G] = total_tiles;
 
     // device buffers that depend on G
-    if ((size_t)n * G > b->partials_cap) {
+    const size_t n_part = ray ? (size_t)chb[n] * s->w : (size_t)n * G;
+    if (n_part > b->partials_cap) {
         if (b->partials_d) cudaFree(b->partials_d);
         b->partials_d = nullptr;
-        RT_BCK(b, cudaMalloc(&b->partials_d, sizeof(double2) * (size_t)n * G));
-        b->partials_cap = (size_t)n * G;
+        b->partials_cap = 0;
+        RT_BCK(b, cudaMalloc(&b->partials_d, sizeof(double2) * n_part));
+        b->partials_cap = n_part;
     }
     if (G + 1 > b->cta_cap) {
         if (b->cta_begin_d) cudaFree(b->cta_begin_d);
@@ -398,27 +400,20 @@ int plan(rt_batch *b, const BatchShape *s)
     b->params.chunk_slots = chunk_slots;
     b->params.n = n;
 
-    // graph: reset partials -> tracer -> per-grid energy
+    // graph: reset partials (chunk counter) -> tracer -> per-grid energy
     if (b->exec) { cudaGraphExecDestroy(b->exec); b->exec = nullptr; }
     if (b->graph) { cudaGraphDestroy(b->graph); b->graph = nullptr; }
     RT_BCK(b, cudaGraphCreate(&b->graph, 0));
+    // (the tiles' CTAs write a partial only where they meet a grid; of the chunks each has its own)
     cudaMemsetParams mp{};
-    mp.dst = b->partials_d;
+    mp.dst = ray ? (void *)b->work_d : (void *)b->partials_d;
     mp.value = 0;
     mp.elementSize = 4;
-    mp.width = (size_t)n * G * sizeof(double2) / 4;
+    mp.width = ray ? 1 : n_part * sizeof(double2) / 4;
     mp.height = 1;
     mp.pitch = 0;
-    cudaGraphNode_t n_reset[2], n_energy;
-    RT_BCK(b, cudaGraphAddMemsetNode(&n_reset[0], b->graph, nullptr, 0, &mp));
-    cudaMemsetParams mw{};
-    mw.dst = b->work_d;
-    mw.value = 0;
-    mw.elementSize = 4;
-    mw.width = 1;
-    mw.height = 1;
-    mw.pitch = 0;
-    RT_BCK(b, cudaGraphAddMemsetNode(&n_reset[1], b->graph, nullptr, 0, &mw));
+    cudaGraphNode_t n_reset, n_energy;
+    RT_BCK(b, cudaGraphAddMemsetNode(&n_reset, b->graph, nullptr, 0, &mp));
     b->kp_args[0] = &b->params;
     b->kp.func = (void *)s->kern;
     b->kp.gridDim = dim3(G);
@@ -426,16 +421,17 @@ int plan(rt_batch *b, const BatchShape *s)
     b->kp.sharedMemBytes = (unsigned)smem;
     b->kp.kernelParams = b->kp_args;
     b->kp.extra = nullptr;
-    RT_BCK(b, cudaGraphAddKernelNode(&b->kern_node, b->graph, n_reset, 2, &b->kp));
+    RT_BCK(b, cudaGraphAddKernelNode(&b->kern_node, b->graph, &n_reset, 1, &b->kp));
     cudaKernelNodeParams ep{};
     const double2 *e_part = b->partials_d;  // argument values are copied into the node
-    unsigned e_g = G;
+    unsigned e_per = ray ? (unsigned)s->w : G;
+    const unsigned *e_chunks = ray ? b->chunk_begin_d : nullptr;
     const rt::DevScalars *const *e_sc = b->sc_d;
     rt_energy *e_out = b->energies_d;
-    void *eargs[4] = {&e_part, &e_g, &e_sc, &e_out};
+    void *eargs[5] = {&e_part, &e_per, &e_chunks, &e_sc, &e_out};
     ep.func = (void *)rt::k_batch_energy;
     ep.gridDim = dim3(n);
-    ep.blockDim = dim3(256);
+    ep.blockDim = dim3(ray ? 1024 : 256);
     ep.sharedMemBytes = 0;
     ep.kernelParams = eargs;
     ep.extra = nullptr;
