@@ -60,6 +60,7 @@ template <int C, int W, int MODE, int MINB>
 cudaError_t launch_shape(const TraceArgs &a, unsigned ntiles, cudaStream_t stream, unsigned *grid_out,
                          unsigned max_grid)
 {
+    constexpr unsigned T = 32 * W * C;  // cells of a tile
     size_t smem = trace_smem_bytes<C, W, MODE>(a);
     // FP64: at most three CTAs per SM, by their shared memory. Two or three fill the FP64 pipe (a warp
     // instruction takes it 16 clocks), and with the tiles handed out as CTAs end, an SM that holds eight
@@ -82,7 +83,17 @@ cudaError_t launch_shape(const TraceArgs &a, unsigned ntiles, cudaStream_t strea
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     unsigned grid = (unsigned)nsm * (unsigned)per_sm;
-    if (grid > ntiles || MODE == RT_FP64) grid = ntiles;
+    if (MODE == RT_FP64) {
+        // A CTA first sums its ray's column up to its first tile, nr / 2 cells on average, which T cells
+        // of work hide while nr <= 16 T or so. Longer rays: several consecutive tiles per CTA, in whole
+        // waves (never fewer CTAs than the chip holds; with less than two waves of tiles one each). us,
+        // one tile per CTA / so: 1048576 cells x 2 rays, 16 bins 7078 / 2066, x 16 rays, 79 bins 51794 /
+        // 7980, 65536 x 16 685 / 422; 16384 x 64 365 / 360, where the two meet.
+        constexpr unsigned kRaySum = 16;
+        const unsigned run = ((unsigned)a.nr + kRaySum * T - 1) / (kRaySum * T);
+        grid = run > 1 && ntiles >= 2 * grid ? grid * std::max(1u, ntiles / run / grid) : ntiles;
+    }
+    if (grid > ntiles) grid = ntiles;
     if (max_grid > 0 && grid > max_grid) grid = max_grid;
     if (grid < 1) grid = 1;
     kern<<<grid, W * 32, smem, stream>>>(a);
