@@ -407,30 +407,47 @@ __device__ __forceinline__ float4 flux_quad(int nr, int nth, int nph, unsigned n
     return acc;
 }
 
+// a + b as their rounded sum and the rest, exactly (Knuth)
+__device__ __forceinline__ float2 two_sum(float a, float b)
+{
+    const float t = a + b, bp = t - a;
+    return make_float2(t, (a - (t - bp)) + (b - bp));
+}
+
 // Per-thread sums in compensated FP32 (TwoSum; GB300's FP64 rate is a small
-// fraction of its FP32 rate). A block's sum stays a pair of floats (48 bits), its partial is FP64.
+// fraction of its FP32 rate).
 struct KSum {
     float s = 0.0f, c = 0.0f;
     __device__ __forceinline__ void add(float v)
     {
-        const float t = s + v;
-        const float bp = t - s;
-        c += (s - (t - bp)) + (v - bp);
-        s = t;
+        const float2 t = two_sum(s, v);
+        c += t.y;
+        s = t.x;
     }
-    __device__ __forceinline__ void add(const KSum &o)
+};
+// A block's sum of them: three floats (what a TwoSum leaves goes into the next one), which lose
+// less than FP64 does; the block's partial is FP64. In FP64 the block sums took 1.5 us more per
+// iteration (64x32x64: 1.72 against 1.67 ms per step), pairs of floats lost 2^-48 per addition.
+struct BSum {
+    float s = 0.0f, c = 0.0f, d = 0.0f;
+    BSum() = default;
+    __device__ __forceinline__ BSum(const KSum &k) : s(k.s), c(k.c) {}
+    __device__ __forceinline__ void add(const BSum &o)
     {
-        add(o.s);
-        c += o.c;
+        const float2 t = two_sum(s, o.s), u = two_sum(c, o.c), v = two_sum(u.x, t.y);
+        s = t.x;
+        c = v.x;
+        d = (d + o.d) + (u.y + v.y);
     }
-    __device__ __forceinline__ KSum shfl(int m) const
+    __device__ __forceinline__ BSum shfl(int m) const
     {
-        KSum r;
+        BSum r;
         r.s = __shfl_xor_sync(0xffffffffu, s, m);
         r.c = __shfl_xor_sync(0xffffffffu, c, m);
+        r.d = __shfl_xor_sync(0xffffffffu, d, m);
         return r;
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
+    __device__ __forceinline__ double value() const { return ((double)d + (double)c) + (double)s; }
 };
 struct KMax {
     float s = 0.0f;
@@ -478,6 +495,7 @@ template <class S>
 __device__ bool grid_reduce(const CgArgs &a, const S &v, double *out, int at = 0)
 {
     __shared__ bool s_last;
+    constexpr bool kMax = std::is_same<S, KMax>::value;
     const S t = block_reduce(v);
     if (threadIdx.x == 0) {
         a.part[at + blockIdx.x] = t.value();
@@ -486,7 +504,6 @@ __device__ bool grid_reduce(const CgArgs &a, const S &v, double *out, int at = 0
     }
     __syncthreads();
     if (!s_last) return false;
-    constexpr bool kMax = std::is_same<S, KMax>::value;
     DSum u;
     KMax m;
     for (int i = threadIdx.x; i < at + (int)gridDim.x; i += blockDim.x) {
@@ -916,7 +933,7 @@ __global__ void __launch_bounds__(256, Q ? 4 : 6) k_it_apply(const CgArgs a, con
         }
     });
     double tot;
-    if (grid_reduce(a, pq, &tot)) {
+    if (grid_reduce(a, BSum(pq), &tot)) {
         if (pend) sc[kDLive] = 1.0;
         sc[kAlpha] = tot > 0.0 ? sc[kRz] / tot : 0.0;
         sc[kPend] = sc[kLast] != 0.0 ? 0.0 : 1.0;  // past max_iter the new step is not taken
@@ -965,7 +982,7 @@ __global__ void __launch_bounds__(256) k_it_jacobi(const CgArgs a)
         rz.add(r * z);
     });
     double tot;
-    if (grid_reduce(a, rz, &tot)) close_step(a, tot);
+    if (grid_reduce(a, BSum(rz), &tot)) close_step(a, tot);
 }
 
 // the loop's condition, at the end of its body (with a limit of its own: whatever the scalars
@@ -1390,12 +1407,12 @@ __global__ void __launch_bounds__(256, Q ? 5 : 6) k_mg_up0(const MgPair P)
         }
     });
     if (ln.nl > 0) {  // k_line_post sums these partials with its own
-        const KSum t = block_reduce(rz);
+        const BSum t = block_reduce(BSum(rz));
         if (threadIdx.x == 0) P.cg.part[blockIdx.x] = t.value();
         return;
     }
     double tot;
-    if (grid_reduce(P.cg, rz, &tot)) close_step(P.cg, tot);
+    if (grid_reduce(P.cg, BSum(rz), &tot)) close_step(P.cg, tot);
 }
 
 // z = x1 + omega T^-1 (b - A x1) of the line rows, and their share of r.z (after the partials of
@@ -1413,7 +1430,7 @@ __global__ void __launch_bounds__(512, 2) k_line_post(const CgArgs a, const Line
                        rz.add(e.y * z);
                    });
     double tot;
-    if (grid_reduce(a, rz, &tot, rows_partials)) close_step(a, tot);
+    if (grid_reduce(a, BSum(rz), &tot, rows_partials)) close_step(a, tot);
 }
 
 #undef MG_LOOP
@@ -1860,7 +1877,7 @@ int rt_fld_step(rt_ctx *ctx, const float *rho, const float *t_gas, const float *
     const auto apply = quads ? k_it_apply<true> : k_it_apply<false>;
     const auto flush = quads ? k_it_flush<true> : k_it_flush<false>;
     // (one limit for all contexts: another thread's smaller step must not lower it; the kernels'
-    // static part, at most 6.7 KB, counts towards the 48 KB a launch has without asking)
+    // static part, at most 6.8 KB, counts towards the 48 KB a launch has without asking)
     auto big_smem = [](const void *kern, size_t bytes) {
         return bytes <= 40 * 1024 ||
                (bytes <= kMaxFldSmem && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
