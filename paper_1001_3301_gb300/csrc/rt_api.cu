@@ -998,10 +998,12 @@ int host_enqueue(rt_ctx *ctx, const float *rho, const float *t_dust, float *q_ab
     // ~1.4-2 M cells per chunk, copies of 6-8 MB per field, since the link moves small copies in both
     // directions at once less efficiently (4 MB: 253 GB/s in total, 16 MB: 312 GB/s, one 256 MB copy
     // each way: 340 GB/s); below 8 M cells up to four chunks of >= 0.5 M cells, since there the first
-    // copies in and the last ones out, which overlap nothing, weigh more (one chunk or ~2 M cells
-    // each -> four, us: 1.6 M cells 169 -> 147, 2.1 M 213 -> 189, 3.1 M 302 -> 260, 4.2 M 333 -> 310,
-    // 6.3 M 450 -> 442, where six take 462; four -> six: 8.4 M cells 565 -> 521-553, 12 M 769 -> 764,
-    // 14 M 921 -> 907; smaller end chunks: 8.4 M cells 562-594)
+    // copies in and the last ones out, which overlap nothing, weigh more. Medians of 60 calls with 1 / 2 /
+    // 4 / 6 chunks in turn in one process, us: 1.05 M cells 123 / 119 / 122 / 130, 2.1 M 217 / 186 / 191 /
+    // 200, 3.1 M 304 / 260 / 259 / 254, 4.2 M 389 / 333 / 306 / 304, 6.3 M 567 / 474 / 440 / 451, 7.9 M
+    // 698 / 575 / 536 / 544, 8.4 M 744 / 609 / 568 / 550, 9.4 M 829 / 677 / 630 / 626, 12.6 M 1103 / 885 /
+    // 815 / 800, 14.7 M 1266 / 1018 / 929 / 921, 16.8 M 1442 / 1154 / 1043 / 1034: six gain 0.6 to 3 %
+    // from 8.4 M on (a call's times spread by 2 to 9 % there) and lose as much below.
     int nch = ctx->ncells >= 1LL << 23 ? (int)std::min<long long>(kHostChunks, std::max<long long>(6, ctx->ncells >> 21))
                                        : (int)std::max<long long>(1, std::min<long long>(4, ctx->ncells >> 19));
     if (nch > ctx->nrays) nch = (int)ctx->nrays;

@@ -543,8 +543,8 @@ __device__ __forceinline__ void for_cells(const CgArgs &a, unsigned b0, const F 
 // phi ring per (j, k)): x0 = omega T^-1 b before the restriction and x1 + omega T^-1 (b - A x1)
 // after the prolongation, symmetric as before and omega lambda(T^-1 A) < 2 as for the points.
 // FP64 PCG on the CPU to a 1e-8 residual: 79 -> 31 iterations on 128x64x64 with 12 % of the
-// rows; lines in every row 29, radial lines 79. On the GPU 253 -> 60 iterations per step on
-// 256x128x256 (dt = 1e4 s), and the largest error of a cell 1.7e-4 -> 5e-6.
+// rows; lines in every row 29, radial lines 79. On the GPU 256 -> 56 iterations per step on
+// 256x128x256 (dt = 1e4 s), and the error against 64 bits 4.3e-6 -> 2.9e-7 (2-norm).
 struct LineOp {
     int j0, j1, nl;             // rows j < j0 and j >= j1: nl of them (j0 = 0, j1 = nth: none)
     int seg;                    // segments a ring is cut into (its last cells are the separators)

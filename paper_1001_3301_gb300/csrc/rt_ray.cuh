@@ -398,7 +398,8 @@ __device__ __forceinline__ void ray_slots(const TraceArgs &p, unsigned wr_begin,
                 }
             }
         } else {
-            // the last lanes of a ray
+            // the last lanes of a ray, and every lane where the rays do not start on vector
+            // boundaries and the shape has no stage
 #pragma unroll
             for (int j = 0; j < C; j += 2) {
                 rho2[j / 2] = make_float2(j < nv ? __ldg(p.rho + base + j) : 0.0f,

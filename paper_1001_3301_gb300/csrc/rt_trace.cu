@@ -51,10 +51,11 @@ __global__ void __launch_bounds__(W * 32, MINB) k_trace(const TraceArgs p)
 }
 
 // Launch one chunk with a persistent grid of (SMs x resident CTAs) CTAs, or fewer
-// when there are fewer tiles. The FP64 mode launches one CTA per tile instead: a tile's
-// work depends on its columns (a midplane tile takes several times the mean) and is long
-// against the CTA's set-up, so the hardware's block scheduler balances the SMs, which
-// contiguous ranges left two thirds idle (128x64x64, 79 bins, tau550 = 1: 0.55 -> 0.25 ms).
+// when there are fewer tiles. The FP64 mode launches one CTA per tile instead
+// (several tiles on long rays, below): a tile's work depends on its columns (a
+// midplane tile takes several times the mean) and is long against the CTA's
+// set-up, so the hardware's block scheduler balances the SMs, which contiguous
+// ranges left two thirds idle (128x64x64, 79 bins, tau550 = 1: 0.55 -> 0.25 ms).
 // Returns the grid size (energy partials written).
 template <int C, int W, int MODE, int MINB>
 cudaError_t launch_shape(const TraceArgs &a, unsigned ntiles, cudaStream_t stream, unsigned *grid_out,
