@@ -608,9 +608,10 @@ int planck_means(const CtxInfo &in, const std::vector<double> &t_nodes, double *
 
 // The last Newton step of ln T after which diffuse_temperature takes a cell. A step dy leaves
 // F''/(2 F') dy^2, with F' = 4 + w L' and F'' = w L'' - w (1 - w) L'^2, 0 <= w <= 1 the source's
-// share: the largest |L''| and |L'| of the table's cubics bound that by kLeft. 5e-4 on means of
-// kappa(nu), 5e-5 to 1e-4 on tables whose kappa(T) is linear between 24 or 32 temperatures (kinks
-// in the mean: L'' in the hundreds; with 5e-4 there, one cell in a thousand was off by up to 2e-5).
+// share: the largest |L''| and |L'| of the table's cubics bound that by kLeft. 4e-4 to 5e-4 on
+// means of kappa(nu) (L'' up to 5), 2e-5 to 1e-4 on tables whose kappa(T) is linear between 8 to 32
+// temperatures (kinks in the mean: L'' 90 to 750; with 5e-4 there, up to one cell in a thousand was
+// off by up to 2e-5).
 double accepted_step(const std::vector<float> &h)
 {
     constexpr double kLeft = 1.5e-7;
