@@ -44,7 +44,7 @@ struct BatchParams {
     float *a[RT_BATCH_MAX];
 };
 
-// warp-slots per warp in one chunk of the warp-per-ray batch
+// most warp-slots per warp in one chunk of the warp-per-ray batch
 constexpr unsigned kBatchChunkWarpSlots = 8;
 
 template <int C, int W, int MODE, int MINB>
@@ -345,9 +345,13 @@ int plan(rt_batch *b, const BatchShape *s)
     }
     const unsigned total_tiles = gtb[n];
     unsigned G = (unsigned)nsm * (unsigned)per_sm;
-    // warp-per-ray kind: chunks of kBatchChunkWarpSlots warp-slots per warp, handed out
-    // in order at run time (so G only needs to fill the GPU)
-    const unsigned chunk_slots = (unsigned)s->w * rt::kBatchChunkWarpSlots;
+    // warp-per-ray kind: chunks of up to kBatchChunkWarpSlots warp-slots per warp, handed out
+    // in order at run time (so G only needs to fill the GPU); fewer on small batches, so that there
+    // are two chunks for every resident CTA: with eight throughout, a few CTAs walked eight slots one
+    // after the other (us, tiles / eight / so: 1 grid of 268 rays, 36 k cells 28 / 89 / 29; 4 grids, 107 k
+    // cells 38 / 61 / 26; 16 grids, 3.0 M cells 138 / 145 / 78; 24 grids, 12 M cells 485 / 209 / 192)
+    const unsigned per_warp = total_tiles / (2u * (unsigned)s->w * (unsigned)nsm * (unsigned)per_sm);
+    const unsigned chunk_slots = (unsigned)s->w * std::min(std::max(per_warp, 1u), rt::kBatchChunkWarpSlots);
     std::vector<unsigned> chb(n + 1, 0);
     for (int gg = 0; gg < n; ++gg) chb[gg + 1] = chb[gg] + (gtb[gg + 1] - gtb[gg] + chunk_slots - 1) / chunk_slots;
     if (ray) {
