@@ -87,13 +87,14 @@ int ray_shapes_lut(int precision, int nr, Shape *out, int max_out)
 //     few: the cost is cells held / nr, weighted per shape (256x128x256, tau550 = 10: C = 8 62 us,
 //     C = 16 65, C = 4 with two warps per ray 99; 384x128x128, tau550 = 1: C = 12 32 us, C = 6 with
 //     two warps 48, C = 16 46);
-//   - grids that do not give every SM eight warps are latency-bound: the fewest cells per lane
-//     (64x32x1: C = 2 7.3 us, C = 8 7.5, C = 16 9.3). With the line at two warps per SM a seventh of
-//     1200 small cases (nr 48 to 512, 24 to 32768 rays, 32 to 128 bins, tau550 = 0.3 to 30) was more
-//     than 5 % slower than the fewest cells whose lanes are 3/4 full, up to 26 %; at eight warps
-//     3.6 % of them, and the mean distance from the best shape is 1.7 % in place of 3.6. us, two
-//     / eight warps: 128x24x32, 128 bins, tau550 = 30 10.4 / 8.5; 256x24x21, the same 10.4 / 8.5; 432x24x14,
-//     79 bins, tau550 = 0.3 7.8 / 6.5; four or sixteen warps: 2.5, 2.6 %;
+//   - grids that do not give every SM eight warps (32 with C = 16) are latency-bound: the fewest
+//     cells per lane (64x32x1: C = 2 7.3 us, C = 8 7.5, C = 16 9.3). With the line at two warps per SM
+//     a seventh of 1200 small cases (nr 48 to 512, 24 to 32768 rays, 32 to 128 bins, tau550 = 0.3 to 30)
+//     was more than 5 % slower than the fewest cells whose lanes are 3/4 full, up to 26 %; so 1.8 % of
+//     them, and the mean distance from the best shape is 1.5 % in place of 3.6 (one line at four, eight,
+//     sixteen warps: 2.5, 1.7, 2.6 %). us, before / so: 128x24x32, 128 bins, tau550 = 30 10.4 / 8.5;
+//     256x24x21, the same 10.4 / 8.5; 432x24x14, 79 bins, tau550 = 0.3 7.8 / 6.5; 432x24x170, 128 bins,
+//     tau550 = 30 28.9 / 25.2;
 //   - longer rays: the chunked form, which needs some 1500 rays to fill the SMs (1024x128x16:
 //     31 us against the tiles' 58; 1024x16x16: tiles 22 us).
 bool ray_default(int precision, int nr, long long nrays, bool tw, Shape *out)
@@ -116,7 +117,7 @@ bool ray_default(int precision, int nr, long long nrays, bool tw, Shape *out)
     for (int i = 0; i < n; ++i) {
         const int c = s[i].cells_per_lane, held = ray_cells_held(c, nr);
         double cost = (double)held / nr * weight(c) * (held > 32 * c ? 1.15 : 1.0);  // two warps per ray
-        if (nrays * held < 1216LL * 32 * c) cost = 100.0 + c;
+        if (nrays * held < (c == 16 ? 4864LL : 1216LL) * 32 * c) cost = 100.0 + c;
         // of one shape's register caps the first but for the two of C = 16 (4 CTAs per SM)
         if (i == 0 || cost < best || (cost == best && c == 16 && s[bi].cells_per_lane == 16)) {
             best = cost;
