@@ -1152,11 +1152,17 @@ int rt_irradiate_lut(rt_ctx *ctx, const float *rho, const float *t_dust, float *
     Shape cand[16];
     const int nc = rt::ray_shapes_lut(ctx->precision, ctx->nr, cand, 16);
     if (nc < 1) return fail(ctx, RT_ERR_INVALID_ARG, "the lookup table needs rays of at most 512 cells");
+    // the context's own shape where one was asked for or tuned and is compiled with the table; else 8
+    // cells per lane, and the fewest on grids of less than eight warps per SM: a cell here is two table
+    // reads whatever its bins, and up to 512 cells 8 is the fastest or within 3 % of it (512x24x682 cells
+    // 51 us, C = 16 58; 256x24x682 29, C = 4 33, C = 16 31; 256x24x4 6.5, C = 4 6.0)
+    const bool few = ctx->nrays * rt::ray_cells_held(8, ctx->nr) < 1216LL * 32 * 8;
     Shape s = cand[0];
-    for (int i = 0; i < nc; ++i)  // the context's own shape where it is compiled with the table
-        if (cand[i].cells_per_lane == ctx->shape.cells_per_lane && cand[i].warps == ctx->shape.warps &&
-            cand[i].min_blocks == ctx->shape.min_blocks && ctx->shape.kind == rt::kKindRay)
-            s = cand[i];
+    for (int i = 0; i < nc; ++i) {
+        const bool own = cand[i].cells_per_lane == ctx->shape.cells_per_lane && cand[i].warps == ctx->shape.warps &&
+                         cand[i].min_blocks == ctx->shape.min_blocks && ctx->shape.kind == rt::kKindRay;
+        if (ctx->shape_forced ? own : !few && cand[i].cells_per_lane == 8) s = cand[i];
+    }
     if (fallback_slots) RT_CK(ctx, cudaMemsetAsync(ctx->lut_count, 0, sizeof(unsigned), ctx->stream));
     ctx->lut_on = true;
     st = trace(ctx, rho, t_dust, q_abs, a_rad, s);
